@@ -152,8 +152,9 @@ __device__ __forceinline__ bool r2c_block(const float* __restrict__ in, int rows
 
 // The part of step 4 after staging, for column block bx of one image: sm holds
 // the Hermitian half [N/2 + 1][2B] complex (and serves as the FFT's exchange
-// buffer afterwards); arguments as for c2r_block.
-template <int N, int B>
+// buffer afterwards); arguments as for c2r_block.  TILES: tile maxima can be
+// asked for (the block's threads divide into whole tiles).
+template <int N, int B, bool TILES>
 __device__ __forceinline__ void c2r_from_stage(float2* sm, int ncols, const float2* __restrict__ stw,
                                                float mid_scale, float* __restrict__ out, int row0, int rows_out,
                                                int out_pitch, float out_scale, unsigned* __restrict__ tmax, int nbx,
@@ -194,7 +195,7 @@ __device__ __forceinline__ void c2r_from_stage(float2* sm, int ncols, const floa
     }
     __syncthreads();
     F::template run<0>(v, sm, t, f, stw);
-    if (tmax) {
+    if constexpr (TILES) if (tmax) {
         // Tile maxima of |map| for the peak pass: thread t holds rows t + T j,
         // j = m + GL q, of its column pair.  A tile is RS = 128 / B consecutive
         // rows of one band (rows T j + RS u .. T j + RS u + RS - 1, u < T / RS) of
@@ -302,7 +303,7 @@ __device__ __forceinline__ bool c2r_block(const float2* __restrict__ in, int nco
         cp_async_wait_all();
         __syncthreads();
     }
-    c2r_from_stage<N, B>(sm, ncols, stw, mid_scale, out, row0, rows_out, out_pitch, out_scale, tmax, nbx, bx);
+    c2r_from_stage<N, B, !fs_wide(N)>(sm, ncols, stw, mid_scale, out, row0, rows_out, out_pitch, out_scale, tmax, nbx, bx);
     return true;
 }
 

@@ -27,38 +27,77 @@
 
 #include "ft_internal.cuh"
 
-__host__ __device__ constexpr bool fs_has(int N) {
-    return N == 128 || N == 256 || N == 512 || N == 1024 || N == 2048 || N == 4096 || N == 8192 ||
-           N == 192 || N == 384 || N == 768 || N == 1536;
+// Schedules: E samples per thread and the radices of the passes (each divides
+// E).  Powers of two hold 16 samples (radix 16, 8, 4, 2 passes); lengths with
+// factors of 3 take the E whose divisors give few passes: 12 (radices 12, 6, 4,
+// 3, 2), 18 (18, 9, 6, 3, 2), 24 (24, 12, 8, 6) or 36 (18, 12).  Steps 1 / 2-3 / 4 of
+// 16 Mpx in square images, us, against the generic shared-memory kernels: 486^2
+// 38 / 38 / 32 (113 / 187 / 89), 1152^2 36 / 37 / 34 (109 / 132 / 86), 1944^2
+// 43 / 35 / 36 (127 / 191 / 104), 3456^2 51 / 36 / 46 (199 / 182 / 162).  Where two
+// schedules compete the choice is measured too: 1152 as 12 12 8 with E = 24
+// against 12 12 4 2 with E = 12 36 / 37 / 34 (44 / 35 / 42), 2304 as 24 12 8 against
+// 12 12 4 4 40 / 30 / 41 (55 / 35 / 53), 576 as 24 24 against 12 12 4 30 / 35 / 28
+// (35 / 35 / 37); but 288 as 12 12 2 against 24 12 29 / 38 / 28 (29 / 47 / 27), and
+// 1296 as 6 6 6 6 with E = 12 against 12 12 9 with E = 36, which spills, the same
+// forward and a faster adjoint (50 against 58).
+struct FsSched {
+    int N, E, nst, r[6];
+};
+__host__ __device__ constexpr FsSched fs_sched(int N) {
+    switch (N) {
+        case 128: return {128, 16, 2, {16, 8}};
+        case 144: return {144, 12, 2, {12, 12}};
+        case 162: return {162, 18, 2, {18, 9}};
+        case 192: return {192, 12, 4, {4, 4, 4, 3}};
+        case 216: return {216, 12, 3, {12, 6, 3}};
+        case 256: return {256, 16, 2, {16, 16}};
+        case 288: return {288, 12, 3, {12, 12, 2}};
+        case 324: return {324, 18, 2, {18, 18}};
+        case 384: return {384, 12, 5, {4, 4, 4, 2, 3}};
+        case 432: return {432, 12, 3, {12, 12, 3}};
+        case 486: return {486, 18, 3, {18, 9, 3}};
+        case 512: return {512, 16, 3, {16, 8, 4}};
+        case 576: return {576, 24, 2, {24, 24}};
+        case 648: return {648, 18, 3, {18, 18, 2}};
+        case 768: return {768, 12, 5, {4, 4, 4, 4, 3}};
+        case 864: return {864, 12, 3, {12, 12, 6}};
+        case 972: return {972, 18, 3, {18, 18, 3}};
+        case 1024: return {1024, 16, 3, {16, 16, 4}};
+        case 1152: return {1152, 24, 3, {12, 12, 8}};
+        case 1296: return {1296, 12, 4, {6, 6, 6, 6}};
+        case 1458: return {1458, 18, 3, {18, 9, 9}};
+        case 1536: return {1536, 12, 6, {4, 4, 4, 4, 2, 3}};
+        case 1728: return {1728, 12, 3, {12, 12, 12}};
+        case 1944: return {1944, 18, 3, {18, 18, 6}};
+        case 2048: return {2048, 16, 3, {16, 16, 8}};
+        case 2304: return {2304, 24, 3, {24, 12, 8}};
+        case 2592: return {2592, 36, 3, {18, 12, 12}};
+        case 2916: return {2916, 18, 3, {18, 18, 9}};
+        case 3072: return {3072, 24, 4, {8, 8, 8, 6}};
+        case 3456: return {3456, 24, 3, {24, 12, 12}};
+        case 3888: return {3888, 36, 3, {18, 18, 12}};
+        case 4096: return {4096, 16, 3, {16, 16, 16}};
+        case 8192: return {8192, 16, 4, {16, 16, 16, 2}};
+    }
+    return {0, 1, 0, {0}};
 }
-__host__ __device__ constexpr int fs_E(int N) { return N % 3 == 0 ? 12 : 16; }
+__host__ __device__ constexpr bool fs_has(int N) { return fs_sched(N).N != 0; }
+__host__ __device__ constexpr int fs_E(int N) { return fs_sched(N).E; }
 __host__ __device__ constexpr int fs_T(int N) { return N / fs_E(N); }
-__host__ __device__ constexpr int fs_nst(int N) {
-    return N == 128 ? 2 : N == 256 ? 2 : N == 512 ? 3 : N == 1024 ? 3 : N == 2048 ? 3 : N == 4096 ? 3
-         : N == 8192 ? 4 : N == 192 ? 4 : N == 384 ? 5 : N == 768 ? 5 : N == 1536 ? 6 : 0;
-}
-__host__ __device__ constexpr int fs_radix(int N, int s) {
-    return N == 128 ? (s == 0 ? 16 : 8)
-         : N == 256 ? 16
-         : N == 512 ? (s == 0 ? 16 : s == 1 ? 8 : 4)
-         : N == 1024 ? (s < 2 ? 16 : 4)
-         : N == 2048 ? (s < 2 ? 16 : 8)
-         : N == 4096 ? 16
-         : N == 8192 ? (s < 3 ? 16 : 2)
-         : N == 192 ? (s < 3 ? 4 : 3)
-         : N == 384 ? (s < 3 ? 4 : s == 3 ? 2 : 3)
-         : N == 768 ? (s < 4 ? 4 : 3)
-         : N == 1536 ? (s < 4 ? 4 : s == 4 ? 2 : 3)
-         : 0;
-}
+__host__ __device__ constexpr int fs_nst(int N) { return fs_sched(N).nst; }
+__host__ __device__ constexpr int fs_radix(int N, int s) { return fs_sched(N).r[s]; }
 __host__ __device__ constexpr int fs_P(int N, int s) {
     int p = 1;
     for (int j = 0; j < s; ++j) p *= fs_radix(N, j);
     return p;
 }
-// seed powers of a pass with radix R (exponents 1 << j, j < fs_nseed(R)) and the
+// seed powers of a pass with radix R (exponents 1 << j below R) and the
 // twiddle row stride of a full or a seed table, rounded up to even (16-byte rows)
-__host__ __device__ constexpr int fs_nseed(int R) { return R == 16 ? 4 : R == 8 ? 3 : R == 2 ? 1 : 2; }
+__host__ __device__ constexpr int fs_nseed(int R) {
+    int n = 0;
+    while ((1 << n) < R) ++n;
+    return n;
+}
 __host__ __device__ constexpr int fs_rs(int R, bool seed) { return ((seed ? fs_nseed(R) : R) + 1) & ~1; }
 __host__ __device__ constexpr int fs_twoff(int N, int s, bool seed) {
     int o = 0;
@@ -74,13 +113,35 @@ __host__ __device__ constexpr int fs_twsize(int N, bool seed) { return fs_twoff(
 // 256, and the peak pass is faster on the 16 x 16 tiles that gives) and the row
 // kernels (128 threads: at N = 1024, 2 rows per block run 116 us per
 // 64 x 1024^2, 4 rows 128 us, 1 row 142 us)
+//
+// The lengths with radices 6 to 24 (fs_wide) hold more than 64 registers' worth of
+// samples per thread (E = 18, 24, 36) or more temporaries (E = 12): fs_resident
+// threads share a multiprocessor (72, 80 or 112 registers each), and a column
+// block takes 8 column pairs (64-byte image rows) where at most 512 threads then
+// transform them, else 4 (16 or 32 where it would fall below 200 threads).
+// Measured as above: 16 pairs instead of 8 at 324 32 / 31 against 30 / 28 (steps 1 /
+// 4), at 648 46 / 43 against 35 / 31; 8 instead of 4 at 864 47 / 46 against 36 / 34;
+// 2 instead of 4 at 2304 and above slower or equal.
 __host__ __device__ constexpr int fs_clampB(int v, int hi) { return v < 1 ? 1 : (v > hi ? hi : v); }
-__host__ __device__ constexpr int fs_Bcol(int N) { return fs_T(N) >= 256 ? 1024 / fs_T(N) : fs_clampB(512 / fs_T(N), 32); }
+__host__ __device__ constexpr bool fs_wide(int N) { return N % 3 == 0 && N != 192 && N != 384 && N != 768 && N != 1536; }
+__host__ __device__ constexpr int fs_resident(int N) {
+    return !fs_wide(N) || fs_E(N) == 12 ? 1024 : fs_E(N) == 18 ? 864 : fs_E(N) == 24 ? 768 : 576;
+}
+__host__ __device__ constexpr int fs_minblocks(int N, int threads) {
+    return fs_resident(N) / threads > 0 ? fs_resident(N) / threads : 1;
+}
+__host__ __device__ constexpr int fs_Bwide(int N) {
+    return fs_T(N) * 32 <= 288 ? 32 : fs_T(N) * 16 <= 192 ? 16 : fs_T(N) * 8 <= 512 ? 8 : 4;
+}
+__host__ __device__ constexpr int fs_Bcol(int N) {
+    return fs_wide(N) ? fs_Bwide(N) : fs_T(N) >= 256 ? 1024 / fs_T(N) : fs_clampB(512 / fs_T(N), 32);
+}
 __host__ __device__ constexpr int fs_Bc2r(int N) {
-    return fs_T(N) >= 256 ? 1024 / fs_T(N)
+    return fs_wide(N) ? fs_Bwide(N)
+         : fs_T(N) >= 256 ? 1024 / fs_T(N)
                           : fs_clampB(N == 1024 ? 512 / fs_T(N) : (256 / fs_T(N) < 4 ? 4 : 256 / fs_T(N)), 32);
 }
-__host__ __device__ constexpr int fs_Brow(int N) { return fs_clampB(128 / fs_T(N), 16); }
+__host__ __device__ constexpr int fs_Brow(int N) { return fs_clampB((128 + (fs_wide(N) ? fs_T(N) / 2 : 0)) / fs_T(N), 16); }
 // padded shared-memory slot of sample n (one spare slot every 16 samples
 // spreads the strided stores of the first pass over the banks)
 __host__ __device__ constexpr int spos(int n) { return n + (n >> 4); }
@@ -97,31 +158,77 @@ __device__ __forceinline__ void cp_async_wait_all() {
 template <int SIGN>
 __device__ __forceinline__ float2 tw_sign(float2 w) { return SIGN > 0 ? make_float2(w.x, -w.y) : w; }
 
-// w[q] = w_k^q (conjugated for SIGN > 0), q = 1 .. R-1, from the seed row at wp
+// w[q] = w_k^q (conjugated for SIGN > 0), q = 1 .. R-1, from the seed row at wp:
+// the powers 1, 2, 4, ... are read, the others are products of two earlier ones
 template <int R, int SIGN>
 __device__ __forceinline__ void tw_powers(const float4* __restrict__ wp, float2 (&w)[R]) {
-    const float4 a = __ldg(wp);
-    w[1] = tw_sign<SIGN>(make_float2(a.x, a.y));
-    if constexpr (R == 3) {
-        w[2] = tw_sign<SIGN>(make_float2(a.z, a.w));
-    } else if constexpr (R >= 4) {
-        w[2] = tw_sign<SIGN>(make_float2(a.z, a.w));
-        w[3] = cmul(w[1], w[2]);
-        if constexpr (R >= 8) {
-            const float4 b = __ldg(wp + 1);
-            w[4] = tw_sign<SIGN>(make_float2(b.x, b.y));
-            w[5] = cmul(w[1], w[4]);
-            w[6] = cmul(w[2], w[4]);
-            w[7] = cmul(w[3], w[4]);
-            if constexpr (R == 16) {
-                w[8] = tw_sign<SIGN>(make_float2(b.z, b.w));
 #pragma unroll
-                for (int q = 9; q < 16; ++q) w[q] = cmul(w[q - 8], w[8]);
-            }
+    for (int h = 0; h < fs_rs(R, true) / 2; ++h) {
+        const float4 a = __ldg(wp + h);
+        w[1 << (2 * h)] = tw_sign<SIGN>(make_float2(a.x, a.y));
+        if ((2 << (2 * h)) < R) w[2 << (2 * h)] = tw_sign<SIGN>(make_float2(a.z, a.w));
+    }
+#pragma unroll
+    for (int b = 2; b < R; b *= 2)
+#pragma unroll
+        for (int q = b + 1; q < 2 * b && q < R; ++q) w[q] = cmul(w[q - b], w[b]);
+}
+
+// radix 9 as 3 x 3 with the internal twiddles exp(SIGN 2 pi i m / 9)
+template <int SIGN>
+struct Dft<9, SIGN> {
+    __device__ __forceinline__ static void run(float2* u) {
+        const float c1 = 0.76604444311897803520f, s1 = 0.64278760968653932632f;    // 2 pi / 9
+        const float c2 = 0.17364817766693034885f, s2 = 0.98480775301220805937f;    // 4 pi / 9
+        const float c4 = -0.93969262078590838405f, s4 = 0.34202014332566873304f;   // 8 pi / 9
+        float2 a[3][3];
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) {
+            float2 t[3] = {u[n2], u[3 + n2], u[6 + n2]};
+            Dft<3, SIGN>::run(t);
+#pragma unroll
+            for (int k1 = 0; k1 < 3; ++k1) a[n2][k1] = t[k1];
+        }
+        a[1][1] = cmul(a[1][1], make_float2(c1, SIGN * s1));
+        a[1][2] = cmul(a[1][2], make_float2(c2, SIGN * s2));
+        a[2][1] = cmul(a[2][1], make_float2(c2, SIGN * s2));
+        a[2][2] = cmul(a[2][2], make_float2(c4, SIGN * s4));
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) {
+            float2 t[3] = {a[0][k1], a[1][k1], a[2][k1]};
+            Dft<3, SIGN>::run(t);
+#pragma unroll
+            for (int k2 = 0; k2 < 3; ++k2) u[k1 + 3 * k2] = t[k2];
         }
     }
-    static_assert(R == 2 || R == 3 || R == 4 || R == 8 || R == 16, "radix without seed powers");
-}
+};
+
+// radix A B with A, B coprime by the prime-factor map: with n = (B a + A b) mod
+// A B and k = the residue pair (k mod A, k mod B), exp(2 pi i n k / (A B)) splits
+// into exp(2 pi i a k / A) exp(2 pi i b k / B), so no internal twiddles are needed
+template <int A, int B, int SIGN>
+struct DftCoprime {
+    __device__ __forceinline__ static void run(float2* u) {
+        float2 x[A][B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            float2 t[A];
+#pragma unroll
+            for (int a = 0; a < A; ++a) t[a] = u[(B * a + A * b) % (A * B)];
+            Dft<A, SIGN>::run(t);
+#pragma unroll
+            for (int a = 0; a < A; ++a) x[a][b] = t[a];
+        }
+#pragma unroll
+        for (int a = 0; a < A; ++a) Dft<B, SIGN>::run(x[a]);
+#pragma unroll
+        for (int k = 0; k < A * B; ++k) u[k] = x[k % A][k % B];
+    }
+};
+template <int SIGN> struct Dft<6, SIGN> : DftCoprime<2, 3, SIGN> {};
+template <int SIGN> struct Dft<12, SIGN> : DftCoprime<4, 3, SIGN> {};
+template <int SIGN> struct Dft<18, SIGN> : DftCoprime<2, 9, SIGN> {};
+template <int SIGN> struct Dft<24, SIGN> : DftCoprime<8, 3, SIGN> {};
 
 // radix-16 as 4 x 4 with the internal twiddles exp(SIGN 2 pi i m / 16)
 template <int SIGN>
@@ -298,8 +405,10 @@ cudaError_t launch_col_c2r_fast(const float2* in, int ncols, int in_pitch, size_
                                 unsigned* err = nullptr, long long wait = FT_WAIT_CYCLES);
 // tiles of the tile maxima of launch_col_c2r_fast for length N: rows x cols
 // cells, bands = N / rows tiles per column block; false without a schedule.
-// A tile is 256 cells: 128 / B rows of one column block of 2B columns.
-__host__ __device__ constexpr int c2r_tile_rows(int N) { return 128 / fs_Bc2r(N); }
+// A tile is 256 cells: 128 / B rows of one column block of 2B columns, held by
+// whole warps; lengths whose column block does not divide that way (fs_wide)
+// write no maxima (rows 0 here, false from c2r_tile_shape).
+__host__ __device__ constexpr int c2r_tile_rows(int N) { return fs_wide(N) ? 0 : 128 / fs_Bc2r(N); }
 bool c2r_tile_shape(int N, int* rows, int* cols, int* bands);
 // (err: bit 1 set when a bulk-copy wait ran out after `wait` SM cycles)
 cudaError_t launch_nvmt_rows_fast(float2* ws, int W, int Hp, int L, int interp, const FftLen& fx,
