@@ -264,10 +264,9 @@ int ft_plan_get_variant(ft_plan plan);
  *
  * Images whose sides both have a fixed-length schedule up to 2048 (128, 192,
  * 256, 384, 512, 768, 1024, 1536, 2048), with the linear or cubic interpolator,
- * run in the grouped kernels: one persistent launch per stage over all of them
- * (step 1; steps 2-3; step 4 with the maxima of |P| per 256-cell tile; the peak
- * pass from those maxima), each block taking (image, block) items from a device
- * work queue, largest images first, and running the fixed-length code of the
+ * run in the grouped kernels: one launch per stage over all of them (step 1;
+ * steps 2-3; step 4 with the maxima of |P| per 256-cell tile; the peak pass from
+ * those maxima), each block running the fixed-length code of one (image, block)
  * item's length; 4 launches (3 with top_k = 0) whatever the number of shapes.
  * Every other shape group keeps a plan of its own (one per shape) whose
  * ft_detect (ft_forward when top_k = 0) runs on one of up to 8 side streams

@@ -7,7 +7,7 @@
 // schedule up to 2048 (128, 192, 256, 384, 512, 768, 1024, 1536, 2048) with the
 // linear or cubic interpolator run in the grouped kernels of k_batch.cu: one
 // persistent launch per stage over all of them (step 1, steps 2-3, step 4 with
-// tile maxima, the peak pass), fed by device work queues, with the batch's own
+// tile maxima, the peak pass), one block per (image, block) item, with the batch's own
 // workspace.  Every other shape group keeps a plan of its own (tables and
 // workspace) and runs its ft_detect on one of up to FT_BATCH_MAX_STREAMS side
 // streams forked from and joined back into the caller's stream.  With
@@ -77,7 +77,7 @@ struct ft_batch_s {
     BatchImg* d_imgs = nullptr;
     int2* d_items[3][2] = {};               // (image, block) items per stage and threads option
     int nitems[3][2] = {};
-    unsigned* d_queue = nullptr;            // one counter per stage
+    bool pdl = true;                        // programmatic dependent launch of the stages (FT_PDL=0: off)
     float2* d_ws = nullptr;                 // half spectra of the grouped images
     unsigned* d_tmax = nullptr;             // tile maxima of step 4
     int threads[3] = {kDefaultThreads[0], kDefaultThreads[1], kDefaultThreads[2]};
@@ -218,26 +218,24 @@ static void drop_graph(ft_batch_s* b) {
 
 static int opt_index(int stage, int threads) { return threads == kThreadOpts[stage][1] ? 1 : 0; }
 
-// the grouped kernels: queues cleared, then one launch per stage
+// the grouped kernels, one launch per stage
 static ft_status enqueue_grouped(ft_batch_s* b, const float* imgs, float* maps, int top_k, float thr, ft_peak* out,
                                  int32_t* cnt, cudaStream_t st) {
     if (b->ng == 0) return FT_OK;
     const int o0 = opt_index(0, b->threads[0]), o1 = opt_index(1, b->threads[1]), o2 = opt_index(2, b->threads[2]);
-    cudaError_t e = cudaMemsetAsync(b->d_queue, 0, 4 * sizeof(unsigned), st);
-    if (e != cudaSuccess) return ft_record_cuda(e, "ft_batch: clear the work queues");
-    e = launch_batch_r2c(b->d_imgs, b->d_items[0][o0], b->nitems[0][o0], b->d_queue, imgs, b->d_ws, b->threads[0],
-                         b->maxH, st);
+    cudaError_t e = launch_batch_r2c(b->d_imgs, b->d_items[0][o0], b->nitems[0][o0], imgs, b->d_ws, b->threads[0],
+                                     b->maxH, st, b->pdl);
     if (e != cudaSuccess) return ft_record_cuda(e, "ft_batch: step 1 (grouped)");
-    e = launch_batch_rows(b->d_imgs, b->d_items[1][o1], b->nitems[1][o1], b->d_queue + 1, b->d_ws, b->interp,
-                          b->threads[1], b->maxW, st);
+    e = launch_batch_rows(b->d_imgs, b->d_items[1][o1], b->nitems[1][o1], b->d_ws, b->interp, b->threads[1], b->maxW,
+                          st, b->pdl);
     if (e != cudaSuccess) return ft_record_cuda(e, "ft_batch: steps 2-3 (grouped)");
-    e = launch_batch_c2r(b->d_imgs, b->d_items[2][o2], b->nitems[2][o2], b->d_queue + 2, b->d_ws, maps,
-                         top_k > 0 ? b->d_tmax : nullptr, b->threads[2], b->maxH, st);
+    e = launch_batch_c2r(b->d_imgs, b->d_items[2][o2], b->nitems[2][o2], b->d_ws, maps,
+                         top_k > 0 ? b->d_tmax : nullptr, b->threads[2], b->maxH, st, b->pdl);
     if (e != cudaSuccess) return ft_record_cuda(e, "ft_batch: step 4 (grouped)");
     if (top_k > 0) {
         const size_t sm = batch_peaks_smem(b->himgs.data(), b->ng, b->threads[2], top_k);
-        e = launch_batch_peaks(b->d_imgs, b->ng, b->d_queue + 3, maps, b->d_tmax, b->threads[2], top_k, thr, out, cnt,
-                               sm, st);
+        e = launch_batch_peaks(b->d_imgs, b->ng, maps, b->d_tmax, b->threads[2], top_k, thr, out, cnt, sm, st,
+                               b->pdl);
         if (e != cudaSuccess) return ft_record_cuda(e, "ft_batch: peaks (grouped)");
     }
     return FT_OK;
@@ -385,6 +383,11 @@ static ft_status setup_grouped(ft_batch_s* b) {
     }
     b->ng = (int)b->himgs.size();
     if (b->ng == 0) return FT_OK;
+    // steps 2-3 walk the images backwards: their first blocks read the half
+    // spectra step 1 wrote last, still in L2, and step 4 starts on the rows
+    // written last (every item holds the same number of samples, so the order
+    // does not change the tail of a launch)
+    for (int o = 0; o < 2; ++o) std::reverse(items[2 + o].begin(), items[2 + o].end());
     cudaError_t e = cudaMalloc(&b->d_imgs, b->himgs.size() * sizeof(BatchImg));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_imgs, b->himgs.data(), b->himgs.size() * sizeof(BatchImg), cudaMemcpyHostToDevice);
     for (int st = 0; st < 3 && e == cudaSuccess; ++st)
@@ -394,7 +397,6 @@ static ft_status setup_grouped(ft_batch_s* b) {
             e = cudaMalloc(&b->d_items[st][o], v.size() * sizeof(int2));
             if (e == cudaSuccess) e = cudaMemcpy(b->d_items[st][o], v.data(), v.size() * sizeof(int2), cudaMemcpyHostToDevice);
         }
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_queue, 4 * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_ws, (size_t)ws * sizeof(float2));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tmax, (size_t)(tm > 0 ? tm : 1) * sizeof(unsigned));
     if (e != cudaSuccess) {
@@ -418,6 +420,8 @@ ft_status ft_batch_create(ft_batch* out, int n, const int32_t* H, const int32_t*
     b->n = n;
     b->interp = interp;
     if (tune_cache) b->cache = tune_cache;
+    const char* pdl = getenv("FT_PDL");
+    b->pdl = !(pdl && !strcmp(pdl, "0"));
     int dev = 0;
     cudaDeviceProp prop;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&prop, dev) == cudaSuccess) b->gpu = prop.name;
@@ -491,7 +495,6 @@ ft_status ft_batch_destroy(ft_batch b) {
     for (int st = 0; st < 3; ++st)
         for (int o = 0; o < 2; ++o)
             if (b->d_items[st][o]) cudaFree(b->d_items[st][o]);
-    if (b->d_queue) cudaFree(b->d_queue);
     if (b->d_ws) cudaFree(b->d_ws);
     if (b->d_tmax) cudaFree(b->d_tmax);
     for (int s = 0; s < FT_BATCH_MAX_STREAMS; ++s) {

@@ -2,7 +2,7 @@
 // k_rows.cu for what each step computes), built on the register-resident FFT of
 // fft_fast.cuh.  The per-plan kernels of k_fast.cu run one of these per CUDA
 // block over a uniform batch; the mixed-size batch kernels of k_batch.cu run
-// them from a work queue over images of different lengths.  B, the transforms
+// them over images of different lengths.  B, the transforms
 // per block, is a template parameter: the block has fs_T(N) * B threads.
 //  * the column R2C reads its first pass directly from global memory; the
 //    other two stage their inputs into shared memory with 16-byte cp.async

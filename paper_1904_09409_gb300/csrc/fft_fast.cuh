@@ -39,7 +39,9 @@
 // 12 12 4 4 40 / 30 / 41 (55 / 35 / 53), 576 as 24 24 against 12 12 4 30 / 35 / 28
 // (35 / 35 / 37); but 288 as 12 12 2 against 24 12 29 / 38 / 28 (29 / 47 / 27), and
 // 1296 as 6 6 6 6 with E = 12 against 12 12 9 with E = 36, which spills, the same
-// forward and a faster adjoint (50 against 58).
+// forward and a faster adjoint (50 against 58).  192, 384, 768 and 1536 start with
+// radix 12 and save a pass against radix 4 passes and a last radix 3 (384^2 40 / 42 /
+// 34 -> 37 / 35 / 32, 1536^2 51 / 41 / 49 -> 47 / 40 / 45).
 struct FsSched {
     int N, E, nst, r[6];
 };
@@ -48,25 +50,25 @@ __host__ __device__ constexpr FsSched fs_sched(int N) {
         case 128: return {128, 16, 2, {16, 8}};
         case 144: return {144, 12, 2, {12, 12}};
         case 162: return {162, 18, 2, {18, 9}};
-        case 192: return {192, 12, 4, {4, 4, 4, 3}};
+        case 192: return {192, 12, 3, {12, 4, 4}};
         case 216: return {216, 12, 3, {12, 6, 3}};
         case 256: return {256, 16, 2, {16, 16}};
         case 288: return {288, 12, 3, {12, 12, 2}};
         case 324: return {324, 18, 2, {18, 18}};
-        case 384: return {384, 12, 5, {4, 4, 4, 2, 3}};
+        case 384: return {384, 12, 4, {12, 4, 4, 2}};
         case 432: return {432, 12, 3, {12, 12, 3}};
         case 486: return {486, 18, 3, {18, 9, 3}};
         case 512: return {512, 16, 3, {16, 8, 4}};
         case 576: return {576, 24, 2, {24, 24}};
         case 648: return {648, 18, 3, {18, 18, 2}};
-        case 768: return {768, 12, 5, {4, 4, 4, 4, 3}};
+        case 768: return {768, 12, 4, {12, 4, 4, 4}};
         case 864: return {864, 12, 3, {12, 12, 6}};
         case 972: return {972, 18, 3, {18, 18, 3}};
         case 1024: return {1024, 16, 3, {16, 16, 4}};
         case 1152: return {1152, 24, 3, {12, 12, 8}};
         case 1296: return {1296, 12, 4, {6, 6, 6, 6}};
         case 1458: return {1458, 18, 3, {18, 9, 9}};
-        case 1536: return {1536, 12, 6, {4, 4, 4, 4, 2, 3}};
+        case 1536: return {1536, 12, 5, {12, 4, 4, 4, 2}};
         case 1728: return {1728, 12, 3, {12, 12, 12}};
         case 1944: return {1944, 18, 3, {18, 18, 6}};
         case 2048: return {2048, 16, 3, {16, 16, 8}};

@@ -440,19 +440,17 @@ int batch_c2r_blocks(int H, int W, int threads);
 // tile shape of step 4's maxima: rows x cols cells, bands x column blocks tiles
 void batch_tile_shape(int H, int W, int threads, int* rows, int* cols, int* bands, int* nbx);
 bool batch_threads_ok(int stage, int threads);   // stage 0 r2c, 1 rows, 2 c2r
-// The four stage kernels, each a persistent loop over a device work queue of
-// `items` (image, block) pairs (*queue counts taken items and must be 0 at the
-// launch; the peak stage takes one image per item).  grid = 0 picks the
-// resident-block count of the device.
-cudaError_t launch_batch_r2c(const BatchImg* imgs, const int2* items, int nitems, unsigned* queue, const float* in,
-                             float2* ws, int threads, int maxH, cudaStream_t st);
-cudaError_t launch_batch_rows(const BatchImg* imgs, const int2* items, int nitems, unsigned* queue, float2* ws,
-                              int interp, int threads, int maxW, cudaStream_t st);
-cudaError_t launch_batch_c2r(const BatchImg* imgs, const int2* items, int nitems, unsigned* queue, const float2* ws,
-                             float* maps, unsigned* tmax, int threads, int maxH, cudaStream_t st);
-cudaError_t launch_batch_peaks(const BatchImg* imgs, int nimg, unsigned* queue, const float* maps, const unsigned* tmax,
+// The four stage kernels: one block per `items` entry, an (image, block) pair (the
+// peak stage: one block per image); pdl: programmatic dependent launch.
+cudaError_t launch_batch_r2c(const BatchImg* imgs, const int2* items, int nitems, const float* in, float2* ws,
+                             int threads, int maxH, cudaStream_t st, bool pdl);
+cudaError_t launch_batch_rows(const BatchImg* imgs, const int2* items, int nitems, float2* ws, int interp,
+                              int threads, int maxW, cudaStream_t st, bool pdl);
+cudaError_t launch_batch_c2r(const BatchImg* imgs, const int2* items, int nitems, const float2* ws, float* maps,
+                             unsigned* tmax, int threads, int maxH, cudaStream_t st, bool pdl);
+cudaError_t launch_batch_peaks(const BatchImg* imgs, int nimg, const float* maps, const unsigned* tmax,
                                int c2r_threads, int top_k, float threshold, ft_peak* out, int32_t* count,
-                               size_t smem, cudaStream_t st);
+                               size_t smem, cudaStream_t st, bool pdl);
 size_t batch_peaks_smem(const BatchImg* host_imgs, int nimg, int c2r_threads, int top_k);
 
 // line verification of Sec. 4.5 (k_verify.cu): image element (v, u) of the
