@@ -668,23 +668,37 @@ class Batch:
 
 
 # ------------------------------------------------------------ autograd wrapper
+_funnel_function = None
+
+
+def _autograd_function():
+    """The autograd.Function of funnel_transform, made once (torch is imported on
+    first use): making a new one on every call cost most of the call's host time."""
+    global _funnel_function
+    if _funnel_function is None:
+        import torch
+
+        class _Funnel(torch.autograd.Function):
+            @staticmethod
+            def forward(ctx, x, plan):
+                ctx.plan = plan
+                x = x.contiguous()
+                out = torch.empty((x.shape[0], plan.Hp, plan.S), dtype=torch.float32, device=x.device)
+                ft_forward(plan, x, out)
+                return out
+
+            @staticmethod
+            def backward(ctx, g):
+                plan = ctx.plan
+                g = g.contiguous()
+                gi = torch.empty((g.shape[0], plan.H, plan.W), dtype=torch.float32, device=g.device)
+                ft_backward(plan, g, gi)
+                return gi, None
+
+        _funnel_function = _Funnel
+    return _funnel_function
+
+
 def funnel_transform(img, plan: Plan):
     """Differentiable forward: P = A img through ft_forward / ft_backward."""
-    import torch
-
-    class _Funnel(torch.autograd.Function):
-        @staticmethod
-        def forward(ctx, x):
-            x = x.contiguous()
-            out = torch.empty((x.shape[0], plan.Hp, plan.S), dtype=torch.float32, device=x.device)
-            ft_forward(plan, x, out)
-            return out
-
-        @staticmethod
-        def backward(ctx, g):
-            g = g.contiguous()
-            gi = torch.empty((g.shape[0], plan.H, plan.W), dtype=torch.float32, device=g.device)
-            ft_backward(plan, g, gi)
-            return gi
-
-    return _Funnel.apply(img)
+    return _autograd_function().apply(img, plan)
