@@ -14,12 +14,11 @@
 // global memory directly.  All index arithmetic is by compile-time constants.
 //
 // Twiddles come from a per-length table (FP64 values rounded to FP32, built on
-// the host): for pass s >= 1, row k of a full table holds w_k^q at column q
-// (q = 0 .. R-1), w_k = exp(-2 pi i k / (P R)); row k of a seed table holds
-// only w_k^e for the exponents e = 1, 2, 4, 8 below R (1, 2 for R = 3), and a
-// thread builds the other powers as products of at most four seeds (a few
-// FP32 roundings).  Rows are padded to an even length so that pairs load as
-// float4.  A radix-16 group reads 8 float4 of a full row against 2 of a seed
+// the host): for pass s >= 1, row k of a full table holds w_k^q, q = 1 .. R-1,
+// w_k = exp(-2 pi i k / (P R)); row k of a seed table holds only some of these
+// powers and a thread builds the others as products (at most three for radix 16: a
+// few FP32 roundings).  Entries are stored in pairs that load as float4.  A
+// radix-16 group reads 8 float4 of a full row against 2 of a seed
 // row and 11 complex products: the row kernels (steps 2-3, scattered rows k
 // per lane) run faster on seed tables (103 against 112 us per 64 x 1024^2),
 // the column kernels on full ones (step 4: 121 against 128 us).
@@ -93,17 +92,38 @@ __host__ __device__ constexpr int fs_P(int N, int s) {
     for (int j = 0; j < s; ++j) p *= fs_radix(N, j);
     return p;
 }
-// seed powers of a pass with radix R (exponents 1 << j below R) and the
-// twiddle row stride of a full or a seed table, rounded up to even (16-byte rows)
-__host__ __device__ constexpr int fs_nseed(int R) {
+// entries of a table row: a full table holds the powers 1 .. R - 1, a seed table
+// of radix 12 and above the powers 1, 2, 4, 8, ..., below that 1 .. b and the
+// multiples of b (b = 3 for R = 3, 6, 9, 2 for R = 4, else 4), as many float4
+// but with every other power one product of two entries
+__host__ __device__ constexpr int fs_seedbase(int R) { return R == 3 || R == 6 || R == 9 ? 3 : R == 4 ? 2 : 4; }
+__host__ __device__ constexpr int fs_nent(int R, bool seed) {
+    if (!seed) return R - 1;
+    const int b = fs_seedbase(R);
+    if (R < 12) return R <= b ? R - 1 : b + (R - 1) / b - 1;
     int n = 0;
     while ((1 << n) < R) ++n;
     return n;
 }
-__host__ __device__ constexpr int fs_rs(int R, bool seed) { return ((seed ? fs_nseed(R) : R) + 1) & ~1; }
+// the exponent of entry j, and the float4 (pairs of entries) a row takes
+__host__ __device__ constexpr int fs_entexp(int R, bool seed, int j) {
+    const int b = fs_seedbase(R);
+    return !seed ? j + 1 : R >= 12 ? 1 << j : j < b ? j + 1 : (j - b + 2) * b;
+}
+__host__ __device__ constexpr int fs_pairs(int R, bool seed) { return (fs_nent(R, seed) + 1) / 2; }
+// float4 index of pair h of row k of a pass with P rows: by rows (the pairs of a
+// row adjacent), or by pairs (those of successive rows adjacent) in the full
+// tables of the long column lengths, whose warps hold 8 to 16 rows: a load then
+// touches one or two lines instead of one per row (steps 1 and 4 of four 4096^2
+// images 180 / 178 -> 169 / 162 us, 8192 in 16 Mpx 72 / 70 -> 62 / 60; equal
+// within noise at 1024 and below, with 4 rows per warp or fewer)
+__host__ __device__ constexpr bool fs_bypairs(int N, bool seed) { return !seed && N > 1024; }
+__host__ __device__ constexpr int fs_pairpos(int N, int R, int P, bool seed, int h, int k) {
+    return fs_bypairs(N, seed) ? h * P + k : k * fs_pairs(R, seed) + h;
+}
 __host__ __device__ constexpr int fs_twoff(int N, int s, bool seed) {
     int o = 0;
-    for (int j = 1; j < s; ++j) o += fs_P(N, j) * fs_rs(fs_radix(N, j), seed);
+    for (int j = 1; j < s; ++j) o += fs_P(N, j) * 2 * fs_pairs(fs_radix(N, j), seed);
     return o;
 }
 __host__ __device__ constexpr int fs_twsize(int N, bool seed) { return fs_twoff(N, fs_nst(N), seed); }
@@ -160,20 +180,29 @@ __device__ __forceinline__ void cp_async_wait_all() {
 template <int SIGN>
 __device__ __forceinline__ float2 tw_sign(float2 w) { return SIGN > 0 ? make_float2(w.x, -w.y) : w; }
 
-// w[q] = w_k^q (conjugated for SIGN > 0), q = 1 .. R-1, from the seed row at wp:
-// the powers 1, 2, 4, ... are read, the others are products of two earlier ones
-template <int R, int SIGN>
-__device__ __forceinline__ void tw_powers(const float4* __restrict__ wp, float2 (&w)[R]) {
+// w[q] = w_k^q (conjugated for SIGN > 0), q = 1 .. R-1, from row k of the table wp
+// of a pass: the entries are read, the powers a seed table lacks are products of
+// two earlier ones
+template <int N, int R, int P, int SIGN, bool SEED>
+__device__ __forceinline__ void tw_powers(const float4* __restrict__ wp, int k, float2 (&w)[R]) {
+    constexpr int NE = fs_nent(R, SEED), SB = fs_seedbase(R);
+    wp += fs_pairpos(N, R, P, SEED, 0, k);
 #pragma unroll
-    for (int h = 0; h < fs_rs(R, true) / 2; ++h) {
-        const float4 a = __ldg(wp + h);
-        w[1 << (2 * h)] = tw_sign<SIGN>(make_float2(a.x, a.y));
-        if ((2 << (2 * h)) < R) w[2 << (2 * h)] = tw_sign<SIGN>(make_float2(a.z, a.w));
+    for (int h = 0; h < fs_pairs(R, SEED); ++h) {
+        const float4 a = __ldg(wp + fs_pairpos(N, R, P, SEED, h, 0));
+        w[fs_entexp(R, SEED, 2 * h)] = tw_sign<SIGN>(make_float2(a.x, a.y));
+        if (2 * h + 1 < NE) w[fs_entexp(R, SEED, 2 * h + 1)] = tw_sign<SIGN>(make_float2(a.z, a.w));
     }
+    if constexpr (SEED && R < 12) {
 #pragma unroll
-    for (int b = 2; b < R; b *= 2)
+        for (int q = SB + 1; q < R; ++q)
+            if (q % SB != 0) w[q] = cmul(w[q - q % SB], w[q % SB]);
+    } else if constexpr (SEED) {
 #pragma unroll
-        for (int q = b + 1; q < 2 * b && q < R; ++q) w[q] = cmul(w[q - b], w[b]);
+        for (int b = 2; b < R; b *= 2)
+#pragma unroll
+            for (int q = b + 1; q < 2 * b && q < R; ++q) w[q] = cmul(w[q - b], w[b]);
+    }
 }
 
 // radix 9 as 3 x 3 with the internal twiddles exp(SIGN 2 pi i m / 9)
@@ -292,25 +321,12 @@ struct FastFft {
         constexpr int R = fs_radix(N, s), P = fs_P(N, s), G = E / R;
 #pragma unroll
         for (int m = 0; m < G; ++m) {
-            if constexpr (P > 1 && SEED) {
-                constexpr int RS = fs_rs(R, true);
+            if constexpr (P > 1) {
                 const int k = (t + m * T) % P;
                 float2 w[R];
-                tw_powers<R, SIGN>(reinterpret_cast<const float4*>(stw + fs_twoff(N, s, true) + k * RS), w);
+                tw_powers<N, R, P, SIGN, SEED>(reinterpret_cast<const float4*>(stw + fs_twoff(N, s, SEED)), k, w);
 #pragma unroll
                 for (int q = 1; q < R; ++q) v[m * R + q] = cmul(v[m * R + q], w[q]);
-            } else if constexpr (P > 1) {
-                constexpr int RS = fs_rs(R, false);
-                const int k = (t + m * T) % P;
-                const float4* w = reinterpret_cast<const float4*>(stw + fs_twoff(N, s, false) + k * RS);
-#pragma unroll
-                for (int h = 0; h < RS / 2; ++h) {
-                    const float4 ww = __ldg(w + h);
-                    if (2 * h >= 1 && 2 * h < R)
-                        v[m * R + 2 * h] = cmul(v[m * R + 2 * h], tw_sign<SIGN>(make_float2(ww.x, ww.y)));
-                    if (2 * h + 1 < R)
-                        v[m * R + 2 * h + 1] = cmul(v[m * R + 2 * h + 1], tw_sign<SIGN>(make_float2(ww.z, ww.w)));
-                }
             }
             Dft<R, SIGN>::run(&v[m * R]);
         }

@@ -144,18 +144,17 @@ static ft_status build_chirps(ft_plan p) {
 }
 
 // Per-pass twiddles of the fixed-length kernels: for pass s >= 1 with radix R and
-// P = product of the earlier radices, row k (stride fs_rs(R, seed)) holds
-// exp(-2 pi i q k / (P R)) at column q (full table), or at column j the power
-// q = 1 << j for j < fs_nseed(R) (seed table: the row lengths fx, fw, fm), taken
-// from the exact-index table tw of length N; padding entries are zero.
+// P = product of the earlier radices, the powers w_k^q, w_k = exp(-2 pi i k / (P R)),
+// q = fs_entexp(R, seed, j) for entry j, k < P, from the exact-index table tw of
+// length N; pair h = j / 2 of row k is float4 fs_pairpos(...) of the pass.
 static void stage_twiddles(int N, const float2* tw, float2* out, bool seed) {
     for (int s = 1; s < fs_nst(N); ++s) {
-        const int R = fs_radix(N, s), P = fs_P(N, s), step = N / (P * R), RS = fs_rs(R, seed);
-        const int ncol = seed ? fs_nseed(R) : R;
+        const int R = fs_radix(N, s), P = fs_P(N, s), step = N / (P * R), NE = fs_nent(R, seed);
         float2* o = out + fs_twoff(N, s, seed);
         for (int k = 0; k < P; ++k)
-            for (int j = 0; j < RS; ++j)
-                o[k * RS + j] = j < ncol ? tw[(seed ? 1 << j : j) * k * step] : make_float2(0.f, 0.f);
+            for (int j = 0; j < 2 * fs_pairs(R, seed); ++j)
+                o[2 * fs_pairpos(N, R, P, seed, j / 2, k) + (j & 1)] =
+                    j < NE ? tw[fs_entexp(R, seed, j) * k * step] : make_float2(0.f, 0.f);
     }
 }
 
