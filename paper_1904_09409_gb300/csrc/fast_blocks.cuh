@@ -36,12 +36,15 @@ __device__ __forceinline__ void r2c_finish(float2 (&v)[fs_E(N)], float2* sm, int
     // element E - 1 - j >= E/2 of thread T - t; thread 0 writes l = T j
     // (j <= E/2) and needs Z[N - l], its own element E - j (element 0 for l = 0).
     // So only elements j >= E/2 go through shared memory.
+    const int st = spos(t), snt = spos(-t);
 #pragma unroll
     for (int m = 0; m < GL; ++m)
 #pragma unroll
         for (int q = 0; q < RL; ++q)
-            if (m + GL * q >= E / 2 && FT_IN(spos(F::out_pos(t, m, q)) * B + f, F::SLOTS, FT_DBG_FFT_SLOT))
-                sm[spos(F::out_pos(t, m, q)) * B + f] = v[m * RL + q];
+            if (m + GL * q >= E / 2) {
+                const int o = spos_plus(t, st, F::out_pos(0, m, q)) * B + f;
+                if (FT_IN(o, F::SLOTS, FT_DBG_FFT_SLOT)) sm[o] = v[m * RL + q];
+            }
     __syncthreads();
     if (!colok) return;
     auto el = [&](int j) -> float2 { return v[(j % GL) * RL + j / GL]; };
@@ -57,7 +60,7 @@ __device__ __forceinline__ void r2c_finish(float2 (&v)[fs_E(N)], float2* sm, int
     if (t != 0) {
 #pragma unroll
         for (int j = 0; j < E / 2; ++j) {
-            const int k = spos(N - t - T * j) * B + f;
+            const int k = spos_plus(-t, snt, N - T * j) * B + f;
             split_z(t + T * j, el(j), FT_IN(k, F::SLOTS, FT_DBG_FFT_SLOT) ? sm[k] : make_float2(0.f, 0.f), mid_scale);
         }
     } else {
@@ -330,6 +333,7 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
     constexpr int R0 = fs_radix(N, 0), G0 = E / R0;
     constexpr int RL = fs_radix(N, fs_nst(N) - 1), GL = E / RL;
     constexpr int STEPX = N / R0;                      // x' distance between a thread's elements
+    static_assert(R0 % 2 == 0, "half a row is whole elements of the first pass");
     using F = FastFft<N, +1, B, true>;
     // [B][W + 4] input rows (sample x at 2 + x, 16-byte aligned, two zeros on
     // each side) in the FFT's own exchange buffer: they are read only by the
@@ -396,12 +400,15 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
         const float2 zero = make_float2(0.f, 0.f);
 #pragma unroll
         for (int m = 0; m < G0; ++m) {
+            // element q is the sample x' = i for i < N/2, i - N beyond (i = t + m T +
+            // q N / R0: the row rotated by N/2), visited in ascending x'
             const int i = t + m * T;
             const int num = (i - N / 2) * Hp;
             int qf = floor_div(num, den);
             int rem = num - qf * den;
 #pragma unroll
-            for (int q = 0; q < R0; ++q) {
+            for (int qq = 0; qq < R0; ++qq) {
+                const int q = (qq + R0 / 2) % R0;
                 const float fr = (float)rem * inv;
                 const int c0 = qf + halfW;
                 float2 acc;
@@ -429,21 +436,14 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
         }
     }
     __syncthreads();                                   // the staged rows are dead from here
-    // The centring factor (-1)^i of the gathered samples is a shift of the
-    // transform by N/2: with Z the transform of the taps, the row gets
-    // G[s] = (-1)^(s + N/2) Z[(s + N/2) mod N], i.e. Z[s'] (times (-1)^s') goes
-    // to position (s' + N/2) mod N
+    // The centring factors (-1)^i of the gathered samples and (-1)^(s + N/2) of the
+    // result are rotations by N/2 of the transform's output and of its input
     F::template run<0>(v, sm, t, f, stw);
     if (l >= L) return true;
     float2* row = base + (size_t)l * N;
 #pragma unroll
     for (int m = 0; m < GL; ++m)
 #pragma unroll
-        for (int q = 0; q < RL; ++q) {
-            const int s = F::out_pos(t, m, q);
-            float2 val = v[m * RL + q];
-            if (s & 1) val = make_float2(-val.x, -val.y);
-            row[s < N / 2 ? s + N / 2 : s - N / 2] = val;
-        }
+        for (int q = 0; q < RL; ++q) row[fs_rotate<N, RL>(F::out_pos(t, m, q), q)] = v[m * RL + q];
     return true;
 }

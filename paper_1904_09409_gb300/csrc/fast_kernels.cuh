@@ -238,22 +238,20 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
 #pragma unroll
     for (int m = 0; m < G0; ++m)
 #pragma unroll
-        for (int q = 0; q < R0; ++q) {
-            const int s = F::template in_pos<0>(t, m, q);
-            float2 g = (l < L) ? row[s] : make_float2(0.f, 0.f);
-            if (s & 1) g = make_float2(-g.x, -g.y);
-            v[m * R0 + q] = g;
-        }
+        for (int q = 0; q < R0; ++q)
+            v[m * R0 + q] = (l < L) ? row[fs_rotate<N, R0>(F::template in_pos<0>(t, m, q), q)] : make_float2(0.f, 0.f);
     F::template run<0>(v, sm, t, f, stw);
-    // gV[x'] = (-1)^{i + N/2} z[i], i = x' + N/2
+    // gV[x'] = (-1)^{i + N/2} z[i], i = x' + N/2, z the transform of (-1)^s g[s]: the
+    // signs are the rotations of the transform's input and output by N/2
+    const int st = spos(t);
 #pragma unroll
     for (int m = 0; m < GL; ++m)
 #pragma unroll
         for (int q = 0; q < RL; ++q) {
-            const int i = F::out_pos(t, m, q);
-            float2 z = v[m * RL + q];
-            if ((i + N / 2) & 1) z = make_float2(-z.x, -z.y);
-            sm[spos(i) * B + f] = z;
+            const int c = F::out_pos(0, m, q);
+            const int o = RL % 2 == 0 ? spos_plus(t, st, q < RL / 2 ? c + N / 2 : c - N / 2)
+                                      : spos(fs_rotate<N, RL>(t + c, q));
+            sm[o * B + f] = v[m * RL + q];
         }
     __syncthreads();
     if (l >= L) return;

@@ -168,6 +168,14 @@ __host__ __device__ constexpr int fs_Brow(int N) { return fs_clampB((128 + (fs_w
 // spreads the strided stores of the first pass over the banks)
 __host__ __device__ constexpr int spos(int n) { return n + (n >> 4); }
 __host__ __device__ constexpr int fs_slots(int N) { return spos(N - 1) + 1; }
+// the slot of sample n + c, given sn = spos(n): for a constant c that is a
+// multiple of 16 a constant distance, which becomes the access's immediate offset
+__device__ __forceinline__ int spos_plus(int n, int sn, int c) { return (c & 15) == 0 ? sn + c + (c >> 4) : spos(n + c); }
+// position pos of element q of a pass with radix R, rotated by half the length
+template <int N, int R>
+__device__ __forceinline__ int fs_rotate(int pos, int q) {
+    return (R % 2 == 0 ? q < R / 2 : pos < N / 2) ? pos + N / 2 : pos - N / 2;
+}
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
@@ -339,21 +347,24 @@ struct FastFft {
         for (int m = 0; m < G; ++m) {
             const int i = t + m * T;
             const int k = i % P;
-            const int j = (i - k) * R + k;
+            const int j = (i - k) * R + k, sj = spos(j);
 #pragma unroll
-            for (int q = 0; q < R; ++q)
-                if (FT_IN(spos(j + q * P) * B + f, SLOTS, FT_DBG_FFT_SLOT)) sm[spos(j + q * P) * B + f] = v[m * R + q];
+            for (int q = 0; q < R; ++q) {
+                const int o = spos_plus(j, sj, q * P) * B + f;
+                if (FT_IN(o, SLOTS, FT_DBG_FFT_SLOT)) sm[o] = v[m * R + q];
+            }
         }
     }
 
     template <int s>
     __device__ __forceinline__ static void load(float2 (&v)[E], const float2* sm, int t, int f) {
         constexpr int R = fs_radix(N, s), G = E / R;
+        const int st = spos(t);
 #pragma unroll
         for (int m = 0; m < G; ++m)
 #pragma unroll
             for (int q = 0; q < R; ++q) {
-                const int k = spos(in_pos<s>(t, m, q)) * B + f;
+                const int k = spos_plus(t, st, in_pos<s>(0, m, q)) * B + f;
                 v[m * R + q] = FT_IN(k, SLOTS, FT_DBG_FFT_SLOT) ? sm[k] : make_float2(0.f, 0.f);
             }
     }
