@@ -3,174 +3,225 @@
 // there for the derivation),
 //     row F (W) --F_W^- --> Fh --pre-chirp, 1/W--> y (M) --F_M^- --x Hc--> --F_M^+-->
 //     z --post-chirp, 1/M, support mask, (-1)^k--> V (S) --F_S^+--> G, (-1)^(s+S/2)
-// for W = S and M = 2W where all three lengths have a compile-time schedule.
+// for W = S and M = 2W where both lengths have a compile-time schedule.
 //
-// One block takes row l of B images (B = 256 / fs_T(M), at least 1): the four
-// transforms of each image's row run in registers (B side by side, exchanging
-// through one shared buffer), and the row's chirp tables (pre-chirp W + 1
-// entries, post-chirp S, chirp spectrum M) are read once per block for its B
-// images.  The grid runs the images fastest, so consecutive blocks share row l
-// and its tables stay in L2: the tables are read from memory about once per
-// call instead of once per image.  Between the transforms the data goes
-// through shared memory once (the re-indexing u mod W, the change from the
-// forward transform's output order to the inverse's input order, the
-// truncation to S samples); threads that hold no transform of the shorter
-// lengths W and S only join the barriers.
+// A length-M transform has G = fs_T(M) / fs_T(W) times the threads of a length-W
+// one (2 for the powers of two), so a block of B fs_T(M) threads takes G B rows:
+// the transforms of length W and S run on all G B rows at once, the two of length
+// M on B rows at a time in G rounds, and every thread has work in every pass.
+// (One round of B rows per block, half of the threads idle in the passes of length
+// W and S, took 124 us per 16 x 1024^2, this form 108, with
+// the centring factors as rotations and constant shared-memory offsets.)  Between the transforms the rows live
+// in a second shared buffer; the exchanges go through the first.  Rows are
+// numbered l batch + image, so consecutive rows share the chirp tables of row l
+// (pre-chirp W + 1 entries, post-chirp S, chirp spectrum M), which are read from
+// memory about once per call, and blocks are full whatever the batch.  The kernel
+// is bound by issue and latency at 16 warps per multiprocessor (four transforms
+// in a row keep about 170 registers live unbounded; 128 leave at most a few words
+// spilled), so what counts is the number of passes and table loads per row.
 #include "fft_fast.cuh"
 
-template <int W, int M, int S>
+template <int W>
 struct FrShape {
-    static constexpr int TM = fs_T(M), TW = fs_T(W), TS = fs_T(S);
-    static constexpr int B = TM >= 256 ? 1 : 256 / TM;         // rows (images) per block
+    static constexpr int M = 2 * W, TM = fs_T(M), TW = fs_T(W);
+    // rows per round: about 128 threads, or 256 where 128 / TM rows would leave most of
+    // a warp empty
+    static constexpr int B = TM >= 128 ? 1 : 128 / TM * TM >= 112 ? 128 / TM : 256 / TM;
+    static constexpr int G = TM / TW;                          // rounds
+    static constexpr int NR = G * B;                           // rows per block
     static constexpr int NT = TM * B;
-    // resident blocks of NT threads per multiprocessor the registers are sized
-    // for: four transforms in a row keep about 170 registers live unbounded;
-    // 128 (two blocks of 256 threads) leaves at most a few words spilled
+    // resident blocks of NT threads per multiprocessor the registers are sized for
     static constexpr int MINB = 512 / NT > 0 ? 512 / NT : 1;
-    static_assert(TW <= TM && TS <= TM, "the length-M transform has the most threads");
-    static constexpr int SLOTS_W = FastFft<W, -1, B>::SLOTS, SLOTS_M = FastFft<M, -1, B>::SLOTS,
-                         SLOTS_S = FastFft<S, -1, B>::SLOTS;
-    static constexpr int SLOTS = SLOTS_M > SLOTS_W ? (SLOTS_M > SLOTS_S ? SLOTS_M : SLOTS_S)
-                                                   : (SLOTS_W > SLOTS_S ? SLOTS_W : SLOTS_S);
+    static_assert(G >= 1 && G * TW == TM, "the rows of a block keep every thread busy");
+    static constexpr int SX_W = FastFft<W, -1, NR>::SLOTS, SX_M = FastFft<M, -1, B>::SLOTS;
+    static constexpr int SX = SX_M > SX_W ? SX_M : SX_W;       // exchange slots
+    static constexpr int SLOTS = SX + SX_W;                    // and the rows between the transforms
 };
 
-template <int W, int M, int S>
-__global__ void __launch_bounds__(FrShape<W, M, S>::NT, FrShape<W, M, S>::MINB)
+// row of the block's sample index: its frequency l, image and first element
+struct FrRow {
+    int l;
+    bool ok;                // a row of the launch (l = 0, the DC row, included)
+    float2* p;
+};
+__device__ __forceinline__ FrRow fr_row(float2* ws, int r, int L, int batch, int S) {
+    FrRow o;
+    o.l = r / batch;
+    o.ok = o.l < L;
+    o.p = ws + ((size_t)(r - o.l * batch) * L + o.l) * S;
+    return o;
+}
+
+// a copy of a thread index that the compiler takes for a new value: each transform
+// of the chain computes its shared-memory addresses from its own copy, so that
+// those of one transform are not kept in registers through the others
+__device__ __forceinline__ int fr_fresh(int t) {
+    asm volatile("" : "+r"(t));
+    return t;
+}
+
+// prefetch into L1 the chirp tables of the rows of frequencies l0 .. l1 (len
+// complex values each, contiguous over l): one 128-byte line per thread and step
+__device__ __forceinline__ void fr_prefetch(const float2* table, int len, int l0, int l1, int nt) {
+    const char* p = reinterpret_cast<const char*>(table + (size_t)l0 * len);
+    const int bytes = (l1 - l0 + 1) * len * (int)sizeof(float2);
+    for (int o = threadIdx.x * 128; o < bytes; o += nt * 128) asm volatile("prefetch.global.L1 [%0];" ::"l"(p + o));
+}
+
+// the samples k = x' + S/2 of row l inside the support, x' H' / (2 l) in
+// [-W/2, W/2 - 1]: lo <= k <= hi
+__device__ __forceinline__ void fr_support(int l, int Hp, int W, int S, int& lo, int& hi) {
+    lo = ceil_div(-(W / 2) * 2 * l, Hp) + S / 2;
+    hi = floor_div((W / 2 - 1) * 2 * l, Hp) + S / 2;
+}
+
+template <int W>
+__global__ void __launch_bounds__(FrShape<W>::NT, FrShape<W>::MINB)
 k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, const float2* __restrict__ stw_w,
                          const float2* __restrict__ stw_m, const float2* __restrict__ stw_s,
                          const float2* __restrict__ chirp_u, const float2* __restrict__ chirp_x,
                          const float2* __restrict__ hc) {
-    using Sh = FrShape<W, M, S>;
-    constexpr int B = Sh::B, TW = Sh::TW, TS = Sh::TS;
-    constexpr int EW = fs_E(W), EM = fs_E(M), ES = fs_E(S);
-    using FW = FastFft<W, -1, B, true>;
+    using Sh = FrShape<W>;
+    constexpr int M = Sh::M, S = W, B = Sh::B, NR = Sh::NR;
+    constexpr int EW = fs_E(W), EM = fs_E(M);
+    using FW = FastFft<W, -1, NR, true>;
     using FMf = FastFft<M, -1, B, true>;
     using FMi = FastFft<M, +1, B, true>;
-    using FS = FastFft<S, +1, B, true>;
+    using FS = FastFft<S, +1, NR, true>;
     constexpr int R0W = fs_radix(W, 0), G0W = EW / R0W, RLW = fs_radix(W, fs_nst(W) - 1), GLW = EW / RLW;
     constexpr int R0M = fs_radix(M, 0), G0M = EM / R0M, RLM = fs_radix(M, fs_nst(M) - 1), GLM = EM / RLM;
-    constexpr int R0S = fs_radix(S, 0), G0S = ES / R0S, RLS = fs_radix(S, fs_nst(S) - 1), GLS = ES / RLS;
-    extern __shared__ float2 sm[];
-    const int l = blockIdx.y;
-    const int f = threadIdx.x % B, t = threadIdx.x / B;
-    const int img = blockIdx.x * B + f;
-    const bool rowok = img < batch;
-    float2* row = ws + ((size_t)img * L + l) * S;       // W values in, S values out
-    if (l == 0) {                                       // the DC row is zero (the whole block)
-        if (rowok)
-            for (int k = t; k < S; k += Sh::TM) row[k] = make_float2(0.f, 0.f);
-        return;
+    static_assert(R0W % 2 == 0 && R0M % 2 == 0, "halves of a row are whole elements of the first pass");
+    extern __shared__ __align__(16) float2 sm[];
+    float2* rows = sm + Sh::SX;                        // [spos(k)][NR]
+    pdl_trigger();
+    {   // the tables of the block's frequencies (they do not depend on the predecessor)
+        const int l0 = blockIdx.x * NR / batch, l1 = min((blockIdx.x * NR + NR - 1) / batch, L - 1);
+        if (l1 - l0 < 2) {
+            fr_prefetch(chirp_u, W + 1, l0, l1, Sh::NT);
+            fr_prefetch(hc, M, l0, l1, Sh::NT);
+            fr_prefetch(chirp_x, S, l0, l1, Sh::NT);
+        }
     }
+    pdl_wait();
 
-    // ---- F_W^- of the row (threads t < TW)
-    if (t < TW) {
+    const int fr = threadIdx.x % NR, tr0 = threadIdx.x / NR;
+    const FrRow rw = fr_row(ws, blockIdx.x * NR + fr, L, batch, S);
+    // ---- F_W^- of the block's rows
+    {
+        const int tr = fr_fresh(tr0);
         float2 v[EW];
 #pragma unroll
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q)
-                v[m * R0W + q] = rowok ? row[FW::template in_pos<0>(t, m, q)] : make_float2(0.f, 0.f);
-        FW::template run<0>(v, sm, t, f, stw_w);
+                v[m * R0W + q] = rw.ok ? __ldcg(rw.p + fs_rotate<W, R0W>(FW::template in_pos<0>(tr, m, q), q))
+                                       : make_float2(0.f, 0.f);
+        FW::template run<0>(v, sm, tr, fr, stw_w);
 #pragma unroll
         for (int m = 0; m < GLW; ++m)
 #pragma unroll
-            for (int q = 0; q < RLW; ++q) sm[spos(FW::out_pos(t, m, q)) * B + f] = v[m * RLW + q];
-    } else {
-        FW::template idle<0>();
+            for (int q = 0; q < RLW; ++q) rows[spos_plus(tr, spos(tr), FW::out_pos(0, m, q)) * NR + fr] = v[m * RLW + q];
     }
     __syncthreads();
 
-    // ---- y[i] = Fh[u mod W] (+-1/W, halved at u = +-W/2) x pre-chirp, u = i - W/2 (i <= W), 0 beyond
-    float2 v[EM];
-    {
-        const float2* cu = chirp_u + (size_t)l * (W + 1);
-        const float invW = 1.f / (float)W;
+    const int f = threadIdx.x % B, t0 = threadIdx.x / B;
+#pragma unroll 1
+    for (int g = 0; g < Sh::G; ++g) {
+        const int fg = g * B + f;
+        const FrRow rm = fr_row(ws, blockIdx.x * NR + fg, L, batch, S);
+        const int t = fr_fresh(t0), st = spos(t);
+        const int l = rm.ok ? rm.l : 0;                // the tables' row; rows past the end are not stored
+        // ---- y[i] = Fh[u mod W] (halved at u = +-W/2) x pre-chirp, u = i - W/2 (i <= W),
+        // 0 beyond: only element q = R0M / 2 of thread 0 (i = W) of the upper half
+        float2 v[EM];
+        {
+            const float2* cu = chirp_u + (size_t)l * (W + 1);
+#pragma unroll
+            for (int m = 0; m < G0M; ++m)
+#pragma unroll
+                for (int q = 0; q < R0M; ++q) {
+                    constexpr bool quarters = R0M % 4 == 0;        // i < W/2 is decided by q
+                    float2 y = make_float2(0.f, 0.f);
+                    if (q < R0M / 2 || (q == R0M / 2 && m == 0 && t == 0)) {
+                        const int i = FMf::template in_pos<0>(t, m, q);
+                        const int c = FMf::template in_pos<0>(0, m, q);
+                        int slot;
+                        if (quarters)
+                            slot = spos_plus(t, st, q < R0M / 4 ? c + W / 2 : c - W / 2);
+                        else
+                            slot = spos(i < W / 2 ? i + W / 2 : i - W / 2);
+                        float2 a = rows[slot * NR + fg];
+                        if (m == 0 && (q == 0 || q == R0M / 2) && t == 0) a = cscale(a, 0.5f);
+                        y = cmul(a, __ldg(cu + i));
+                    }
+                    v[m * R0M + q] = y;
+                }
+        }
+        // ---- F_M^-, times the chirp spectrum, back to the input order, F_M^+
+        FMf::template run<0>(v, sm, t, f, stw_m);
+        {
+            const float2* hl = hc + (size_t)l * M;
+#pragma unroll
+            for (int m = 0; m < GLM; ++m)
+#pragma unroll
+                for (int q = 0; q < RLM; ++q) {
+                    const int k = FMf::out_pos(t, m, q);
+                    sm[spos_plus(t, st, FMf::out_pos(0, m, q)) * B + f] = cmul(v[m * RLM + q], __ldg(hl + k));
+                }
+        }
+        __syncthreads();
+        const int ti = fr_fresh(t0), sti = spos(ti);
 #pragma unroll
         for (int m = 0; m < G0M; ++m)
 #pragma unroll
-            for (int q = 0; q < R0M; ++q) {
-                const int i = FMf::template in_pos<0>(t, m, q);
-                float2 y = make_float2(0.f, 0.f);
-                if (i <= W) {
-                    const int u = i - W / 2;
-                    const int k = u < 0 ? u + W : u;
-                    float sc = (u & 1) ? -invW : invW;
-                    if (u == W / 2 || u == -W / 2) sc *= 0.5f;
-                    const float2 a = sm[spos(k) * B + f];
-                    y = cmul(make_float2(a.x * sc, a.y * sc), __ldg(cu + i));
-                }
-                v[m * R0M + q] = y;
-            }
-    }
-    __syncthreads();
-
-    // ---- F_M^-, times the chirp spectrum, back to the input order, F_M^+
-    FMf::template run<0>(v, sm, t, f, stw_m);
-    {
-        const float2* hl = hc + (size_t)l * M;
-#pragma unroll
-        for (int m = 0; m < GLM; ++m)
-#pragma unroll
-            for (int q = 0; q < RLM; ++q) {
-                const int k = FMf::out_pos(t, m, q);
-                sm[spos(k) * B + f] = cmul(v[m * RLM + q], __ldg(hl + k));
-            }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < G0M; ++m)
-#pragma unroll
-        for (int q = 0; q < R0M; ++q) v[m * R0M + q] = sm[spos(FMi::template in_pos<0>(t, m, q)) * B + f];
-    __syncthreads();
-    FMi::template run<0>(v, sm, t, f, stw_m);
-
-    // ---- V[k] = z[k] / M x post-chirp inside the support, (-1)^k, k < S
-    {
-        const float2* cx = chirp_x + (size_t)l * S;
-        const float invM = 1.f / (float)M;
-        const long long den = 2ll * l;
-#pragma unroll
-        for (int m = 0; m < GLM; ++m)
-#pragma unroll
-            for (int q = 0; q < RLM; ++q) {
-                const int k = FMi::out_pos(t, m, q);
-                if (k < S) {
-                    const long long num = (long long)(k - S / 2) * Hp;       // p = num / den
-                    float2 r = make_float2(0.f, 0.f);
-                    if (num >= -(long long)(W / 2) * den && num <= (long long)(W / 2 - 1) * den) {
-                        r = cmul(v[m * RLM + q], __ldg(cx + k));
-                        const float sc = (k & 1) ? -invM : invM;
-                        r = make_float2(r.x * sc, r.y * sc);
-                    }
-                    sm[spos(k) * B + f] = r;
-                }
-            }
-    }
-    __syncthreads();
-
-    // ---- step 3: F_S^+ (threads t < TS), output sign (-1)^(s + S/2)
-    if (t < TS) {
-        float2 g[ES];
-#pragma unroll
-        for (int m = 0; m < G0S; ++m)
-#pragma unroll
-            for (int q = 0; q < R0S; ++q) g[m * R0S + q] = sm[spos(FS::template in_pos<0>(t, m, q)) * B + f];
+            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = sm[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q)) * B + f];
         __syncthreads();
-        FS::template run<0>(g, sm, t, f, stw_s);
-        if (rowok) {
+        FMi::template run<0>(v, sm, ti, f, stw_m);
+        // ---- V[k] = z[k] / (W M) x post-chirp inside the support, for k < S = M / 2 (the
+        // lower half of the last pass's elements), stored rotated by S/2; the DC row is zero
+        {
+            const float2* cx = chirp_x + (size_t)l * S;
+            const float sc = 1.f / ((float)M * (float)W);
+            int lo, hi;
+            fr_support(l, Hp, W, S, lo, hi);
+            if (l == 0) hi = -1;
 #pragma unroll
-            for (int m = 0; m < GLS; ++m)
+            for (int m = 0; m < GLM; ++m)
 #pragma unroll
-                for (int q = 0; q < RLS; ++q) {
-                    const int s = FS::out_pos(t, m, q);
-                    float2 val = g[m * RLS + q];
-                    if ((s + S / 2) & 1) val = make_float2(-val.x, -val.y);
-                    row[s] = val;
+                for (int q = 0; q < RLM; ++q) {
+                    const int k = FMi::out_pos(ti, m, q);
+                    if (RLM % 2 == 0 ? q < RLM / 2 : k < S) {
+                        float2 r = make_float2(0.f, 0.f);
+                        if (k >= lo && k <= hi) r = cscale(cmul(v[m * RLM + q], __ldg(cx + k)), sc);
+                        int slot;
+                        if (RLM % 4 == 0)                          // k < S/2 is decided by q
+                            slot = spos_plus(ti, sti, FMi::out_pos(0, m, q) + (q < RLM / 4 ? S / 2 : -S / 2));
+                        else
+                            slot = spos(k < S / 2 ? k + S / 2 : k - S / 2);
+                        rows[slot * NR + fg] = r;
+                    }
                 }
         }
-    } else {
-        __syncthreads();
-        FS::template idle<0>();
+    }
+    __syncthreads();
+
+    // ---- step 3: F_S^+ of the block's rows.  The centring factors (-1)^k of V and
+    // (-1)^(s + S/2) of G are the rotations by S/2 of its input and output
+    {
+        const int tr = fr_fresh(tr0), str = spos(tr);
+        float2 v[EW];
+#pragma unroll
+        for (int m = 0; m < G0W; ++m)
+#pragma unroll
+            for (int q = 0; q < R0W; ++q)
+                v[m * R0W + q] = rows[spos_plus(tr, str, FS::template in_pos<0>(0, m, q)) * NR + fr];
+        FS::template run<0>(v, sm, tr, fr, stw_s);
+        if (rw.ok) {
+#pragma unroll
+            for (int m = 0; m < GLW; ++m)
+#pragma unroll
+                for (int q = 0; q < RLW; ++q) rw.p[fs_rotate<S, RLW>(FS::out_pos(tr, m, q), q)] = v[m * RLW + q];
+        }
     }
 }
 
@@ -178,151 +229,163 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
 // O the output sign, D_x the post-chirp / 1/M / mask / (-1)^k, D_h the chirp
 // spectrum, D_u the pre-chirp and P the re-indexing u mod W with its weights,
 //     gF = F_W^+ P^T conj(D_u) F_M^+ conj(D_h) F_M^- conj(D_x) F_S^- O gG.
-template <int W, int M, int S>
-__global__ void __launch_bounds__(FrShape<W, M, S>::NT, FrShape<W, M, S>::MINB)
+// conj(D_u) is applied as F_M^+ ends, and P^T stores entry i = u + W/2 at u mod
+// W; the two Nyquist entries i = 0 and i = W share index W/2, so the second goes
+// to a slot of its own and is added when F_W^+ reads index W/2.
+template <int W>
+__global__ void __launch_bounds__(FrShape<W>::NT, FrShape<W>::MINB)
 k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, const float2* __restrict__ stw_w,
                              const float2* __restrict__ stw_m, const float2* __restrict__ stw_s,
                              const float2* __restrict__ chirp_u, const float2* __restrict__ chirp_x,
                              const float2* __restrict__ hc) {
-    using Sh = FrShape<W, M, S>;
-    constexpr int B = Sh::B, TW = Sh::TW, TS = Sh::TS;
-    constexpr int EW = fs_E(W), EM = fs_E(M), ES = fs_E(S);
-    using FS = FastFft<S, -1, B, true>;
+    using Sh = FrShape<W>;
+    constexpr int M = Sh::M, S = W, B = Sh::B, NR = Sh::NR;
+    constexpr int EW = fs_E(W), EM = fs_E(M);
+    using FS = FastFft<S, -1, NR, true>;
     using FMf = FastFft<M, -1, B, true>;
     using FMi = FastFft<M, +1, B, true>;
-    using FW = FastFft<W, +1, B, true>;
+    using FW = FastFft<W, +1, NR, true>;
     constexpr int R0W = fs_radix(W, 0), G0W = EW / R0W, RLW = fs_radix(W, fs_nst(W) - 1), GLW = EW / RLW;
     constexpr int R0M = fs_radix(M, 0), G0M = EM / R0M, RLM = fs_radix(M, fs_nst(M) - 1), GLM = EM / RLM;
-    constexpr int R0S = fs_radix(S, 0), G0S = ES / R0S, RLS = fs_radix(S, fs_nst(S) - 1), GLS = ES / RLS;
-    extern __shared__ float2 sm[];
-    const int l = blockIdx.y;
-    const int f = threadIdx.x % B, t = threadIdx.x / B;
-    const int img = blockIdx.x * B + f;
-    const bool rowok = img < batch;
-    float2* row = ws + ((size_t)img * L + l) * S;       // S values in, W values out
-    if (l == 0) {
-        if (rowok)
-            for (int x = t; x < W; x += Sh::TM) row[x] = make_float2(0.f, 0.f);
-        return;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* rows = sm + Sh::SX;
+    __shared__ float2 nyq[NR];
+    pdl_trigger();
+    {   // the tables of the block's frequencies (they do not depend on the predecessor)
+        const int l0 = blockIdx.x * NR / batch, l1 = min((blockIdx.x * NR + NR - 1) / batch, L - 1);
+        if (l1 - l0 < 2) {
+            fr_prefetch(chirp_u, W + 1, l0, l1, Sh::NT);
+            fr_prefetch(hc, M, l0, l1, Sh::NT);
+            fr_prefetch(chirp_x, S, l0, l1, Sh::NT);
+        }
     }
+    pdl_wait();
 
-    // ---- O, F_S^- (threads t < TS)
-    if (t < TS) {
-        float2 g[ES];
+    const int fr = threadIdx.x % NR, tr0 = threadIdx.x / NR;
+    const FrRow rw = fr_row(ws, blockIdx.x * NR + fr, L, batch, S);
+    // ---- O, F_S^-, (-1)^k: rotations by S/2 of the input and the output
+    {
+        const int tr = fr_fresh(tr0);
+        float2 v[EW];
 #pragma unroll
-        for (int m = 0; m < G0S; ++m)
+        for (int m = 0; m < G0W; ++m)
 #pragma unroll
-            for (int q = 0; q < R0S; ++q) {
-                const int s = FS::template in_pos<0>(t, m, q);
-                float2 val = rowok ? row[s] : make_float2(0.f, 0.f);
-                if ((s + S / 2) & 1) val = make_float2(-val.x, -val.y);
-                g[m * R0S + q] = val;
+            for (int q = 0; q < R0W; ++q)
+                v[m * R0W + q] = rw.ok ? __ldcg(rw.p + fs_rotate<S, R0W>(FS::template in_pos<0>(tr, m, q), q))
+                                       : make_float2(0.f, 0.f);
+        FS::template run<0>(v, sm, tr, fr, stw_s);
+#pragma unroll
+        for (int m = 0; m < GLW; ++m)
+#pragma unroll
+            for (int q = 0; q < RLW; ++q) {
+                const int c = FS::out_pos(0, m, q);
+                const int slot = RLW % 2 == 0 ? spos_plus(tr, spos(tr), q < RLW / 2 ? c + S / 2 : c - S / 2)
+                                              : spos(fs_rotate<S, RLW>(tr + c, q));
+                rows[slot * NR + fr] = v[m * RLW + q];
             }
-        FS::template run<0>(g, sm, t, f, stw_s);
-#pragma unroll
-        for (int m = 0; m < GLS; ++m)
-#pragma unroll
-            for (int q = 0; q < RLS; ++q) sm[spos(FS::out_pos(t, m, q)) * B + f] = g[m * RLS + q];
-    } else {
-        FS::template idle<0>();
     }
     __syncthreads();
 
-    // ---- conj(D_x) on k < S, zero beyond, F_M^-
-    float2 v[EM];
-    {
-        const float2* cx = chirp_x + (size_t)l * S;
-        const float invM = 1.f / (float)M;
-        const long long den = 2ll * l;
+    const int f = threadIdx.x % B, t0 = threadIdx.x / B;
+#pragma unroll 1
+    for (int g = 0; g < Sh::G; ++g) {
+        const int fg = g * B + f;
+        const FrRow rm = fr_row(ws, blockIdx.x * NR + fg, L, batch, S);
+        const int t = fr_fresh(t0), st = spos(t);
+        const int l = rm.ok ? rm.l : 0;
+        // ---- conj(D_x) on k < S = M / 2, zero beyond and for the DC row, F_M^-
+        float2 v[EM];
+        {
+            const float2* cx = chirp_x + (size_t)l * S;
+            const float sc = 1.f / ((float)M * (float)W);
+            int lo, hi;
+            fr_support(l, Hp, W, S, lo, hi);
+            if (l == 0) hi = -1;
+#pragma unroll
+            for (int m = 0; m < G0M; ++m)
+#pragma unroll
+                for (int q = 0; q < R0M; ++q) {
+                    float2 r = make_float2(0.f, 0.f);
+                    if (q < R0M / 2) {
+                        const int k = FMf::template in_pos<0>(t, m, q);
+                        if (k >= lo && k <= hi) {
+                            const float2 c = __ldg(cx + k);
+                            const float2 a = rows[spos_plus(t, st, FMf::template in_pos<0>(0, m, q)) * NR + fg];
+                            r = cscale(cmul(a, make_float2(c.x, -c.y)), sc);
+                        }
+                    }
+                    v[m * R0M + q] = r;
+                }
+        }
+        FMf::template run<0>(v, sm, t, f, stw_m);
+        {
+            const float2* hl = hc + (size_t)l * M;
+#pragma unroll
+            for (int m = 0; m < GLM; ++m)
+#pragma unroll
+                for (int q = 0; q < RLM; ++q) {
+                    const int k = FMf::out_pos(t, m, q);
+                    const float2 h = __ldg(hl + k);
+                    sm[spos_plus(t, st, FMf::out_pos(0, m, q)) * B + f] = cmul(v[m * RLM + q], make_float2(h.x, -h.y));
+                }
+        }
+        __syncthreads();
+        const int ti = fr_fresh(t0), sti = spos(ti);
 #pragma unroll
         for (int m = 0; m < G0M; ++m)
 #pragma unroll
-            for (int q = 0; q < R0M; ++q) {
-                const int k = FMf::template in_pos<0>(t, m, q);
-                float2 r = make_float2(0.f, 0.f);
-                if (k < S) {
-                    const long long num = (long long)(k - S / 2) * Hp;
-                    if (num >= -(long long)(W / 2) * den && num <= (long long)(W / 2 - 1) * den) {
-                        const float2 c = __ldg(cx + k);
-                        r = cmul(sm[spos(k) * B + f], make_float2(c.x, -c.y));
-                        const float sc = (k & 1) ? -invM : invM;
-                        r = make_float2(r.x * sc, r.y * sc);
+            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = sm[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q)) * B + f];
+        __syncthreads();
+        FMi::template run<0>(v, sm, ti, f, stw_m);
+        // ---- conj(D_u) and P^T on the entries i = u + W/2 <= W (halved at u = +-W/2)
+        {
+            const float2* cu = chirp_u + (size_t)l * (W + 1);
+#pragma unroll
+            for (int m = 0; m < GLM; ++m)
+#pragma unroll
+                for (int q = 0; q < RLM; ++q) {
+                    const int i = FMi::out_pos(ti, m, q);
+                    if (RLM % 2 == 0 ? (q < RLM / 2 || (q == RLM / 2 && m == 0 && ti == 0)) : i <= W) {
+                        const float2 c = __ldg(cu + i);
+                        float2 r = cmul(v[m * RLM + q], make_float2(c.x, -c.y));
+                        if (i == 0 || i == W) r = cscale(r, 0.5f);
+                        if (i == W)
+                            nyq[fg] = r;
+                        else
+                            rows[spos(i < W / 2 ? i + W / 2 : i - W / 2) * NR + fg] = r;
                     }
                 }
-                v[m * R0M + q] = r;
-            }
-    }
-    __syncthreads();
-    FMf::template run<0>(v, sm, t, f, stw_m);
-    {
-        const float2* hl = hc + (size_t)l * M;
-#pragma unroll
-        for (int m = 0; m < GLM; ++m)
-#pragma unroll
-            for (int q = 0; q < RLM; ++q) {
-                const int k = FMf::out_pos(t, m, q);
-                const float2 h = __ldg(hl + k);
-                sm[spos(k) * B + f] = cmul(v[m * RLM + q], make_float2(h.x, -h.y));
-            }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < G0M; ++m)
-#pragma unroll
-        for (int q = 0; q < R0M; ++q) v[m * R0M + q] = sm[spos(FMi::template in_pos<0>(t, m, q)) * B + f];
-    __syncthreads();
-    FMi::template run<0>(v, sm, t, f, stw_m);
-#pragma unroll
-    for (int m = 0; m < GLM; ++m)
-#pragma unroll
-        for (int q = 0; q < RLM; ++q) {
-            const int k = FMi::out_pos(t, m, q);
-            if (k <= W) sm[spos(k) * B + f] = v[m * RLM + q];       // z[i], i = u + W/2 <= W
         }
+    }
     __syncthreads();
 
-    // ---- conj(D_u) and P^T: index x collects u = x (x <= W/2) or x - W, and
-    // index W/2 also u = -W/2; weight (-1)^u / W, halved at u = +-W/2; then F_W^+
-    if (t < TW) {
-        const float2* cu = chirp_u + (size_t)l * (W + 1);
-        const float invW = 1.f / (float)W;
-        float2 a[EW];
+    // ---- F_W^+ (the DC row's gradient is zero: its V is); the weight (-1)^u is a
+    // rotation of the result by W/2
+    {
+        const int tr = fr_fresh(tr0), str = spos(tr);
+        float2 v[EW];
 #pragma unroll
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q) {
-                const int x = FW::template in_pos<0>(t, m, q);
-                const int u = x <= W / 2 ? x : x - W;
-                float sc = (u & 1) ? -invW : invW;
-                if (x == W / 2) sc *= 0.5f;
-                const int i = u + W / 2;
-                const float2 c = __ldg(cu + i);
-                float2 r = cmul(sm[spos(i) * B + f], make_float2(c.x, -c.y));
-                r = make_float2(r.x * sc, r.y * sc);
-                if (x == W / 2) {                       // u = -W/2, the same weight
-                    const float2 c2 = __ldg(cu);
-                    const float2 r2 = cmul(sm[f], make_float2(c2.x, -c2.y));
-                    const float sc2 = ((-W / 2) & 1) ? -0.5f * invW : 0.5f * invW;
-                    r = make_float2(r.x + r2.x * sc2, r.y + r2.y * sc2);
-                }
-                a[m * R0W + q] = r;
+                float2 a = rows[spos_plus(tr, str, FW::template in_pos<0>(0, m, q)) * NR + fr];
+                if (FW::template in_pos<0>(tr, m, q) == W / 2) a = cadd(a, nyq[fr]);
+                v[m * R0W + q] = a;
             }
-        __syncthreads();
-        FW::template run<0>(a, sm, t, f, stw_w);
-        if (rowok) {
+        FW::template run<0>(v, sm, tr, fr, stw_w);
+        if (rw.ok) {
 #pragma unroll
             for (int m = 0; m < GLW; ++m)
 #pragma unroll
-                for (int q = 0; q < RLW; ++q) row[FW::out_pos(t, m, q)] = a[m * RLW + q];
+                for (int q = 0; q < RLW; ++q) rw.p[fs_rotate<W, RLW>(FW::out_pos(tr, m, q), q)] = v[m * RLW + q];
         }
-    } else {
-        __syncthreads();
-        FW::template idle<0>();
     }
 }
 
 // ------------------------------------------------------------------ dispatch
-#define FR_FAST_LENGTHS(X) X(128) X(192) X(256) X(384) X(512) X(768) X(1024) X(2048)
+#define FR_FAST_LENGTHS(X) \
+    X(128) X(144) X(162) X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512) X(576) X(648) X(768) X(864) \
+    X(972) X(1024) X(1152) X(1536) X(2048)
 
 bool fourier_fast_ok(int W, int M, int S) {
     if (W != S || M != 2 * W) return false;
@@ -338,33 +401,25 @@ bool fourier_fast_ok(int W, int M, int S) {
 template <int N>
 static cudaError_t go_fourier(bool adj, float2* ws, int Hp, int L, int batch, const float2* stw_w,
                               const float2* stw_m, const float2* stw_s, const float2* cu, const float2* cx,
-                              const float2* hc, cudaStream_t st) {
-    using Sh = FrShape<N, 2 * N, N>;
+                              const float2* hc, cudaStream_t st, bool pdl) {
+    using Sh = FrShape<N>;
     const size_t sm = (size_t)Sh::SLOTS * sizeof(float2);
-    const dim3 grid((batch + Sh::B - 1) / Sh::B, L);
-    cudaError_t e;
-    if (adj) {
-        e = cudaFuncSetAttribute(k_nvmt_rows_fourier_adj_fast<N, 2 * N, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
-        if (e != cudaSuccess) return e;
-        k_nvmt_rows_fourier_adj_fast<N, 2 * N, N><<<grid, Sh::NT, sm, st>>>(ws, Hp, L, batch, stw_w, stw_m, stw_s, cu,
-                                                                           cx, hc);
-    } else {
-        e = cudaFuncSetAttribute(k_nvmt_rows_fourier_fast<N, 2 * N, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
-        if (e != cudaSuccess) return e;
-        k_nvmt_rows_fourier_fast<N, 2 * N, N><<<grid, Sh::NT, sm, st>>>(ws, Hp, L, batch, stw_w, stw_m, stw_s, cu, cx,
-                                                                       hc);
-    }
-    return cudaGetLastError();
+    const auto k = adj ? k_nvmt_rows_fourier_adj_fast<N> : k_nvmt_rows_fourier_fast<N>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = ((unsigned)L * (unsigned)batch + Sh::NR - 1) / Sh::NR;
+    return launch_maybe_pdl(k, dim3(blocks), dim3(Sh::NT), sm, st, pdl, ws, Hp, L, batch, stw_w, stw_m, stw_s, cu, cx,
+                            hc);
 }
 
 cudaError_t launch_nvmt_rows_fourier_fast(bool adjoint, float2* ws, int W, int S, int Hp, int L, const FftLen& fw,
                                           const FftLen& fm, const FftLen& fs, const float2* chirp_u,
-                                          const float2* chirp_x, const float2* hc, int batch, cudaStream_t st) {
+                                          const float2* chirp_x, const float2* hc, int batch, cudaStream_t st,
+                                          bool pdl) {
     if (!fourier_fast_ok(W, fm.N, S) || !fw.stw || !fm.stw || !fs.stw) return cudaErrorNotSupported;
     switch (W) {
-#define X(n) case n: return go_fourier<n>(adjoint, ws, Hp, L, batch, fw.stw, fm.stw, fs.stw, chirp_u, chirp_x, hc, st);
+#define X(n) \
+    case n: return go_fourier<n>(adjoint, ws, Hp, L, batch, fw.stw, fm.stw, fs.stw, chirp_u, chirp_x, hc, st, pdl);
         FR_FAST_LENGTHS(X)
 #undef X
     }

@@ -239,7 +239,7 @@ static cudaError_t nvmt_rows(ft_plan p, float2* ws, int batch, cudaStream_t st) 
         const size_t nu = (size_t)p->L * (p->W + 1), nx = (size_t)p->L * p->S;
         if (fourier_fast(p))
             return launch_nvmt_rows_fourier_fast(false, ws, p->W, p->S, p->Hp, p->L, p->fw, p->fm, p->fx, p->d_chirp,
-                                                 p->d_chirp + nu, p->d_chirp + nu + nx, batch, st);
+                                                 p->d_chirp + nu, p->d_chirp + nu + nx, batch, st, p->pdl);
         return launch_nvmt_rows_fourier(ws, p->W, p->S, p->Hp, p->L, p->fw, p->fm, p->fx, p->d_chirp,
                                         p->d_chirp + nu, p->d_chirp + nu + nx, batch, st);
     }
@@ -257,7 +257,7 @@ static cudaError_t nvmt_rows_adj(ft_plan p, float2* ws, int batch, cudaStream_t 
         const size_t nu = (size_t)p->L * (p->W + 1), nx = (size_t)p->L * p->S;
         if (fourier_fast(p))
             return launch_nvmt_rows_fourier_fast(true, ws, p->W, p->S, p->Hp, p->L, p->fw, p->fm, p->fx, p->d_chirp,
-                                                 p->d_chirp + nu, p->d_chirp + nu + nx, batch, st);
+                                                 p->d_chirp + nu, p->d_chirp + nu + nx, batch, st, p->pdl);
         return launch_nvmt_rows_fourier_adj(ws, p->W, p->S, p->Hp, p->L, p->fw, p->fm, p->fx, p->d_chirp,
                                             p->d_chirp + nu, p->d_chirp + nu + nx, batch, st);
     }
