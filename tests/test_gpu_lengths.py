@@ -61,3 +61,34 @@ def test_wide_length_matches_generic_kernels_and_oracle(torch, N, interp):
         assert _gpu.rel_l2(fast[0][0], oracle.funnel_ref(imgs[0], N, N, interp)) <= 1e-5
         ref = oracle.adjoint_ref(g[0].cpu().numpy().astype(np.float64), H, W, interp)
         assert _gpu.rel_l2(fast[1][0], ref) <= 1e-5
+
+
+FOURIER = [128, 144, 162, 192, 216, 256, 288, 324, 384, 432, 486, 512, 576, 648, 768, 864, 972, 1024, 1152, 1536, 2048]
+
+
+@pytest.mark.parametrize("W", FOURIER)
+def test_fourier_rows_match_generic_kernel(torch, W):
+    """The register-resident chirp-z row kernels (n_slope = W) against the generic
+    ones, forward and adjoint, with a number of rows that leaves the last block
+    partly empty; same bound as between any two FP32 implementations above."""
+    from paper_1904_09409_gb300 import funnel as f
+    H, n = 96, 3
+    rng = np.random.default_rng(W)
+    x = torch.from_numpy(rng.standard_normal((n, H, W)).astype(np.float32)).cuda()
+    g = torch.from_numpy(rng.standard_normal((n, H, W)).astype(np.float32)).cuda()
+    out = []
+    with f.Plan(H, W, W, H, "fourier") as plan:
+        for variant in (0, 1):
+            f.ft_plan_set_variant(plan, variant)
+            m, gi = torch.empty_like(g), torch.empty_like(x)
+            f.ft_forward(plan, x, m)
+            f.ft_backward(plan, g, gi)
+            torch.cuda.synchronize()
+            out.append((m.cpu().numpy().astype(np.float64), gi.cpu().numpy().astype(np.float64)))
+    for a, b in zip(*out):
+        assert np.all(np.isfinite(a))
+        assert _gpu.rel_l2(a, b) <= 2e-6
+    lhs = float(np.sum(out[0][0] * g.cpu().numpy()))
+    rhs = float(np.sum(out[0][1] * x.cpu().numpy()))
+    scale = np.linalg.norm(out[0][0]) * np.linalg.norm(g.cpu().numpy().astype(np.float64))
+    assert abs(lhs - rhs) <= 1e-5 * scale
