@@ -310,16 +310,28 @@ __device__ __forceinline__ bool c2r_block(const float2* __restrict__ in, int nco
     return true;
 }
 
-// row pitch (complex) of the staged spectrum rows: W samples between two zero
-// samples on each side (so a clamped tap index needs no bounds test); W + 4
-// keeps 16-byte alignment for cp.async and shifts successive rows by 8 banks
-__host__ __device__ constexpr int srow_pitch(int W) { return W + 4; }
+// zero samples on each side of a staged spectrum row, so that a clamped tap index
+// needs no bounds test (linear: taps c, c + 1; cubic: c - 1 .. c + 2), and the row
+// pitch (complex): an even number of samples keeps 16-byte alignment for the
+// copies, and successive rows are shifted by 8 or 16 banks
+__host__ __device__ constexpr int srow_pad(int interp) { return interp == FT_INTERP_LINEAR ? 2 : 4; }
+__host__ __device__ constexpr int srow_pitch(int W, int interp) { return W + 2 * srow_pad(interp); }
+
+// Keys' weights (a = -1/2) of the taps floor - 1 .. floor + 2 at fraction fr in
+// [0, 1): keys_w of the four distances as polynomials in fr, without its branches
+__device__ __forceinline__ void keys_weights(float fr, float (&w)[4]) {
+    const float f2 = fr * fr, h = 0.5f * fr;
+    w[0] = fmaf(f2, 1.f - h, -h);                      // -f^3/2 + f^2 - f/2
+    w[1] = fmaf(f2, fmaf(1.5f, fr, -2.5f), 1.f);       // 3 f^3/2 - 5 f^2/2 + 1
+    w[2] = fmaf(f2, fmaf(-1.5f, fr, 2.f), h);          // -3 f^3/2 + 2 f^2 + f/2
+    w[3] = f2 * (h - 0.5f);                            // f^3/2 - f^2/2
+}
 
 // Steps 2-3 in place for rows bx B .. bx B + B - 1 of one image's half spectrum
 // base[L][N] (W columns of image data per row before, N = n_slope values of G
 // after): the NVMT gather with the exact positions x' H' / (2 l), then the
 // exp(+j) transform along x'.  Row 0 becomes zero.  Shared memory: the larger
-// of the FFT's exchange buffer and B staged rows of srow_pitch(W) complex.
+// of the FFT's exchange buffer and B staged rows of srow_pitch(W, INTERP) complex.
 // BULK: each staged row arrives by one bulk copy (the copy engine, not the
 // threads' load/store path) completing on an mbarrier, waited for with the
 // bound `wait` in SM cycles; when a wait runs out, bit 1 of *err is set, the
@@ -335,11 +347,12 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
     constexpr int STEPX = N / R0;                      // x' distance between a thread's elements
     static_assert(R0 % 2 == 0, "half a row is whole elements of the first pass");
     using F = FastFft<N, +1, B, true>;
-    // [B][W + 4] input rows (sample x at 2 + x, 16-byte aligned, two zeros on
+    // [B][WP] input rows (sample x at PAD + x, 16-byte aligned, PAD zeros on
     // each side) in the FFT's own exchange buffer: they are read only by the
     // gather, which ends before the first exchange
     float2* srow = sm;
-    const int WP = srow_pitch(W);
+    constexpr int PAD = srow_pad(INTERP);
+    const int WP = srow_pitch(W, INTERP);
     const int f = threadIdx.x % B;
     const int t = threadIdx.x / B;
     const int l0 = bx * B;
@@ -347,9 +360,9 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
 
     // stage the block's B spectrum rows (W complex each)
     const int chunks = W >> 1;                         // two complex per 16 bytes
-    if (threadIdx.x < 2 * B) {
-        const int r = threadIdx.x >> 1;
-        *reinterpret_cast<float4*>(srow + r * WP + ((threadIdx.x & 1) ? W + 2 : 0)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i < PAD * B; i += fs_T(N) * B) {       // two zeros per 16 bytes
+        const int r = i / PAD, j = 2 * (i % PAD);
+        *reinterpret_cast<float4*>(srow + r * WP + (j < PAD ? j : W + j)) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if constexpr (BULK) {
         __shared__ uint64_t mbar;
@@ -359,11 +372,11 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
             mbar_init(mb, 1);
             mbar_arrive_expect_tx(mb, (uint32_t)(nrows * W * sizeof(float2)));
             for (int r = 0; r < nrows; ++r)
-                bulk_g2s(srow + r * WP + 2, base + (size_t)(l0 + r) * N, (uint32_t)(W * sizeof(float2)), mb);
+                bulk_g2s(srow + r * WP + PAD, base + (size_t)(l0 + r) * N, (uint32_t)(W * sizeof(float2)), mb);
         }
         for (int r = nrows; r < B; ++r)                // rows past the end: zeros
             for (int c = threadIdx.x; c < chunks; c += fs_T(N) * B)
-                *reinterpret_cast<float4*>(srow + r * WP + 2 + 2 * c) = make_float4(0.f, 0.f, 0.f, 0.f);
+                *reinterpret_cast<float4*>(srow + r * WP + PAD + 2 * c) = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();                               // the mbarrier is initialised
         const bool ok = mbar_wait(mb, 0, wait);
         if (__syncthreads_or(!ok)) {
@@ -374,7 +387,7 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
     } else {
 #pragma unroll
         for (int r = 0; r < B; ++r) {
-            float2* dst = srow + r * WP + 2;
+            float2* dst = srow + r * WP + PAD;
             const float2* src = base + (size_t)(l0 + r) * N;
             if (l0 + r < L) {
                 for (int c = threadIdx.x; c < chunks; c += fs_T(N) * B) cp_async16(dst + 2 * c, src + 2 * c);
@@ -391,7 +404,7 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = make_float2(0.f, 0.f);
     if (l >= 1 && l < L) {
-        const float2* myrow = srow + f * WP + 2;
+        const float2* myrow = srow + f * WP + PAD;
         const int den = 2 * l;
         const float inv = 1.f / (float)den;
         const int step = STEPX * Hp;
@@ -419,13 +432,16 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
                     const float2 a0 = ok ? myrow[cc] : zero, a1 = ok ? myrow[cc + 1] : zero;
                     acc = make_float2(fmaf(fr, a1.x - a0.x, a0.x), fmaf(fr, a1.y - a0.y, a0.y));
                 } else {
+                    // taps c0 - 1 .. c0 + 2; outside 0 .. W-1 the padding's zeros
+                    const int cc = min(max(c0, -3), W + 1);
+                    float w[4];
+                    keys_weights(fr, w);
                     acc = zero;
 #pragma unroll
-                    for (int d = -1; d <= 2; ++d) {
-                        const float2 a = (unsigned)(c0 + d) < (unsigned)W ? myrow[c0 + d] : zero;
-                        const float w = keys_w(fr - (float)d);
-                        acc.x = fmaf(w, a.x, acc.x);
-                        acc.y = fmaf(w, a.y, acc.y);
+                    for (int d = 0; d < 4; ++d) {
+                        const float2 a = FT_IN(cc + d + PAD - 1, WP, FT_DBG_NVMT_GATHER) ? myrow[cc + d - 1] : zero;
+                        acc.x = fmaf(w[d], a.x, acc.x);
+                        acc.y = fmaf(w[d], a.y, acc.y);
                     }
                 }
                 v[m * R0 + q] = acc;

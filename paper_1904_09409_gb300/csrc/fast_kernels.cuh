@@ -283,7 +283,14 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
             for (int j = 0; j < ND; ++j) {
                 if (rem[j] > lim && xp[j] >= -N / 2 && xp[j] < N / 2 && FT_IN(xp[j] + N / 2, N, FT_DBG_NVMT_ADJ)) {
                     const float fr = (float)(Hp - 1 - rem[j]) * inv;
-                    const float w = INTERP == FT_INTERP_LINEAR ? (j == 0 ? 1.f - fr : fr) : keys_w(fr - (float)(DLO + j));
+                    float w;
+                    if constexpr (INTERP == FT_INTERP_LINEAR) {
+                        w = j == 0 ? 1.f - fr : fr;
+                    } else {
+                        float k4[4];                   // the one the unrolled j uses is computed
+                        keys_weights(fr, k4);
+                        w = k4[j];
+                    }
                     const float2 g = sm[spos(xp[j] + N / 2) * B + f];
                     acc.x = fmaf(w, g.x, acc.x);
                     acc.y = fmaf(w, g.y, acc.y);
@@ -461,7 +468,7 @@ template <int N, int INTERP>
 static cudaError_t go_rows_i(float2* ws, int W, int Hp, int L, const float2* stw, int batch, cudaStream_t st,
                              bool pdl, unsigned* err, long long wait) {
     constexpr int B = fs_Brow(N);
-    const size_t slots = FastFft<N, +1, B>::SLOTS, rows = (size_t)srow_pitch(W) * B;
+    const size_t slots = FastFft<N, +1, B>::SLOTS, rows = (size_t)srow_pitch(W, INTERP) * B;
     const size_t sm = (slots > rows ? slots : rows) * sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(k_nvmt_rows_fast<N, INTERP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;

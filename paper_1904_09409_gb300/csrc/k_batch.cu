@@ -131,7 +131,7 @@ void batch_tile_shape(int H, int W, int threads, int* rows, int* cols, int* band
 }
 
 // shared memory of the transform stages: the exchange buffer of B = threads / T
-// transforms (and, for the rows, B staged rows of W + 4 samples), the largest
+// transforms (and, for the rows, B staged rows with their padding), the largest
 // over the lengths up to maxlen
 static size_t stage_smem(int stage, int threads, int maxlen) {
     size_t best = 0;
@@ -139,7 +139,8 @@ static size_t stage_smem(int stage, int threads, int maxlen) {
         if (n > maxlen) continue;
         const int B = threads / fs_T(n);
         size_t v = (size_t)fs_slots(n) * B;
-        if (stage == 1 && (size_t)srow_pitch(n) * B > v) v = (size_t)srow_pitch(n) * B;
+        if (stage == 1 && (size_t)srow_pitch(n, FT_INTERP_CUBIC) * B > v)
+            v = (size_t)srow_pitch(n, FT_INTERP_CUBIC) * B;
         if (v * sizeof(float2) > best) best = v * sizeof(float2);
     }
     return best;
