@@ -54,6 +54,7 @@ __device__ __forceinline__ bool ft_in_range(long long i, long long n, unsigned c
 // the flag words of the units with checks (host; the device must be idle)
 unsigned ft_debug_read_fast();
 unsigned ft_debug_read_peak_sparse();
+unsigned ft_debug_read_peak_multi();
 
 // One FFT length N = 2^a 3^b: its radix sequence and twiddle table
 // tw[t] = exp(-2 pi i t / N), t in [0, N), rounded to FP32 from FP64 values.
@@ -259,6 +260,10 @@ __device__ float2* cta_fft(float2* a, float2* b, const FftLen& L, int logB) {
     return a;
 }
 
+// the peak passes: one block per image from tile maxima, per-tile keys, and from
+// tile maxima over the whole GPU
+enum { FT_PASS_SPARSE = 1, FT_PASS_DENSE = 2, FT_PASS_MULTI = 3 };
+
 // -------------------------------------------------------------- plan object
 struct ft_plan_s {
     int H, W, S, Hp, L, interp, top;   // the transform's own sizes (transposed for the inverse space)
@@ -285,7 +290,9 @@ struct ft_plan_s {
     int col_logB_max, row_logB_max;  // the largest that fit the shared-memory budget
     int use_fast_y, use_fast_x;      // fixed-length kernels in use for H' / S
     int variant;            // see ft_plan_set_variant
-    int peak_mode;          // peak pass: 0 = the faster one by the cost model, 1 = from tile maxima, 2 = per-tile keys
+    int peak_mode;          // peak pass: 0 = the fastest by the cost model, else FT_PASS_*
+    void* d_peak_state;     // per-image words of the pass over the whole GPU (zero between calls)
+    size_t peak_state_bytes;
     int num_sms;            // multiprocessors of the plan's device
     int pdl;                // programmatic dependent launch in the forward chain (FT_PDL=0: off)
     int precision;          // ft_precision of step 3 (ft_plan_set_precision)
@@ -375,6 +382,15 @@ bool peak_sparse_fits(int tile_rows, int tile_cols, int top_k);
 cudaError_t launch_peak_sparse(const float* map, const unsigned* tmax, int Hp, int S, int tile_rows, int tile_cols,
                                int batch, int top_k, float threshold, ft_peak* out, int32_t* count, cudaStream_t st,
                                bool pdl = false);
+// The same list again, two launches over the whole GPU (k_peak_multi.cu):
+// scratch of peak_multi_scratch_bytes(tiles per image, batch), and per-image
+// words of peak_multi_state_bytes(batch) that are zero before the first call and
+// that every call leaves so.
+size_t peak_multi_scratch_bytes(int ntiles, int batch);
+size_t peak_multi_state_bytes(int batch);
+cudaError_t launch_peak_multi(const float* map, const unsigned* tmax, int Hp, int S, int tile_rows, int tile_cols,
+                              int batch, int top_k, float threshold, void* scratch, void* state, ft_peak* out,
+                              int32_t* count, cudaStream_t st, bool pdl);
 // tile maxima of given maps (map 8-byte aligned) in tiles of tile_max_shape
 void tile_max_shape(int* tile_rows, int* tile_cols);
 cudaError_t launch_tile_max(const float* map, int Hp, int S, int batch, unsigned* tmax, cudaStream_t st);

@@ -89,21 +89,6 @@ cudaError_t launch_tile_max(const float* map, int Hp, int S, int batch, unsigned
     return cudaGetLastError();
 }
 
-// warps of the peak pass's block: 32, 16 or 8, the most whose shared memory
-// fits the current device (0: none does)
-static int sparse_warps(int rows, int cols, int top_k) {
-    int dev = 0, optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-    if ((rows * cols) % 32 != 0 || (cols & (cols - 1)) != 0) return 0;
-    if (rows * cols > 64 * 32) return 0;                          // a lane's cells fit one 64-bit mask
-    for (int nw = 32; nw >= 8; nw /= 2)
-        if (sparse_smem(rows, cols, top_k, nw, 0) + sizeof(SparseShared) + SP_TM_SMEM * sizeof(unsigned) <=
-            (size_t)optin)
-            return nw;
-    return 0;
-}
-
 bool peak_sparse_fits(int tile_rows, int tile_cols, int top_k) { return sparse_warps(tile_rows, tile_cols, top_k) > 0; }
 
 cudaError_t launch_peak_sparse(const float* map, const unsigned* tmax, int Hp, int S, int tile_rows, int tile_cols,

@@ -45,6 +45,21 @@ static size_t sparse_smem(int rows, int cols, int K, int nw, int ntiles) {
            SP_LIST * sizeof(int) + tms;
 }
 
+// warps of the peak pass's block: 32, 16 or 8, the most whose shared memory
+// fits the current device (0: none does)
+static int sparse_warps(int rows, int cols, int top_k) {
+    int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
+    if ((rows * cols) % 32 != 0 || (cols & (cols - 1)) != 0) return 0;
+    if (rows * cols > 64 * 32) return 0;                          // a lane's cells fit one 64-bit mask
+    for (int nw = 32; nw >= 8; nw /= 2)
+        if (sparse_smem(rows, cols, top_k, nw, 0) + sizeof(SparseShared) + SP_TM_SMEM * sizeof(unsigned) <=
+            (size_t)optin)
+            return nw;
+    return 0;
+}
+
 // One warp's descending sort of 32 values, one per lane (bitonic network over
 // shuffles; blocks of k lanes alternate descending / ascending, the last merge
 // is descending).
@@ -90,84 +105,41 @@ __device__ void block_merge_top(T* mrg, int nl, int warp, int lane) {
 }
 
 
-// One map's pass, run by a whole block of nw = blockDim.x / 32 warps: m is the
-// map [Hp][S], tmax its tile maxima [nty][ntx] (tiles of TH x 2^logTW cells),
-// out / count its K records and its count; spsm is sparse_smem(...) bytes of
-// shared memory, sh the block's shared bookkeeping.
-__device__ __forceinline__ void peak_sparse_block(const float* __restrict__ m, const unsigned* __restrict__ tmax,
-                                                  int Hp, int S, int TH, int logTW, int nty, int ntx, int K,
-                                                  float thr, ft_peak* __restrict__ out, int32_t* __restrict__ count,
-                                                  unsigned char* spsm, SparseShared& sh) {
-    const int TW = 1 << logTW;
-    const int cells = TH * TW;
-    const int nw = blockDim.x >> 5;                    // warps = tiles per batch
-    const int capc = K + nw * (cells / 4);
-    const int P = TW + 8;                              // staged row: columns s0 - 4 .. s0 + TW + 3
-    const size_t stage_bytes = ((size_t)nw * (TH + 2) * P * sizeof(float) + 15) & ~(size_t)15;
-    float* stg0 = reinterpret_cast<float*>(spsm);
-    u64* cand = reinterpret_cast<u64*>(spsm + stage_bytes);
-    u64* keep = cand + capc;
-    u64* mrg = keep + next_pow2(K);                    // [nw][32]
-    int* list = reinterpret_cast<int*>(mrg + nw * 32);
-    const int ntiles = nty * ntx;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* stg = stg0 + (size_t)warp * (TH + 2) * P;
-    const unsigned* tm = tmax;
+// One warp's test of one tile of a map [Hp][S] with tiles of TH x 2^logTW cells
+// ([nty][ntx] of them, the last ones ragged), staged with its one-cell halo
+// (wrapped) in the warp's area stg of (TH + 2) x (2^logTW + 8) floats.
+struct TileTester {
+    const float* m;
+    int Hp, S, TH, TW, ntx, P, lane;
+    float* stg;
     // interior tiles are staged as float4 rows: TW / 4 + 2 vectors per row
-    const int V = (TW >> 2) + 2;
-    const bool vec = (TW & 3) == 0 && V <= 32 && (S & 3) == 0 && (reinterpret_cast<size_t>(m) & 15) == 0;
-    auto valid = [&](unsigned b) { return __uint_as_float(b) >= thr; };
-
-    if (threadIdx.x == 0) {
-        sh.ncand = 0;
-        sh.nlist = 0;
-        sh.bound = thr;
-    }
-    // the tile maxima, copied once when they fit (all loads in flight); then T,
-    // the nw-th largest valid maximum (+1 so that 0 means none): every warp
-    // sorts chunks of 32 maxima with shuffles and keeps the best 32, and a
-    // merge tree over the warps leaves the best 32 of the image
-    {
-        unsigned* tms = reinterpret_cast<unsigned*>(list + SP_LIST);
-        if (ntiles <= SP_TM_SMEM) {
-            for (int i = threadIdx.x; i < ntiles; i += blockDim.x) tms[i] = tm[i];
-            tm = tms;
-        }
-        __syncthreads();
-        unsigned* m32 = reinterpret_cast<unsigned*>(mrg);
-        unsigned run = 0u;
-        for (int c0 = warp; c0 * 32 < ntiles; c0 += 4 * nw) {
-            unsigned v[4];                             // four independent sorts in flight
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = (c0 + u * nw) * 32 + lane;
-                const unsigned b = i < ntiles ? tm[i] : 0u;
-                v[u] = warp_sort_desc((i < ntiles && valid(b)) ? b + 1u : 0u, lane);   // b + 1 fits: b >= 0
-            }
-            const unsigned a = warp_merge_top(warp_merge_top(v[0], v[1], lane), warp_merge_top(v[2], v[3], lane), lane);
-            run = c0 == warp ? a : warp_merge_top(run, a, lane);
-        }
-        m32[warp * 32 + lane] = run;
-        block_merge_top(m32, nw, warp, lane);
-        const unsigned T = m32[nw - 1];
-        if (threadIdx.x == 0) sh.tbits = T == 0u ? 0u : T - 1u;    // fewer than nw: every valid tile
-        __syncthreads();
-    }
-
+    int V;
+    bool vec;
     // test layout: lanes as rpp row groups of cw columns, cpl columns and rh
     // rows per lane; bit k rh + i of a lane's mask is row g rh + i of column
     // cl + cw k of the tile (rh cpl = cells / 32 <= 64)
-    const int cw = min(TW, 32), rpp = 32 / cw, cl = lane & (cw - 1);
-    const int rh = TH / rpp, g = lane / cw, cpl = TW / cw;
+    int cw, cl, rh, g, cpl;
 
-    // warp: the strict local maxima of tile `tile` with |P| >= bound, as the
-    // lanes' masks; returns the warp's largest marked value (bits + 1, 0: none).
-    // The tile and its halo (wrapped) are first copied to the warp's staging
-    // area: interior tiles as aligned 16-byte rows by cp.async (columns
+    __device__ __forceinline__ TileTester(const float* map, int hp, int s, int th, int logTW, int ntx_, float* stage,
+                                          int lane_)
+        : m(map), Hp(hp), S(s), TH(th), TW(1 << logTW), ntx(ntx_), P((1 << logTW) + 8), lane(lane_), stg(stage) {
+        V = (TW >> 2) + 2;
+        vec = (TW & 3) == 0 && V <= 32 && (S & 3) == 0 && (reinterpret_cast<size_t>(m) & 15) == 0;
+        cw = min(TW, 32);
+        const int rpp = 32 / cw;
+        cl = lane & (cw - 1);
+        rh = TH / rpp;
+        g = lane / cw;
+        cpl = TW / cw;
+    }
+
+    // The strict local maxima of tile `tile` with |P| >= bound, as the lanes'
+    // masks; returns the warp's largest marked value (bits + 1, 0: none).
+    // Interior tiles are copied as aligned 16-byte rows by cp.async (columns
     // s0 - 4 .. s0 + TW + 3, all copies of a lane in flight at once), tiles at
     // the left or right edge cell by cell (columns s0 - 1 .. s0 + tw, wrapped);
     // every read of the staged cells takes |P|.
-    auto test_tile = [&](int tile, float bound, unsigned long long& mask) -> unsigned {
+    __device__ __forceinline__ unsigned test(int tile, float bound, unsigned long long& mask) const {
         const int ty = tile / ntx, tx = tile - ty * ntx;
         const int t0 = ty * TH, s0 = tx * TW;
         const int th = min(TH, Hp - t0), tw = min(TW, S - s0);      // ragged last tiles
@@ -260,12 +232,14 @@ __device__ __forceinline__ void peak_sparse_block(const float* __restrict__ m, c
             }
         }
         return __reduce_max_sync(0xffffffffu, best);
-    };
+    }
 
-    // warp, after test_tile on the same tile: the marked cells with |P| >= cut
-    // are appended to cand[] (one atomic for the warp).  The staging area is
-    // reused by the warp's next tile.
-    auto append_tile = [&](int tile, float cut, unsigned long long mask) {
+    // After test() on the same tile: the marked cells with |P| >= cut are appended
+    // to cand[0 .. cap), *ncand counting them (one atomic for the warp; keys past
+    // cap are counted and dropped).  The staging area is reused by the warp's next
+    // tile.
+    __device__ __forceinline__ void append(int tile, float cut, unsigned long long mask, u64* cand, int* ncand,
+                                           int cap) const {
         const int ty = tile / ntx, tx = tile - ty * ntx;
         const int t0 = ty * TH, s0 = tx * TW;
         unsigned long long keepm = 0ull;
@@ -282,17 +256,82 @@ __device__ __forceinline__ void peak_sparse_block(const float* __restrict__ m, c
                 if (lane >= o) incl += y;
             }
             int base = 0;
-            if (lane == 31 && incl) base = atomicAdd(&sh.ncand, incl);
+            if (lane == 31 && incl) base = atomicAdd(ncand, incl);
             base = __shfl_sync(0xffffffffu, base, 31) + incl - cnt;
             for (unsigned long long mk = keepm; mk; mk &= mk - 1ull) {
                 const int bit = __ffsll((long long)mk) - 1, k = bit / rh, i = bit - k * rh;
                 const int c = cl + cw * k;
                 const unsigned lin = (unsigned)(t0 + g * rh + i) * (unsigned)S + (unsigned)(s0 + c);
-                cand[base++] = peak_key(fabsf(stg[(g * rh + i + 1) * P + c + 4]), lin);
+                if (base < cap) cand[base] = peak_key(fabsf(stg[(g * rh + i + 1) * P + c + 4]), lin);
+                ++base;
             }
         }
         __syncwarp();
-    };
+    }
+};
+
+// One map's pass, run by a whole block of nw = blockDim.x / 32 warps: m is the
+// map [Hp][S], tmax its tile maxima [nty][ntx] (tiles of TH x 2^logTW cells),
+// out / count its K records and its count; spsm is sparse_smem(...) bytes of
+// shared memory, sh the block's shared bookkeeping.
+__device__ __forceinline__ void peak_sparse_block(const float* __restrict__ m, const unsigned* __restrict__ tmax,
+                                                  int Hp, int S, int TH, int logTW, int nty, int ntx, int K,
+                                                  float thr, ft_peak* __restrict__ out, int32_t* __restrict__ count,
+                                                  unsigned char* spsm, SparseShared& sh) {
+    const int TW = 1 << logTW;
+    const int cells = TH * TW;
+    const int nw = blockDim.x >> 5;                    // warps = tiles per batch
+    const int capc = K + nw * (cells / 4);
+    const int P = TW + 8;                              // staged row: columns s0 - 4 .. s0 + TW + 3
+    const size_t stage_bytes = ((size_t)nw * (TH + 2) * P * sizeof(float) + 15) & ~(size_t)15;
+    float* stg0 = reinterpret_cast<float*>(spsm);
+    u64* cand = reinterpret_cast<u64*>(spsm + stage_bytes);
+    u64* keep = cand + capc;
+    u64* mrg = keep + next_pow2(K);                    // [nw][32]
+    int* list = reinterpret_cast<int*>(mrg + nw * 32);
+    const int ntiles = nty * ntx;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* stg = stg0 + (size_t)warp * (TH + 2) * P;
+    const unsigned* tm = tmax;
+    auto valid = [&](unsigned b) { return __uint_as_float(b) >= thr; };
+
+    if (threadIdx.x == 0) {
+        sh.ncand = 0;
+        sh.nlist = 0;
+        sh.bound = thr;
+    }
+    // the tile maxima, copied once when they fit (all loads in flight); then T,
+    // the nw-th largest valid maximum (+1 so that 0 means none): every warp
+    // sorts chunks of 32 maxima with shuffles and keeps the best 32, and a
+    // merge tree over the warps leaves the best 32 of the image
+    {
+        unsigned* tms = reinterpret_cast<unsigned*>(list + SP_LIST);
+        if (ntiles <= SP_TM_SMEM) {
+            for (int i = threadIdx.x; i < ntiles; i += blockDim.x) tms[i] = tm[i];
+            tm = tms;
+        }
+        __syncthreads();
+        unsigned* m32 = reinterpret_cast<unsigned*>(mrg);
+        unsigned run = 0u;
+        for (int c0 = warp; c0 * 32 < ntiles; c0 += 4 * nw) {
+            unsigned v[4];                             // four independent sorts in flight
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = (c0 + u * nw) * 32 + lane;
+                const unsigned b = i < ntiles ? tm[i] : 0u;
+                v[u] = warp_sort_desc((i < ntiles && valid(b)) ? b + 1u : 0u, lane);   // b + 1 fits: b >= 0
+            }
+            const unsigned a = warp_merge_top(warp_merge_top(v[0], v[1], lane), warp_merge_top(v[2], v[3], lane), lane);
+            run = c0 == warp ? a : warp_merge_top(run, a, lane);
+        }
+        m32[warp * 32 + lane] = run;
+        block_merge_top(m32, nw, warp, lane);
+        const unsigned T = m32[nw - 1];
+        if (threadIdx.x == 0) sh.tbits = T == 0u ? 0u : T - 1u;    // fewer than nw: every valid tile
+        __syncthreads();
+    }
+
+    const TileTester tester(m, Hp, S, TH, logTW, ntx, stg, lane);
 
     // whole block: exactly the best K candidates stay, the bound becomes value(kth)
     auto compact = [&]() {
@@ -358,7 +397,7 @@ __device__ __forceinline__ void peak_sparse_block(const float* __restrict__ m, c
             unsigned best = 0u;
             if (j < nl && __uint_as_float(tm[list[j]]) >= bound) {
                 tile = list[j];
-                best = test_tile(tile, bound, mask);
+                best = tester.test(tile, bound, mask);
             }
             // the K-th largest of the warps' best values (distinct candidates of
             // distinct tiles) is a lower bound of value(kth): only the marked
@@ -376,7 +415,7 @@ __device__ __forceinline__ void peak_sparse_block(const float* __restrict__ m, c
                 }
                 if (lk != 0u) cut = fmaxf(cut, __uint_as_float(lk - 1u));
             }
-            if (tile >= 0) append_tile(tile, cut, mask);
+            if (tile >= 0) tester.append(tile, cut, mask, cand, &sh.ncand, capc);
             __syncthreads();
             if (K <= 32)
                 keep_best();

@@ -195,6 +195,20 @@ static ft_status ensure(ft_plan p, void** ptr, size_t* have, size_t need, const 
     return FT_OK;
 }
 
+// ensure() for counters that kernels expect zero and leave zero: a new buffer is
+// cleared on the stream
+static ft_status zeroed(ft_plan p, void** ptr, size_t* have, size_t need, cudaStream_t st, const char* what) {
+    if (need <= *have && *ptr) return FT_OK;
+    const ft_status s = ensure(p, ptr, have, need, what);
+    if (s != FT_OK) return s;
+    const cudaError_t e = cudaMemsetAsync(*ptr, 0, need, st);
+    if (e == cudaSuccess) return FT_OK;
+    cudaFree(*ptr);
+    *ptr = nullptr;
+    *have = 0;
+    return cuda_fail(e, what);
+}
+
 static size_t spec_bytes(ft_plan p, int batch) { return (size_t)batch * p->L * p->S * sizeof(float2); }
 static size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 // workspace: [half spectra][transposed image (inverse space only)][aux: peak keys or loss partials]
@@ -293,7 +307,7 @@ ft_status ft_debug_flags(uint32_t* flags) {
     if (!flags) return FT_ERR_INVALID_ARG;
     *flags = 0;
     FT_CUDA(cudaDeviceSynchronize(), "ft_debug_flags");
-    *flags = ft_debug_read_fast() | ft_debug_read_peak_sparse();
+    *flags = ft_debug_read_fast() | ft_debug_read_peak_sparse() | ft_debug_read_peak_multi();
     return FT_OK;
 }
 
@@ -416,7 +430,10 @@ ft_status ft_plan_create_space(ft_plan* out, int img_H, int img_W, int n_slope, 
     const char* pdl = getenv("FT_PDL");
     p->pdl = !(pdl && !strcmp(pdl, "0"));
     const char* pm = getenv("FT_PEAKS");
-    p->peak_mode = pm && !strcmp(pm, "sparse") ? 1 : (pm && !strcmp(pm, "dense") ? 2 : 0);
+    p->peak_mode = !pm ? 0
+                 : !strcmp(pm, "sparse") ? FT_PASS_SPARSE
+                 : !strcmp(pm, "dense") ? FT_PASS_DENSE
+                 : !strcmp(pm, "multi") ? FT_PASS_MULTI : 0;
     if (cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess || p->num_sms < 1)
         p->num_sms = 1;
     *out = p;
@@ -433,6 +450,7 @@ ft_status ft_plan_destroy(ft_plan p) {
     if (p->d_tw) cudaFree(p->d_tw);
     if (p->d_chirp) cudaFree(p->d_chirp);
     if (p->d_tc_err) cudaFree(p->d_tc_err);
+    if (p->d_peak_state) cudaFree(p->d_peak_state);
     if (p->d_img_host) cudaFree(p->d_img_host);
     if (p->d_map_host) cudaFree(p->d_map_host);
     if (p->d_peaks_host) cudaFree(p->d_peaks_host);
@@ -585,44 +603,54 @@ int ft_peaks_launches(ft_plan p, int batch) {
 // split precision: the length-4096 column transforms on the tensor cores too
 static bool tc_columns(ft_plan p);
 
-// The tile shape of ft_detect's peak pass (the tiles whose maxima step 4
-// writes), or false when ft_detect runs ft_forward and ft_peaks instead: step 4
-// must be the fixed-length FP32 kernel on the caller's stream, and the pass's
-// shared memory must fit.
-// Whether the pass from tile maxima beats the per-tile key kernels for this
-// call.  It runs one block per image, so it costs one image's serial chain per
-// wave of images: selecting among the tiles, then batches of 32 tiles (one at
-// 1024^2 and 2048^2 with top_k = 32, over 20 at 4096^2 with top_k = 100: the
-// batch count grows like (tiles x top_k)^2), plus, for ft_peaks, one streaming
-// read for the tile maxima.  The key kernels spread every cell over the whole GPU
-// but have a fixed latency of two dependent kernels, the second also one block
-// per image.  Constants in microseconds, fitted to GB300 measurements of
-// ft_detect both ways (1024^2 with 1-128 images, 512^2, 2048^2 and 4096^2; the
-// model picks the faster pass in all 15 cases).  The pass from tile maxima
-// occupies only one multiprocessor per image, so plans whose calls share the GPU
-// with others (ft_batch) always take it.  FT_PEAKS=sparse / dense at plan
-// creation fixes the choice.
-static bool sparse_is_faster(ft_plan p, int batch, int top_k, bool with_tile_max) {
-    if (p->peak_mode) return p->peak_mode == 1;
+// The peak pass that this call is expected to be fastest with.  The pass from tile
+// maxima runs one block per image, so it costs one image's serial chain per wave of
+// images: selecting among the tiles, then batches of 32 tiles (one at 1024^2 and
+// 2048^2 with top_k = 32, over 20 at 4096^2 with top_k = 100: the batch count grows
+// like (tiles x top_k)^2), for top_k > 32 a radix selection per batch, and for
+// ft_peaks one streaming read for the tile maxima.  The key kernels spread every
+// cell over the whole GPU but have a fixed latency of two dependent kernels, the
+// second one block per image over the keys of all tiles.  The pass over the whole
+// GPU has the latency of two kernels, tests a number of tiles that grows with top_k
+// and selects among few candidates; it needs clearly more tiles than peaks (else
+// its bound is the threshold).  Constants in microseconds, fitted to GB300
+// measurements of ft_detect with each pass (256^2 to 4096^2, 1 to 128 images,
+// top_k 1 to 1024; us, one block per image / keys / whole GPU): 1024^2 x 64, K 32
+// 33 / 128 / 64; 2048^2 x 1, K 8 33 / 33 / 23; 2048^2 x 4, K 32 35 / 73 / 31;
+// 2048^2 x 16, K 32 37 / 137 / 55; 2048^2 x 8, K 100 73 / 96 / 45; 4096^2 x 4, K 8
+// 104 / 129 / 44; 4096^2 x 4, K 100 160 / 140 / 62; 1024^2 x 16, K 300 223 / 105 /
+// 64; 512^2 x 16, K 1000 320 / 71 / 113.  The pass from tile maxima occupies only one
+// multiprocessor per image, so plans whose calls share the GPU with others
+// (ft_batch) always take it, as does the pipeline of ft_detect_batches, which hides
+// it.  FT_PEAKS=sparse / dense / multi at plan creation fixes the choice.
+static int peak_pass(ft_plan p, int batch, int top_k, bool with_tile_max, bool multi_ok) {
+    if (p->peak_mode) return p->peak_mode == FT_PASS_MULTI && !multi_ok ? FT_PASS_SPARSE : p->peak_mode;
     const double cells = (double)p->Hp * p->S, tiles = cells / 256.0;
     const int waves = (batch + p->num_sms - 1) / p->num_sms;
     const double x = tiles * top_k / 1.5e6;
-    const double sparse = waves * (1.2e-3 * tiles + 12.0 * (1.0 + x * x)) + (with_tile_max ? 0.7e-6 * cells * batch : 0.0);
-    const double dense = 1.6e-6 * cells * batch + 27.0;
-    return sparse < dense;
+    const double sparse = waves * (1.2e-3 * tiles + 12.0 * (1.0 + x * x) + (top_k > 32 ? 0.25 * top_k : 0.0)) +
+                          (with_tile_max ? 0.7e-6 * cells * batch : 0.0);
+    const double dense = 1.6e-6 * cells * batch + 0.7e-7 * cells * top_k + 27.0;
+    const double multi = top_k <= tiles / 16 ? 19.0 + 0.1 * top_k + 1.0e-4 * tiles * batch * (1.0 + top_k / 200.0) : 1e30;
+    if (multi_ok && multi < sparse && multi < dense) return FT_PASS_MULTI;
+    return sparse < dense ? FT_PASS_SPARSE : FT_PASS_DENSE;
 }
 
-static bool sparse_peaks(ft_plan p, int batch, int top_k, int* rows, int* cols, int* bands) {
-    if (!p->use_fast_y || tc_columns(p) || use_lanes(p, batch)) return false;
-    if (!c2r_tile_shape(p->Hp, rows, cols, bands)) return false;
-    return peak_sparse_fits(*rows, *cols, top_k) && sparse_is_faster(p, batch, top_k, false);
+// The pass ft_detect runs on the tile maxima that step 4 writes (FT_PASS_SPARSE or
+// FT_PASS_MULTI, the tiles' shape in *rows, *cols, *bands), or 0 when it runs
+// ft_forward and ft_peaks instead.  multi_ok: FT_PASS_MULTI may be chosen.
+static int detect_pass(ft_plan p, int batch, int top_k, bool multi_ok, int* rows, int* cols, int* bands) {
+    if (!p->use_fast_y || tc_columns(p) || use_lanes(p, batch)) return 0;
+    if (!c2r_tile_shape(p->Hp, rows, cols, bands) || !peak_sparse_fits(*rows, *cols, top_k)) return 0;
+    const int pass = peak_pass(p, batch, top_k, false, multi_ok);
+    return pass == FT_PASS_DENSE ? 0 : pass;
 }
 
 // ft_peaks takes the pass from tile maxima (tiles of tile_max_shape)
 static bool peaks_use_tile_max(ft_plan p, int batch, int top_k) {
     int tr, tc;
     tile_max_shape(&tr, &tc);
-    return peak_sparse_fits(tr, tc, top_k) && sparse_is_faster(p, batch, top_k, true);
+    return peak_sparse_fits(tr, tc, top_k) && peak_pass(p, batch, top_k, true, false) == FT_PASS_SPARSE;
 }
 
 // scratch of ft_peaks: tile maxima, or the per-tile keys where the pass from
@@ -636,17 +664,24 @@ static size_t peaks_scratch_bytes(ft_plan p, int batch, int top_k) {
     return peaks_use_tile_max(p, batch, top_k) ? tile_max_bytes(p, batch) : peaks_key_bytes(p->Hp, p->S, batch, top_k);
 }
 
-// bytes of ft_detect's tile maxima for this batch (0 when it runs ft_peaks)
-static size_t tmax_bytes(ft_plan p, int batch, int top_k) {
+// bytes of ft_detect's tile maxima for this batch, and with the scratch of the pass
+// over the whole GPU (0 when it runs ft_peaks)
+static size_t tmax_bytes(ft_plan p, int batch, int bands, int cols) {
+    return al256((size_t)batch * bands * ((p->S + cols - 1) / cols) * sizeof(unsigned));
+}
+static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_ok) {
     int rows, cols, bands;
-    if (!sparse_peaks(p, batch, top_k, &rows, &cols, &bands)) return 0;
-    return (size_t)batch * bands * ((p->S + cols - 1) / cols) * sizeof(unsigned);
+    const int pass = detect_pass(p, batch, top_k, multi_ok, &rows, &cols, &bands);
+    if (!pass) return 0;
+    return tmax_bytes(p, batch, bands, cols) +
+           (pass == FT_PASS_MULTI ? peak_multi_scratch_bytes(bands * ((p->S + cols - 1) / cols), batch) : 0);
 }
 
 int ft_detect_launches(ft_plan p, int batch, int top_k) {
     if (!p || batch <= 0 || top_k < 1 || top_k > FT_MAX_TOPK) return 0;
     int rows, cols, bands;
-    if (sparse_peaks(p, batch, top_k, &rows, &cols, &bands)) return (p->space == FT_SPACE_INVERSE ? 1 : 0) + 4;
+    const int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
+    if (pass) return (p->space == FT_SPACE_INVERSE ? 1 : 0) + (pass == FT_PASS_MULTI ? 5 : 4);
     return ft_forward_launches(p, batch) + ft_peaks_launches(p, batch);
 }
 
@@ -844,14 +879,20 @@ ft_status ft_detect(ft_plan p, const float* d_img, float* d_map, int batch, int 
     if (!d_img || !d_map || !d_out || !d_count || ((uintptr_t)d_img & 7) || ((uintptr_t)d_map & 7))
         return FT_ERR_INVALID_ARG;
     int rows, cols, bands;
-    if (!sparse_peaks(p, batch, top_k, &rows, &cols, &bands)) {
+    const int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
+    if (!pass) {
         const ft_status s = ft_forward(p, d_img, d_map, batch, stream);
         return s != FT_OK ? s : ft_peaks(p, d_map, batch, top_k, threshold, d_out, d_count, stream);
     }
     // the tile maxima [batch][bands][column blocks] live in the aux region
     const size_t off = aux_off(p, batch);
-    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + tmax_bytes(p, batch, top_k), "cudaMalloc(workspace)");
+    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + detect_scratch_bytes(p, batch, top_k, true),
+                         "cudaMalloc(workspace)");
     if (s != FT_OK) return s;
+    if (pass == FT_PASS_MULTI &&
+        (s = zeroed(p, &p->d_peak_state, &p->peak_state_bytes, peak_multi_state_bytes(batch), (cudaStream_t)stream,
+                    "cudaMalloc(peak state)")) != FT_OK)
+        return s;
     cudaStream_t st = (cudaStream_t)stream;
     float2* ws = (float2*)p->d_ws;
     unsigned* tmax = (unsigned*)((char*)p->d_ws + off);
@@ -862,6 +903,14 @@ ft_status ft_detect(ft_plan p, const float* d_img, float* d_map, int batch, int 
         src = tp;
     }
     if ((s = forward_part(p, src, d_map, ws, nullptr, batch, st, tmax)) != FT_OK) return s;
+    if (pass == FT_PASS_MULTI) {
+        FT_LAUNCH(p, FT_KERNEL_PEAK_SPARSE, st,
+                  launch_peak_multi(d_map, tmax, p->Hp, p->S, rows, cols, batch, top_k, threshold,
+                                    (char*)tmax + tmax_bytes(p, batch, bands, cols), p->d_peak_state, d_out, d_count,
+                                    st, p->pdl),
+                  "peak detection (tile maxima, whole GPU)");
+        return FT_OK;
+    }
     FT_LAUNCH(p, FT_KERNEL_PEAK_SPARSE, st,
               launch_peak_sparse(d_map, tmax, p->Hp, p->S, rows, cols, batch, top_k, threshold, d_out, d_count, st,
                                  p->pdl),
@@ -882,7 +931,7 @@ ft_status ft_detect_batches(ft_plan p, const float* const* d_imgs, int nb, int b
     // the pipeline needs step 1 on the fixed-length kernel right after the peak
     // pass from tile maxima; otherwise one ft_detect per batch
     const bool pipe = p->pdl && p->use_fast_y && !tc_columns(p) && p->space != FT_SPACE_INVERSE &&
-                      sparse_peaks(p, batch, top_k, &rows, &cols, &bands);
+                      detect_pass(p, batch, top_k, false, &rows, &cols, &bands) == FT_PASS_SPARSE;
     if (!pipe) {
         for (int j = 0; j < nb; ++j) {
             const ft_status s = ft_detect(p, d_imgs[j], d_map, batch, top_k, threshold, d_out + j * recs,
@@ -892,7 +941,8 @@ ft_status ft_detect_batches(ft_plan p, const float* const* d_imgs, int nb, int b
         return FT_OK;
     }
     const size_t off = aux_off(p, batch);
-    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + tmax_bytes(p, batch, top_k), "cudaMalloc(workspace)");
+    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + detect_scratch_bytes(p, batch, top_k, false),
+                         "cudaMalloc(workspace)");
     if (s != FT_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     float2* ws = (float2*)p->d_ws;
@@ -1035,10 +1085,13 @@ ft_status ft_detect_host(ft_plan p, const float* h_img, int batch, int top_k, fl
     // size the workspace for one chunk before any copy is in flight (the larger
     // of the two peak passes' scratch: tile maxima or per-tile keys)
     // (a smaller last chunk may take the other peak pass: room for every kind)
-    size_t peak_b = tmax_bytes(p, chunk, top_k);
-    if (tile_max_bytes(p, chunk) > peak_b) peak_b = tile_max_bytes(p, chunk);
-    if (peaks_key_bytes(p->Hp, p->S, chunk, top_k) > peak_b) peak_b = peaks_key_bytes(p->Hp, p->S, chunk, top_k);
-    const size_t need = aux_off(p, chunk) + peak_b;
+    size_t need = 0;
+    for (int nb : {chunk, batch - (nchunks - 1) * chunk}) {
+        size_t peak_b = detect_scratch_bytes(p, nb, top_k, true);
+        if (tile_max_bytes(p, nb) > peak_b) peak_b = tile_max_bytes(p, nb);
+        if (peaks_key_bytes(p->Hp, p->S, nb, top_k) > peak_b) peak_b = peaks_key_bytes(p->Hp, p->S, nb, top_k);
+        if (aux_off(p, nb) + peak_b > need) need = aux_off(p, nb) + peak_b;
+    }
     if ((s = ensure(p, &p->d_ws, &p->ws_bytes, need, "cudaMalloc(workspace)")) != FT_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     FT_CUDA(cudaEventRecord(p->start_event, st), "event");
