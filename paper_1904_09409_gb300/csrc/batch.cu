@@ -46,7 +46,11 @@ struct Group {
 };
 
 // threads-per-block options of the grouped kernels, per stage (step 1, steps
-// 2-3, step 4); the defaults are the per-plan kernels' shapes at length 1024
+// 2-3, step 4); the defaults are the per-plan kernels' shapes.  Step 4 runs 256
+// threads below length 1024 and 512 from there on, where 256 threads hold 4 column
+// pairs or fewer: setup_grouped takes 512 when the images of at least 1024 rows hold
+// more than half of the pixels (96 images of all sizes 483 us with 256, 459 with 512;
+// 64 images up to 768 80 and 86)
 const int kThreadOpts[3][2] = {{256, 512}, {128, 256}, {256, 512}};
 const int kDefaultThreads[3] = {512, 128, 256};
 
@@ -383,6 +387,12 @@ static ft_status setup_grouped(ft_batch_s* b) {
     }
     b->ng = (int)b->himgs.size();
     if (b->ng == 0) return FT_OK;
+    long long tall = 0, all = 0;
+    for (const BatchImg& d : b->himgs) {
+        all += (long long)d.H * d.W;
+        if (d.H >= 1024) tall += (long long)d.H * d.W;
+    }
+    if (2 * tall > all) b->threads[2] = 512;
     // steps 2-3 walk the images backwards: their first blocks read the half
     // spectra step 1 wrote last, still in L2, and step 4 starts on the rows
     // written last (every item holds the same number of samples, so the order
