@@ -77,7 +77,9 @@ k_col_c2r_fast(const float2* __restrict__ in, int ncols, int in_pitch, size_t in
 // gradient of k_loss.cu), while every thread adds r^2 of its samples (FP32,
 // compensated) and the block writes one partial of the image's loss.  Each map
 // cell is loaded by exactly one thread, so the partials of an image's blocks
-// add up to its sum of r^2 (within a block by a fixed shuffle tree).  With
+// add up to its sum of r^2 (within a block by a fixed shuffle tree); the next
+// kernel adds them (LossSum: a launch of its own took 6 us, and counting the blocks
+// so that the last one adds them 15 us of 166 per 64 x 1024^2, the fence's wait).  With
 // tma_nb > 0 the map columns arrive by tensor copies into the exchange buffer
 // (pmap, waited for with the bound `wait`; bit 3 of *err when it runs out, and
 // the block returns without writing), their values go to registers, and the
@@ -106,6 +108,9 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
     __shared__ uint64_t mbar;
     const uint32_t mb = smem_u32(&mbar);
     float2 v[E];
+    pdl_trigger();
+    pdl_wait();
+    float* part = partial + (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     if (tma_nb > 0) {
         // the block's map columns by tensor copies into the exchange buffer, their
         // values to registers, then the target columns into the same buffer
@@ -132,6 +137,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
         if (__syncthreads_or(!ok)) {
             if (threadIdx.x == 0 && err) atomicOr(err, 8u);
             mbar_wait(mb, 0);                          // the copies in flight land first
+            if (threadIdx.x == 0) *part = __int_as_float(0x7fc00000);   // NaN: the loss is incomplete
             return;
         }
 #pragma unroll
@@ -151,6 +157,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
         if (__syncthreads_or(!ok)) {
             if (threadIdx.x == 0 && err) atomicOr(err, 8u);
             mbar_wait(mb, 1);
+            if (threadIdx.x == 0) *part = __int_as_float(0x7fc00000);
             return;
         }
     }
@@ -197,7 +204,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
         float x = lane < NW ? red[lane] : 0.f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) partial[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = x;
+        if (lane == 0) *part = x;
     }
     r2c_finish<N, fs_Bcol(N)>(v, sm, t, f, stw, colok, out + (size_t)blockIdx.y * out_img + c, out_pitch, end_scale,
                               mid_scale);
@@ -221,7 +228,10 @@ k_nvmt_rows_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __
 
 template <int N, int INTERP>
 __global__ void __launch_bounds__(fs_T(N) * fs_Brow(N), fs_minblocks(N, fs_T(N) * fs_Brow(N)))
-k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __restrict__ stw) {
+k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __restrict__ stw, LossSum ls) {
+    pdl_trigger();
+    pdl_wait();
+    if (ls.loss && blockIdx.x == gridDim.x - 1) loss_sum_block(ls, blockIdx.y);
     constexpr int B = fs_Brow(N), E = fs_E(N), T = N / E;
     constexpr int R0 = fs_radix(N, 0), G0 = E / R0;
     constexpr int RL = fs_radix(N, fs_nst(N) - 1), GL = E / RL;
@@ -394,7 +404,7 @@ cudaError_t go_r2c(const float* in, int rows_in, int ncols, int in_pitch, size_t
 template <int N>
 cudaError_t go_r2c_loss(const float* map, const float* target, int ncols, const float2* stw, float2* out,
                                int out_pitch, size_t out_img, float es, float ms, float scale, float gscale,
-                               float* partial, int batch, cudaStream_t st, unsigned* err, long long wait) {
+                               float* partial, int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait) {
     constexpr int B = fs_Bcol(N);
     const size_t sm = (size_t)FastFft<N, -1, B>::SLOTS * sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(k_col_r2c_loss_fast<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -409,9 +419,8 @@ cudaError_t go_r2c_loss(const float* map, const float* target, int ncols, const 
         nb = 0;
     dim3 grid((ncols + 2 * B - 1) / (2 * B), batch);
     const int pf = prefetch_distance(k_col_r2c_loss_fast<N>, fs_T(N) * B, sm);
-    k_col_r2c_loss_fast<N><<<grid, fs_T(N) * B, sm, st>>>(map, target, ncols, cells, stw, out, out_pitch, out_img, es,
-                                                          ms, scale, gscale, partial, pm, tm, h, nb, err, wait, pf);
-    return cudaGetLastError();
+    return launch_maybe_pdl(k_col_r2c_loss_fast<N>, grid, dim3(fs_T(N) * B), sm, st, pdl, map, target, ncols, cells,
+                            stw, out, out_pitch, out_img, es, ms, scale, gscale, partial, pm, tm, h, nb, err, wait, pf);
 }
 
 // Tensor copies of step 4's staging: the N/2 + 1 Hermitian rows in nb boxes of
@@ -485,28 +494,28 @@ cudaError_t go_rows(float2* ws, int W, int Hp, int L, int interp, const float2* 
 }
 
 template <int N, int INTERP>
-static cudaError_t go_rows_adj_i(float2* ws, int W, int Hp, int L, const float2* stw, int batch, cudaStream_t st) {
+static cudaError_t go_rows_adj_i(float2* ws, int W, int Hp, int L, const float2* stw, int batch, cudaStream_t st,
+                                 bool pdl, LossSum ls) {
     constexpr int B = fs_Brow(N);
     const size_t sm = (size_t)FastFft<N, -1, B>::SLOTS * sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(k_nvmt_rows_adjoint_fast<N, INTERP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     dim3 grid((L + B - 1) / B, batch);
-    k_nvmt_rows_adjoint_fast<N, INTERP><<<grid, fs_T(N) * B, sm, st>>>(ws, W, Hp, L, stw);
-    return cudaGetLastError();
+    return launch_maybe_pdl(k_nvmt_rows_adjoint_fast<N, INTERP>, grid, dim3(fs_T(N) * B), sm, st, pdl, ws, W, Hp, L,
+                            stw, ls);
 }
 
 template <int N>
-cudaError_t go_rows_adj(float2* ws, int W, int Hp, int L, int interp, const float2* stw, int batch,
-                               cudaStream_t st) {
-    return interp == FT_INTERP_LINEAR ? go_rows_adj_i<N, FT_INTERP_LINEAR>(ws, W, Hp, L, stw, batch, st)
-                                      : go_rows_adj_i<N, FT_INTERP_CUBIC>(ws, W, Hp, L, stw, batch, st);
+cudaError_t go_rows_adj(float2* ws, int W, int Hp, int L, int interp, const float2* stw, int batch, cudaStream_t st,
+                        bool pdl, LossSum ls) {
+    return interp == FT_INTERP_LINEAR ? go_rows_adj_i<N, FT_INTERP_LINEAR>(ws, W, Hp, L, stw, batch, st, pdl, ls)
+                                      : go_rows_adj_i<N, FT_INTERP_CUBIC>(ws, W, Hp, L, stw, batch, st, pdl, ls);
 }
-
 
 // the launchers of length n
 #define FT_FAST_INSTANTIATE(n) \
     template cudaError_t go_r2c<n>(const float* in, int rows_in, int ncols, int in_pitch, size_t in_img, int row0, const float2* stw, float2* out, int out_pitch, size_t out_img, float es, float ms, int batch, cudaStream_t st, bool pdl, bool follows_peak, unsigned* err, long long wait); \
-    template cudaError_t go_r2c_loss<n>(const float* map, const float* target, int ncols, const float2* stw, float2* out, int out_pitch, size_t out_img, float es, float ms, float scale, float gscale, float* partial, int batch, cudaStream_t st, unsigned* err, long long wait); \
+    template cudaError_t go_r2c_loss<n>(const float* map, const float* target, int ncols, const float2* stw, float2* out, int out_pitch, size_t out_img, float es, float ms, float scale, float gscale, float* partial, int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait); \
     template cudaError_t go_c2r<n>(const float2* in, int ncols, int in_pitch, size_t in_img, const float2* stw, float mid, float* out, int row0, int rows_out, int out_pitch, size_t out_img, float os, unsigned* tmax, int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait); \
     template cudaError_t go_rows<n>(float2* ws, int W, int Hp, int L, int interp, const float2* stw, int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait); \
-    template cudaError_t go_rows_adj<n>(float2* ws, int W, int Hp, int L, int interp, const float2* stw, int batch, cudaStream_t st);
+    template cudaError_t go_rows_adj<n>(float2* ws, int W, int Hp, int L, int interp, const float2* stw, int batch, cudaStream_t st, bool pdl, LossSum ls);

@@ -20,7 +20,7 @@ cudaError_t go_r2c(const float* in, int rows_in, int ncols, int in_pitch, size_t
 template <int N>
 cudaError_t go_r2c_loss(const float* map, const float* target, int ncols, const float2* stw, float2* out,
                                int out_pitch, size_t out_img, float es, float ms, float scale, float gscale,
-                               float* partial, int batch, cudaStream_t st, unsigned* err, long long wait);
+                               float* partial, int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait);
 template <int N>
 cudaError_t go_c2r(const float2* in, int ncols, int in_pitch, size_t in_img, const float2* stw,
                           float mid, float* out, int row0, int rows_out, int out_pitch, size_t out_img,
@@ -31,4 +31,4 @@ cudaError_t go_rows(float2* ws, int W, int Hp, int L, int interp, const float2* 
                            cudaStream_t st, bool pdl, unsigned* err, long long wait);
 template <int N>
 cudaError_t go_rows_adj(float2* ws, int W, int Hp, int L, int interp, const float2* stw, int batch,
-                               cudaStream_t st);
+                               cudaStream_t st, bool pdl, LossSum ls);

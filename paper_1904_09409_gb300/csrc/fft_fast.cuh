@@ -421,7 +421,7 @@ int col_r2c_loss_blocks(const FftLen& f, int ncols);
 cudaError_t launch_col_r2c_loss_fast(const float* map, const float* target, int ncols, const FftLen& f,
                                      float2* out, int out_pitch, size_t out_img, float end_scale, float mid_scale,
                                      float scale, float gscale, float* partial, int batch, cudaStream_t st,
-                                     unsigned* err = nullptr, long long wait = FT_WAIT_CYCLES);
+                                     bool pdl, unsigned* err = nullptr, long long wait = FT_WAIT_CYCLES);
 // tmax (may be NULL; only with row0 = 0 and rows_out = N): the maxima of |out| per
 // tile of c2r_tile_shape rows x columns, [batch][N / rows][ceil(ncols / cols)] as
 // float bits
@@ -443,4 +443,4 @@ bool c2r_tile_shape(int N, int* rows, int* cols, int* bands);
 cudaError_t launch_nvmt_rows_fast(float2* ws, int W, int Hp, int L, int interp, const FftLen& fx,
                                   int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait);
 cudaError_t launch_nvmt_rows_adjoint_fast(float2* ws, int W, int Hp, int L, int interp,
-                                          const FftLen& fx, int batch, cudaStream_t st);
+                                          const FftLen& fx, int batch, cudaStream_t st, bool pdl, LossSum ls);

@@ -117,6 +117,31 @@ static cudaError_t launch_maybe_pdl(void (*k)(KArgs...), dim3 g, dim3 b, size_t 
     return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// The partials of a loss to add up: loss[i] = the sum of partial[i n .. (i + 1) n)
+// divided by cells (loss NULL: none).
+struct LossSum {
+    const float* partial;
+    int n;
+    size_t cells;
+    float* loss;
+};
+// The first warp of the block: image img's sum, lane j adding the partials j, j + 32,
+// ... with compensation (Kahan), then a fixed shuffle tree.
+__device__ __forceinline__ void loss_sum_block(const LossSum& ls, int img) {
+    if (threadIdx.x >= 32) return;
+    const float* v = ls.partial + (size_t)img * ls.n;
+    float s = 0.f, comp = 0.f;
+    for (int i = threadIdx.x; i < ls.n; i += 32) {
+        const float y = v[i] - comp;
+        const float t = s + y;
+        comp = (t - s) - y;
+        s = t;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) ls.loss[img] = s / (float)ls.cells;
+}
+
 // ----------------------------------------------------- NVMT index helpers
 __device__ __forceinline__ int floor_div(int a, int b) {   // b > 0
     int q = a / b;
@@ -485,5 +510,5 @@ cudaError_t launch_transpose(const float* in, float* out, int R, int C, int batc
 cudaError_t launch_abs_mse_grad(const float* map, const float* target, int batch, size_t cells, float scale,
                                 float* loss, float* grad, float* partial, cudaStream_t st);
 size_t loss_partial_bytes(int batch);
-// per-image loss from nblk partials each (fixed order, compensated), divided by cells
-cudaError_t launch_loss_finish(const float* partial, int nblk, size_t cells, float* loss, int batch, cudaStream_t st);
+// the sums alone, one warp per image
+cudaError_t launch_loss_sum(LossSum ls, int batch, cudaStream_t st);

@@ -36,11 +36,11 @@ int col_r2c_loss_blocks(const FftLen& f, int ncols) {
 cudaError_t launch_col_r2c_loss_fast(const float* map, const float* target, int ncols, const FftLen& f,
                                      float2* out, int out_pitch, size_t out_img, float end_scale, float mid_scale,
                                      float scale, float gscale, float* partial, int batch, cudaStream_t st,
-                                     unsigned* err, long long wait) {
+                                     bool pdl, unsigned* err, long long wait) {
     if (ncols & 1) return cudaErrorInvalidValue;
     switch (f.N) {
 #define X(n) case n: return go_r2c_loss<n>(map, target, ncols, f.stw, out, out_pitch, out_img, end_scale, mid_scale, \
-                                           scale, gscale, partial, batch, st, err, wait);
+                                           scale, gscale, partial, batch, st, pdl, err, wait);
         FT_FAST_LENGTHS(X)
 #undef X
     }
@@ -88,9 +88,9 @@ cudaError_t launch_nvmt_rows_fast(float2* ws, int W, int Hp, int L, int interp, 
 }
 
 cudaError_t launch_nvmt_rows_adjoint_fast(float2* ws, int W, int Hp, int L, int interp,
-                                          const FftLen& fx, int batch, cudaStream_t st) {
+                                          const FftLen& fx, int batch, cudaStream_t st, bool pdl, LossSum ls) {
     switch (fx.N) {
-#define X(n) case n: return go_rows_adj<n>(ws, W, Hp, L, interp, fx.stw, batch, st);
+#define X(n) case n: return go_rows_adj<n>(ws, W, Hp, L, interp, fx.stw, batch, st, pdl, ls);
         FT_FAST_LENGTHS(X)
 #undef X
     }

@@ -7,7 +7,7 @@
 // The per-image sums are deterministic: each of LOSS_BLOCKS blocks of an image
 // reduces a fixed slice in a fixed order (FP32 with Kahan compensation per
 // thread, then a tree) and writes one partial; a second kernel adds the
-// partials of an image in index order.
+// partials of an image in a fixed order (LossSum).
 #include "ft_internal.cuh"
 
 #define LOSS_THREADS 256
@@ -42,22 +42,12 @@ k_abs_mse_grad(const float* __restrict__ map, const float* __restrict__ target, 
     if (threadIdx.x == 0) partial[img * gridDim.x + blockIdx.x] = red[0];
 }
 
-__global__ void k_loss_finish(const float* __restrict__ partial, int nblk, size_t cells, float* __restrict__ loss) {
-    const int img = blockIdx.x;
-    float s = 0.f, comp = 0.f;
-    for (int b = 0; b < nblk; ++b) {
-        const float y = partial[(size_t)img * nblk + b] - comp;
-        const float t = s + y;
-        comp = (t - s) - y;
-        s = t;
-    }
-    loss[img] = s / (float)cells;
-}
+__global__ void __launch_bounds__(32) k_loss_sum(LossSum ls) { loss_sum_block(ls, blockIdx.x); }
 
 size_t loss_partial_bytes(int batch) { return (size_t)batch * LOSS_BLOCKS * sizeof(float); }
 
-cudaError_t launch_loss_finish(const float* partial, int nblk, size_t cells, float* loss, int batch, cudaStream_t st) {
-    k_loss_finish<<<batch, 1, 0, st>>>(partial, nblk, cells, loss);
+cudaError_t launch_loss_sum(LossSum ls, int batch, cudaStream_t st) {
+    k_loss_sum<<<batch, 32, 0, st>>>(ls);
     return cudaGetLastError();
 }
 
@@ -68,6 +58,5 @@ cudaError_t launch_abs_mse_grad(const float* map, const float* target, int batch
     k_abs_mse_grad<<<g1, LOSS_THREADS, 0, st>>>(map, target, cells, scale, gscale, grad, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_loss_finish<<<batch, 1, 0, st>>>(partial, LOSS_BLOCKS, cells, loss);
-    return cudaGetLastError();
+    return launch_loss_sum(LossSum{partial, LOSS_BLOCKS, cells, loss}, batch, st);
 }

@@ -266,7 +266,10 @@ static cudaError_t nvmt_rows(ft_plan p, float2* ws, int batch, cudaStream_t st) 
     return launch_nvmt_rows(ws, p->W, p->S, p->Hp, p->L, p->interp, p->fx, p->row_logB_x, batch, st);
 }
 
-static cudaError_t nvmt_rows_adj(ft_plan p, float2* ws, int batch, cudaStream_t st) {
+// ls: the partials of a loss that the kernel adds up on the way (the fixed-length
+// kernels), or a launch of its own after it
+static bool rows_adj_sums(ft_plan p) { return p->interp != FT_INTERP_FOURIER && p->use_fast_x; }
+static cudaError_t nvmt_rows_adj(ft_plan p, float2* ws, int batch, cudaStream_t st, LossSum ls) {
     if (p->interp == FT_INTERP_FOURIER) {
         const size_t nu = (size_t)p->L * (p->W + 1), nx = (size_t)p->L * p->S;
         if (fourier_fast(p))
@@ -275,7 +278,7 @@ static cudaError_t nvmt_rows_adj(ft_plan p, float2* ws, int batch, cudaStream_t 
         return launch_nvmt_rows_fourier_adj(ws, p->W, p->S, p->Hp, p->L, p->fw, p->fm, p->fx, p->d_chirp,
                                             p->d_chirp + nu, p->d_chirp + nu + nx, batch, st);
     }
-    if (p->use_fast_x) return launch_nvmt_rows_adjoint_fast(ws, p->W, p->Hp, p->L, p->interp, p->fx, batch, st);
+    if (p->use_fast_x) return launch_nvmt_rows_adjoint_fast(ws, p->W, p->Hp, p->L, p->interp, p->fx, batch, st, p->pdl, ls);
     return launch_nvmt_rows_adjoint(ws, p->W, p->S, p->Hp, p->L, p->interp, p->fx, p->row_logB_x, batch, st);
 }
 
@@ -755,10 +758,12 @@ ft_status ft_forward(ft_plan p, const float* d_img, float* d_map, int batch, voi
 }
 
 // the adjoint after its first step (the spectrum of the map gradient is in ws)
-static ft_status backward_tail(ft_plan p, float2* ws, float* d_grad_img, int batch, cudaStream_t st) {
+static ft_status backward_tail(ft_plan p, float2* ws, float* d_grad_img, int batch, cudaStream_t st,
+                               LossSum ls = LossSum{}) {
     float* gdst = d_grad_img;
     if (p->space == FT_SPACE_INVERSE) gdst = (float*)((char*)p->d_ws + tposed_off(p, batch));
-    FT_LAUNCH(p, FT_KERNEL_NVMT_ROWS_ADJ, st, nvmt_rows_adj(p, ws, batch, st), "adjoint of steps 2-3");
+    FT_LAUNCH(p, FT_KERNEL_NVMT_ROWS_ADJ, st, nvmt_rows_adj(p, ws, batch, st, ls), "adjoint of steps 2-3");
+    if (ls.loss && !rows_adj_sums(p)) FT_LAUNCH(p, FT_KERNEL_LOSS, st, launch_loss_sum(ls, batch, st), "loss");
     FT_LAUNCH(p, FT_KERNEL_COL_C2R, st,
               col_c2r(p, ws, p->W, 0.5f, gdst, p->top, p->H, p->W, (size_t)p->H * p->W, 1.f, batch, st),
               "adjoint of step 1");
@@ -815,10 +820,9 @@ ft_status ft_abs_mse_backward(ft_plan p, const float* d_map, const float* d_targ
     const float gscale = (float)(1.0 / ((double)batch * (double)cells));
     FT_LAUNCH(p, FT_KERNEL_COL_R2C, st,
               launch_col_r2c_loss_fast(d_map, d_target, p->S, p->fy, ws, p->S, (size_t)p->L * p->S, inv, 2.f * inv,
-                                       scale, gscale, partial, batch, st, p->d_tc_err, p->tc_wait),
+                                       scale, gscale, partial, batch, st, p->pdl, p->d_tc_err, p->tc_wait),
               "loss and adjoint of step 4");
-    FT_LAUNCH(p, FT_KERNEL_LOSS, st, launch_loss_finish(partial, nblk, cells, d_loss, batch, st), "loss");
-    return backward_tail(p, ws, d_grad_img, batch, st);
+    return backward_tail(p, ws, d_grad_img, batch, st, LossSum{partial, nblk, cells, d_loss});
 }
 
 ft_status ft_peaks(ft_plan p, const float* d_map, int batch, int top_k, float threshold,
