@@ -346,15 +346,17 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
     constexpr int RL = fs_radix(N, fs_nst(N) - 1), GL = E / RL;
     constexpr int STEPX = N / R0;                      // x' distance between a thread's elements
     static_assert(R0 % 2 == 0, "half a row is whole elements of the first pass");
-    using F = FastFft<N, +1, B, true>;
+    // one transform per exchange buffer and T consecutive threads per row, so that a
+    // warp reads and writes consecutive samples of one row
+    using F = FastFft<N, +1, 1, true>;
     // [B][WP] input rows (sample x at PAD + x, 16-byte aligned, PAD zeros on
     // each side) in the FFT's own exchange buffer: they are read only by the
     // gather, which ends before the first exchange
     float2* srow = sm;
     constexpr int PAD = srow_pad(INTERP);
     const int WP = srow_pitch(W, INTERP);
-    const int f = threadIdx.x % B;
-    const int t = threadIdx.x / B;
+    const int f = threadIdx.x / T;
+    const int t = threadIdx.x % T;
     const int l0 = bx * B;
     const int l = l0 + f;
 
@@ -454,7 +456,7 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
     __syncthreads();                                   // the staged rows are dead from here
     // The centring factors (-1)^i of the gathered samples and (-1)^(s + N/2) of the
     // result are rotations by N/2 of the transform's output and of its input
-    F::template run<0>(v, sm, t, f, stw);
+    F::template run<0>(v, sm + f * F::SLOTS, t, 0, stw);
     if (l >= L) return true;
     float2* row = base + (size_t)l * N;
 #pragma unroll

@@ -235,10 +235,11 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
     constexpr int B = fs_Brow(N), E = fs_E(N), T = N / E;
     constexpr int R0 = fs_radix(N, 0), G0 = E / R0;
     constexpr int RL = fs_radix(N, fs_nst(N) - 1), GL = E / RL;
-    using F = FastFft<N, -1, B, true>;                 // the row length's seed table
-    extern __shared__ float2 sm[];
-    const int f = threadIdx.x % B;
-    const int t = threadIdx.x / B;
+    using F = FastFft<N, -1, 1, true>;                 // the row length's seed table
+    extern __shared__ float2 smrows[];
+    const int f = threadIdx.x / T;                     // T consecutive threads per row
+    const int t = threadIdx.x % T;
+    float2* sm = smrows + f * F::SLOTS;
     const int l = blockIdx.x * B + f;
     // images in reverse order, as in k_nvmt_rows_fast (L2 reuse with the column
     // kernels before and after, which run in forward order)
@@ -250,7 +251,7 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
 #pragma unroll
         for (int q = 0; q < R0; ++q)
             v[m * R0 + q] = (l < L) ? row[fs_rotate<N, R0>(F::template in_pos<0>(t, m, q), q)] : make_float2(0.f, 0.f);
-    F::template run<0>(v, sm, t, f, stw);
+    F::template run<0>(v, sm, t, 0, stw);
     // gV[x'] = (-1)^{i + N/2} z[i], i = x' + N/2, z the transform of (-1)^s g[s]: the
     // signs are the rotations of the transform's input and output by N/2
     const int st = spos(t);
@@ -261,7 +262,7 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
             const int c = F::out_pos(0, m, q);
             const int o = RL % 2 == 0 ? spos_plus(t, st, q < RL / 2 ? c + N / 2 : c - N / 2)
                                       : spos(fs_rotate<N, RL>(t + c, q));
-            sm[o * B + f] = v[m * RL + q];
+            sm[o] = v[m * RL + q];
         }
     __syncthreads();
     if (l >= L) return;
@@ -301,7 +302,7 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
                         keys_weights(fr, k4);
                         w = k4[j];
                     }
-                    const float2 g = sm[spos(xp[j] + N / 2) * B + f];
+                    const float2 g = sm[spos(xp[j] + N / 2)];
                     acc.x = fmaf(w, g.x, acc.x);
                     acc.y = fmaf(w, g.y, acc.y);
                 }

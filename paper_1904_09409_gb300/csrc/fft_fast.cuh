@@ -112,12 +112,13 @@ __host__ __device__ constexpr int fs_entexp(int R, bool seed, int j) {
 }
 __host__ __device__ constexpr int fs_pairs(int R, bool seed) { return (fs_nent(R, seed) + 1) / 2; }
 // float4 index of pair h of row k of a pass with P rows: by rows (the pairs of a
-// row adjacent), or by pairs (those of successive rows adjacent) in the full
-// tables of the long column lengths, whose warps hold 8 to 16 rows: a load then
+// row adjacent), or by pairs (those of successive rows adjacent) in the seed
+// tables of the row kernels, whose warps hold up to 32 rows, and in the full
+// tables of the long column lengths, whose warps hold 8 to 16: a load then
 // touches one or two lines instead of one per row (steps 1 and 4 of four 4096^2
 // images 180 / 178 -> 169 / 162 us, 8192 in 16 Mpx 72 / 70 -> 62 / 60; equal
 // within noise at 1024 and below, with 4 rows per warp or fewer)
-__host__ __device__ constexpr bool fs_bypairs(int N, bool seed) { return !seed && N > 1024; }
+__host__ __device__ constexpr bool fs_bypairs(int N, bool seed) { return seed || N > 1024; }
 __host__ __device__ constexpr int fs_pairpos(int N, int R, int P, bool seed, int h, int k) {
     return fs_bypairs(N, seed) ? h * P + k : k * fs_pairs(R, seed) + h;
 }
@@ -127,14 +128,16 @@ __host__ __device__ constexpr int fs_twoff(int N, int s, bool seed) {
     return o;
 }
 __host__ __device__ constexpr int fs_twsize(int N, bool seed) { return fs_twoff(N, fs_nst(N), seed); }
-// transforms per block for the column R2C kernels (512 threads; for N >= 4096,
+// transforms per block for the column R2C kernels (512 threads, 256 up to length
+// 512: 32 x 512^2 steps 1 and its transpose 27.1 -> 24.2 us; for N >= 4096,
 // 1024 threads so that a block still reads 4 column pairs = 32-byte row
 // segments), the column C2R kernel (256 threads, at least 4 column pairs, so
 // 512 threads for N = 1536, 2048; for N = 1024 512 threads, 8 column pairs:
-// with the tile maxima of ft_detect 121 us per 64 x 1024^2 against 124 us with
-// 256, and the peak pass is faster on the 16 x 16 tiles that gives) and the row
-// kernels (128 threads: at N = 1024, 2 rows per block run 116 us per
-// 64 x 1024^2, 4 rows 128 us, 1 row 142 us)
+// 98 us per 64 x 1024^2 against 109 with 256, and the peak pass is faster on the
+// 16 x 16 tiles that gives) and the row kernels (64 threads, T consecutive ones per
+// row, so that a warp reads and writes consecutive samples: 64 x 1024^2 84 us, with
+// 128 threads 86, with 256 97; 16 Mpx of 256^2 23 us, with 128 threads and the rows
+// interleaved over the lanes 34, of 128^2 27 against 57)
 //
 // The lengths with radices 6 to 24 (fs_wide) hold more than 64 registers' worth of
 // samples per thread (E = 18, 24, 36) or more temporaries (E = 12): fs_resident
@@ -156,14 +159,29 @@ __host__ __device__ constexpr int fs_Bwide(int N) {
     return fs_T(N) * 32 <= 288 ? 32 : fs_T(N) * 16 <= 192 ? 16 : fs_T(N) * 8 <= 512 ? 8 : 4;
 }
 __host__ __device__ constexpr int fs_Bcol(int N) {
-    return fs_wide(N) ? fs_Bwide(N) : fs_T(N) >= 256 ? 1024 / fs_T(N) : fs_clampB(512 / fs_T(N), 32);
+    return fs_wide(N) ? fs_Bwide(N) : fs_T(N) >= 256 ? 1024 / fs_T(N) : fs_clampB((N <= 512 ? 256 : 512) / fs_T(N), 32);
 }
 __host__ __device__ constexpr int fs_Bc2r(int N) {
     return fs_wide(N) ? fs_Bwide(N)
          : fs_T(N) >= 256 ? 1024 / fs_T(N)
                           : fs_clampB(N == 1024 ? 512 / fs_T(N) : (256 / fs_T(N) < 4 ? 4 : 256 / fs_T(N)), 32);
 }
-__host__ __device__ constexpr int fs_Brow(int N) { return fs_clampB((128 + (fs_wide(N) ? fs_T(N) / 2 : 0)) / fs_T(N), 16); }
+// rows per block of the row kernels: 64 threads for the powers of two and 3 x 2^a up
+// to 1536 (one row from length 1024 on), and for the other lengths, whose T is no
+// multiple of a warp, the count that fills its last warp best with at most 144
+__host__ __device__ constexpr int fs_Brow(int N) {
+    if (!fs_wide(N)) return fs_clampB(64 / fs_T(N), 16);
+    int best = 1, num = 0, den = 1;
+    for (int b = 1; b == 1 || b * fs_T(N) <= 144; ++b) {
+        const int used = b * fs_T(N), alloc = (used + 31) / 32 * 32;
+        if (used >= 48 && used * den > num * alloc) {
+            best = b;
+            num = used;
+            den = alloc;
+        }
+    }
+    return best;
+}
 // padded shared-memory slot of sample n (one spare slot every 16 samples
 // spreads the strided stores of the first pass over the banks)
 __host__ __device__ constexpr int spos(int n) { return n + (n >> 4); }
