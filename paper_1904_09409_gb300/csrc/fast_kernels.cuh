@@ -7,6 +7,8 @@
 
 #include <string.h>
 
+#include <atomic>
+
 #include "fast_blocks.cuh"
 #include "fast_launch.cuh"
 
@@ -373,14 +375,31 @@ static bool r2c_tma_map(const float* in, int rows_in, int ncols, int in_pitch, s
 // the whole GPU at once (0 when it cannot be determined).  Measured per
 // 64 x 1024^2 step (pipelined): 2 waves 345 us, 1 wave 320, 1/2 317, 1/4 316,
 // 1/8 320, none 327.
+// It depends only on the kernel and the device, and the occupancy query is a large
+// part of a small launch's host time, so each launcher keeps it per device (cache:
+// the launcher's own words, 0: unknown, else distance + 1; any thread may fill them).
+#define FT_PF_DEVICES 16
 template <typename K>
-static int prefetch_distance(K k, int threads, size_t sm) {
+static int prefetch_distance(std::atomic<int>* cache, K k, int threads, size_t sm) {
     int dev = 0, per = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev < FT_PF_DEVICES) {
+        const int c = cache[dev].load(std::memory_order_relaxed);
+        if (c) return c - 1;
+    }
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, sm) != cudaSuccess)
         return 0;
-    return per * nsm / 2;
+    const int d = per * nsm / 2;
+    if (dev < FT_PF_DEVICES) cache[dev].store(d + 1, std::memory_order_relaxed);
+    return d;
+}
+
+// dynamic shared memory above the 48 KB that every kernel may use needs the
+// kernel's consent
+template <typename K>
+static cudaError_t allow_smem(K k, size_t sm) {
+    return sm > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) : cudaSuccess;
 }
 
 template <int N>
@@ -389,14 +408,15 @@ cudaError_t go_r2c(const float* in, int rows_in, int ncols, int in_pitch, size_t
                           int batch, cudaStream_t st, bool pdl, bool follows_peak, unsigned* err, long long wait) {
     constexpr int B = fs_Bcol(N);
     const size_t sm = (size_t)FastFft<N, -1, B>::SLOTS * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_col_r2c_fast<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(k_col_r2c_fast<N>, sm);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     memset(&map, 0, sizeof(map));
     int h = 0, nb = 0;
     if (!err || wait < 0 || !r2c_tma_map<N>(in, rows_in, ncols, in_pitch, in_img, batch, &map, &h, &nb)) nb = 0;
     dim3 grid((ncols + 2 * B - 1) / (2 * B), batch);
-    const int pf = prefetch_distance(k_col_r2c_fast<N>, fs_T(N) * B, sm);
+    static std::atomic<int> pfc[FT_PF_DEVICES];
+    const int pf = prefetch_distance(pfc, k_col_r2c_fast<N>, fs_T(N) * B, sm);
     return launch_maybe_pdl(k_col_r2c_fast<N>, grid, dim3(fs_T(N) * B), sm, st, pdl, in, rows_in, ncols, in_pitch,
                             in_img, row0, stw, out, out_pitch, out_img, es, ms, map, h, nb, err, wait, pf,
                             (pdl && follows_peak) ? 1 : 0);
@@ -408,7 +428,7 @@ cudaError_t go_r2c_loss(const float* map, const float* target, int ncols, const 
                                float* partial, int batch, cudaStream_t st, bool pdl, unsigned* err, long long wait) {
     constexpr int B = fs_Bcol(N);
     const size_t sm = (size_t)FastFft<N, -1, B>::SLOTS * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_col_r2c_loss_fast<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(k_col_r2c_loss_fast<N>, sm);
     if (e != cudaSuccess) return e;
     CUtensorMap pm, tm;
     memset(&pm, 0, sizeof(pm));
@@ -419,7 +439,8 @@ cudaError_t go_r2c_loss(const float* map, const float* target, int ncols, const 
         !r2c_tma_map<N>(target, N, ncols, ncols, cells, batch, &tm, &h2, &nb2))
         nb = 0;
     dim3 grid((ncols + 2 * B - 1) / (2 * B), batch);
-    const int pf = prefetch_distance(k_col_r2c_loss_fast<N>, fs_T(N) * B, sm);
+    static std::atomic<int> pfc[FT_PF_DEVICES];
+    const int pf = prefetch_distance(pfc, k_col_r2c_loss_fast<N>, fs_T(N) * B, sm);
     return launch_maybe_pdl(k_col_r2c_loss_fast<N>, grid, dim3(fs_T(N) * B), sm, st, pdl, map, target, ncols, cells,
                             stw, out, out_pitch, out_img, es, ms, scale, gscale, partial, pm, tm, h, nb, err, wait, pf);
 }
@@ -462,14 +483,15 @@ cudaError_t go_c2r(const float2* in, int ncols, int in_pitch, size_t in_img, con
                           long long wait) {
     constexpr int B = fs_Bc2r(N);
     const size_t sm = (size_t)FastFft<N, +1, B>::SLOTS * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_col_c2r_fast<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(k_col_c2r_fast<N>, sm);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     memset(&map, 0, sizeof(map));
     int h = 0, nb = 0;
     if (!err || wait < 0 || !c2r_tma_map<N>(in, in_pitch, in_img, batch, &map, &h, &nb)) nb = 0;
     dim3 grid((ncols + 2 * B - 1) / (2 * B), batch);
-    const int pf = prefetch_distance(k_col_c2r_fast<N>, fs_T(N) * B, sm);
+    static std::atomic<int> pfc[FT_PF_DEVICES];
+    const int pf = prefetch_distance(pfc, k_col_c2r_fast<N>, fs_T(N) * B, sm);
     return launch_maybe_pdl(k_col_c2r_fast<N>, grid, dim3(fs_T(N) * B), sm, st, pdl, in, ncols, in_pitch, in_img, stw,
                             mid, out, row0, rows_out, out_pitch, out_img, os, tmax, map, h, nb, err, wait, pf);
 }
@@ -480,7 +502,7 @@ static cudaError_t go_rows_i(float2* ws, int W, int Hp, int L, const float2* stw
     constexpr int B = fs_Brow(N);
     const size_t slots = FastFft<N, +1, B>::SLOTS, rows = (size_t)srow_pitch(W, INTERP) * B;
     const size_t sm = (slots > rows ? slots : rows) * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_nvmt_rows_fast<N, INTERP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(k_nvmt_rows_fast<N, INTERP>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid((L + B - 1) / B, batch);
     return launch_maybe_pdl(k_nvmt_rows_fast<N, INTERP>, grid, dim3(fs_T(N) * B), sm, st, pdl, ws, W, Hp, L, stw,
@@ -499,7 +521,7 @@ static cudaError_t go_rows_adj_i(float2* ws, int W, int Hp, int L, const float2*
                                  bool pdl, LossSum ls) {
     constexpr int B = fs_Brow(N);
     const size_t sm = (size_t)FastFft<N, -1, B>::SLOTS * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_nvmt_rows_adjoint_fast<N, INTERP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(k_nvmt_rows_adjoint_fast<N, INTERP>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid((L + B - 1) / B, batch);
     return launch_maybe_pdl(k_nvmt_rows_adjoint_fast<N, INTERP>, grid, dim3(fs_T(N) * B), sm, st, pdl, ws, W, Hp, L,
