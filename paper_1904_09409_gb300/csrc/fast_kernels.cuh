@@ -27,7 +27,7 @@ k_col_r2c_fast(const float* __restrict__ in, int rows_in, int ncols, int in_pitc
                size_t out_img, float end_scale, float mid_scale, const __grid_constant__ CUtensorMap tmap,
                int tma_h, int tma_nb, unsigned* __restrict__ err, long long wait, int pf, int follows_peak) {
     extern __shared__ __align__(128) float2 sm[];
-    pdl_trigger();
+    pdl_trigger_large();
     if (!follows_peak) pdl_wait();
     const float* src = in + (size_t)blockIdx.y * in_img;
     float2* dst = out + (size_t)blockIdx.y * out_img;
@@ -54,7 +54,7 @@ k_col_c2r_fast(const float2* __restrict__ in, int ncols, int in_pitch, size_t in
                const __grid_constant__ CUtensorMap tmap, int tma_h, int tma_nb, unsigned* __restrict__ err,
                long long wait, int pf) {
     extern __shared__ __align__(128) float2 sm[];
-    pdl_trigger();
+    pdl_trigger_large();
     pdl_wait();
     constexpr int bands = c2r_tile_rows(N) ? N / c2r_tile_rows(N) : 0;
     const float2* src = in + (size_t)blockIdx.y * in_img;
@@ -110,7 +110,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
     __shared__ uint64_t mbar;
     const uint32_t mb = smem_u32(&mbar);
     float2 v[E];
-    pdl_trigger();
+    pdl_trigger_large();
     pdl_wait();
     float* part = partial + (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     if (tma_nb > 0) {
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(fs_T(N) * fs_Brow(N), fs_minblocks(N, fs_T(N) 
 k_nvmt_rows_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __restrict__ stw,
                  unsigned* __restrict__ err, long long wait) {
     extern __shared__ __align__(128) float2 sm[];
-    pdl_trigger();
+    pdl_trigger_large();
     pdl_wait();
     // images in reverse order: the first blocks read the half spectra step 1
     // wrote last (still in L2), and step 4, in forward order, starts on the
@@ -231,7 +231,7 @@ k_nvmt_rows_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __
 template <int N, int INTERP>
 __global__ void __launch_bounds__(fs_T(N) * fs_Brow(N), fs_minblocks(N, fs_T(N) * fs_Brow(N)))
 k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __restrict__ stw, LossSum ls) {
-    pdl_trigger();
+    pdl_trigger_large();
     pdl_wait();
     if (ls.loss && blockIdx.x == gridDim.x - 1) loss_sum_block(ls, blockIdx.y);
     constexpr int B = fs_Brow(N), E = fs_E(N), T = N / E;

@@ -94,10 +94,19 @@ __device__ __forceinline__ float2 twiddle(const float2* __restrict__ tw, int t) 
 // predecessor has completed and its writes are visible, and is a no-op for a
 // kernel launched without the attribute.  Every such kernel calls it before its
 // first read or write of device memory.  pdl_trigger() lets the successor be
-// launched early (steps 1-4 call it when their blocks start, the peak pass
-// after its wait).
+// launched early (steps 1-4 call it when their blocks start if their grid is
+// large, the peak pass after its wait).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The transform kernels trigger when their blocks start only if the grid is large,
+// so that the successor's blocks fill the multiprocessors that the last wave leaves.
+// With few blocks there is no such wave, and the waiting blocks of the successor
+// only get in the way (forward, us, trigger always / never: 4 x 512^2 17.4 / 10.5,
+// 1024^2 20.3 / 14.4, 1536x576 25.3 / 16.6; 32 x 512^2 38.9 / 39.3, 64 x 1024^2 268.2 /
+// 269.9; the line at 1024 blocks has the better of the two in every case).
+__device__ __forceinline__ void pdl_trigger_large() {
+    if (gridDim.x * gridDim.y >= 1024u) pdl_trigger();
+}
 
 // launch kernel k (grid g, block b, sm bytes of dynamic shared memory) on st,
 // with programmatic stream serialisation when pdl is set

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
 k_batch_r2c(const BatchImg* __restrict__ imgs, const int2* __restrict__ items, const float* __restrict__ in,
             float2* __restrict__ ws) {
     extern __shared__ float2 sm[];
-    pdl_trigger();
+    pdl_trigger_large();
     const int2 it = items[blockIdx.x];
     const BatchImg& d = imgs[it.x];
     const int W = d.W;
@@ -47,7 +47,7 @@ template <int NT, int INTERP>
 __global__ void __launch_bounds__(NT, 1024 / NT)
 k_batch_rows(const BatchImg* __restrict__ imgs, const int2* __restrict__ items, float2* __restrict__ ws) {
     extern __shared__ float2 sm[];
-    pdl_trigger();
+    pdl_trigger_large();
     const int2 it = items[blockIdx.x];
     const BatchImg& d = imgs[it.x];
     const int H = d.H, W = d.W;
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
 k_batch_c2r(const BatchImg* __restrict__ imgs, const int2* __restrict__ items, const float2* __restrict__ ws,
             float* __restrict__ maps, unsigned* __restrict__ tmax) {
     extern __shared__ float2 sm[];
-    pdl_trigger();
+    pdl_trigger_large();
     const int2 it = items[blockIdx.x];
     const BatchImg& d = imgs[it.x];
     const int H = d.H, W = d.W;
