@@ -10,7 +10,7 @@
 // the transforms of length W and S run on all G B rows at once, the two of length
 // M on B rows at a time in G rounds, and every thread has work in every pass.
 // (One round of B rows per block, half of the threads idle in the passes of length
-// W and S, took 124 us per 16 x 1024^2, this form 108, with
+// W and S, took 124 us per 16 x 1024^2, this form 103, with
 // the centring factors as rotations and constant shared-memory offsets.)  Between the transforms the rows live
 // in a second shared buffer; the exchanges go through the first.  Rows are
 // numbered l batch + image, so consecutive rows share the chirp tables of row l
@@ -18,7 +18,9 @@
 // memory about once per call, and blocks are full whatever the batch.  The kernel
 // is bound by issue and latency at 16 warps per multiprocessor (four transforms
 // in a row keep about 170 registers live unbounded; 128 leave at most a few words
-// spilled), so what counts is the number of passes and table loads per row.
+// spilled), so what counts is the number of passes and table loads per row.  Its
+// blocks are too large to share a multiprocessor with waiting ones of step 4, so it
+// does not trigger early (1024x512, two images: 30.0 us per forward, now 22.0).
 #include "fft_fast.cuh"
 
 template <int W>
@@ -60,14 +62,6 @@ __device__ __forceinline__ int fr_fresh(int t) {
     return t;
 }
 
-// prefetch into L1 the chirp tables of the rows of frequencies l0 .. l1 (len
-// complex values each, contiguous over l): one 128-byte line per thread and step
-__device__ __forceinline__ void fr_prefetch(const float2* table, int len, int l0, int l1, int nt) {
-    const char* p = reinterpret_cast<const char*>(table + (size_t)l0 * len);
-    const int bytes = (l1 - l0 + 1) * len * (int)sizeof(float2);
-    for (int o = threadIdx.x * 128; o < bytes; o += nt * 128) asm volatile("prefetch.global.L1 [%0];" ::"l"(p + o));
-}
-
 // the samples k = x' + S/2 of row l inside the support, x' H' / (2 l) in
 // [-W/2, W/2 - 1]: lo <= k <= hi
 __device__ __forceinline__ void fr_support(int l, int Hp, int W, int S, int& lo, int& hi) {
@@ -84,27 +78,21 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
     using Sh = FrShape<W>;
     constexpr int M = Sh::M, S = W, B = Sh::B, NR = Sh::NR;
     constexpr int EW = fs_E(W), EM = fs_E(M);
-    using FW = FastFft<W, -1, NR, true>;
-    using FMf = FastFft<M, -1, B, true>;
-    using FMi = FastFft<M, +1, B, true>;
-    using FS = FastFft<S, +1, NR, true>;
+    using FW = FastFft<W, -1, 1, true>;
+    using FMf = FastFft<M, -1, 1, true>;
+    using FMi = FastFft<M, +1, 1, true>;
+    using FS = FastFft<S, +1, 1, true>;
     constexpr int R0W = fs_radix(W, 0), G0W = EW / R0W, RLW = fs_radix(W, fs_nst(W) - 1), GLW = EW / RLW;
     constexpr int R0M = fs_radix(M, 0), G0M = EM / R0M, RLM = fs_radix(M, fs_nst(M) - 1), GLM = EM / RLM;
     static_assert(R0W % 2 == 0 && R0M % 2 == 0, "halves of a row are whole elements of the first pass");
     extern __shared__ __align__(16) float2 sm[];
     float2* rows = sm + Sh::SX;                        // [spos(k)][NR]
-    pdl_trigger();
-    {   // the tables of the block's frequencies (they do not depend on the predecessor)
-        const int l0 = blockIdx.x * NR / batch, l1 = min((blockIdx.x * NR + NR - 1) / batch, L - 1);
-        if (l1 - l0 < 2) {
-            fr_prefetch(chirp_u, W + 1, l0, l1, Sh::NT);
-            fr_prefetch(hc, M, l0, l1, Sh::NT);
-            fr_prefetch(chirp_x, S, l0, l1, Sh::NT);
-        }
-    }
     pdl_wait();
 
-    const int fr = threadIdx.x % NR, tr0 = threadIdx.x / NR;
+    // T consecutive threads per transform, each transform in an exchange buffer of its own
+    const int fr = threadIdx.x / Sh::TW, tr0 = threadIdx.x % Sh::TW;
+    float2* smr = sm + fr * FW::SLOTS;
+    float2* rowr = rows + fr * FW::SLOTS;
     const FrRow rw = fr_row(ws, blockIdx.x * NR + fr, L, batch, S);
     // ---- F_W^- of the block's rows
     {
@@ -116,18 +104,20 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
             for (int q = 0; q < R0W; ++q)
                 v[m * R0W + q] = rw.ok ? __ldcg(rw.p + fs_rotate<W, R0W>(FW::template in_pos<0>(tr, m, q), q))
                                        : make_float2(0.f, 0.f);
-        FW::template run<0>(v, sm, tr, fr, stw_w);
+        FW::template run<0>(v, smr, tr, 0, stw_w);
 #pragma unroll
         for (int m = 0; m < GLW; ++m)
 #pragma unroll
-            for (int q = 0; q < RLW; ++q) rows[spos_plus(tr, spos(tr), FW::out_pos(0, m, q)) * NR + fr] = v[m * RLW + q];
+            for (int q = 0; q < RLW; ++q) rowr[spos_plus(tr, spos(tr), FW::out_pos(0, m, q))] = v[m * RLW + q];
     }
     __syncthreads();
 
-    const int f = threadIdx.x % B, t0 = threadIdx.x / B;
+    const int f = threadIdx.x / Sh::TM, t0 = threadIdx.x % Sh::TM;
+    float2* smf = sm + f * FMf::SLOTS;
 #pragma unroll 1
     for (int g = 0; g < Sh::G; ++g) {
         const int fg = g * B + f;
+        float2* rowg = rows + fg * FW::SLOTS;
         const FrRow rm = fr_row(ws, blockIdx.x * NR + fg, L, batch, S);
         const int t = fr_fresh(t0), st = spos(t);
         const int l = rm.ok ? rm.l : 0;                // the tables' row; rows past the end are not stored
@@ -150,7 +140,7 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
                             slot = spos_plus(t, st, q < R0M / 4 ? c + W / 2 : c - W / 2);
                         else
                             slot = spos(i < W / 2 ? i + W / 2 : i - W / 2);
-                        float2 a = rows[slot * NR + fg];
+                        float2 a = rowg[slot];
                         if (m == 0 && (q == 0 || q == R0M / 2) && t == 0) a = cscale(a, 0.5f);
                         y = cmul(a, __ldg(cu + i));
                     }
@@ -158,7 +148,7 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
                 }
         }
         // ---- F_M^-, times the chirp spectrum, back to the input order, F_M^+
-        FMf::template run<0>(v, sm, t, f, stw_m);
+        FMf::template run<0>(v, smf, t, 0, stw_m);
         {
             const float2* hl = hc + (size_t)l * M;
 #pragma unroll
@@ -166,7 +156,7 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
 #pragma unroll
                 for (int q = 0; q < RLM; ++q) {
                     const int k = FMf::out_pos(t, m, q);
-                    sm[spos_plus(t, st, FMf::out_pos(0, m, q)) * B + f] = cmul(v[m * RLM + q], __ldg(hl + k));
+                    smf[spos_plus(t, st, FMf::out_pos(0, m, q))] = cmul(v[m * RLM + q], __ldg(hl + k));
                 }
         }
         __syncthreads();
@@ -174,9 +164,9 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
 #pragma unroll
         for (int m = 0; m < G0M; ++m)
 #pragma unroll
-            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = sm[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q)) * B + f];
+            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = smf[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q))];
         __syncthreads();
-        FMi::template run<0>(v, sm, ti, f, stw_m);
+        FMi::template run<0>(v, smf, ti, 0, stw_m);
         // ---- V[k] = z[k] / (W M) x post-chirp inside the support, for k < S = M / 2 (the
         // lower half of the last pass's elements), stored rotated by S/2; the DC row is zero
         {
@@ -198,7 +188,7 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
                             slot = spos_plus(ti, sti, FMi::out_pos(0, m, q) + (q < RLM / 4 ? S / 2 : -S / 2));
                         else
                             slot = spos(k < S / 2 ? k + S / 2 : k - S / 2);
-                        rows[slot * NR + fg] = r;
+                        rowg[slot] = r;
                     }
                 }
         }
@@ -214,8 +204,8 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q)
-                v[m * R0W + q] = rows[spos_plus(tr, str, FS::template in_pos<0>(0, m, q)) * NR + fr];
-        FS::template run<0>(v, sm, tr, fr, stw_s);
+                v[m * R0W + q] = rowr[spos_plus(tr, str, FS::template in_pos<0>(0, m, q))];
+        FS::template run<0>(v, smr, tr, 0, stw_s);
         if (rw.ok) {
 #pragma unroll
             for (int m = 0; m < GLW; ++m)
@@ -241,27 +231,21 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
     using Sh = FrShape<W>;
     constexpr int M = Sh::M, S = W, B = Sh::B, NR = Sh::NR;
     constexpr int EW = fs_E(W), EM = fs_E(M);
-    using FS = FastFft<S, -1, NR, true>;
-    using FMf = FastFft<M, -1, B, true>;
-    using FMi = FastFft<M, +1, B, true>;
-    using FW = FastFft<W, +1, NR, true>;
+    using FS = FastFft<S, -1, 1, true>;
+    using FMf = FastFft<M, -1, 1, true>;
+    using FMi = FastFft<M, +1, 1, true>;
+    using FW = FastFft<W, +1, 1, true>;
     constexpr int R0W = fs_radix(W, 0), G0W = EW / R0W, RLW = fs_radix(W, fs_nst(W) - 1), GLW = EW / RLW;
     constexpr int R0M = fs_radix(M, 0), G0M = EM / R0M, RLM = fs_radix(M, fs_nst(M) - 1), GLM = EM / RLM;
     extern __shared__ __align__(16) float2 sm[];
     float2* rows = sm + Sh::SX;
     __shared__ float2 nyq[NR];
-    pdl_trigger();
-    {   // the tables of the block's frequencies (they do not depend on the predecessor)
-        const int l0 = blockIdx.x * NR / batch, l1 = min((blockIdx.x * NR + NR - 1) / batch, L - 1);
-        if (l1 - l0 < 2) {
-            fr_prefetch(chirp_u, W + 1, l0, l1, Sh::NT);
-            fr_prefetch(hc, M, l0, l1, Sh::NT);
-            fr_prefetch(chirp_x, S, l0, l1, Sh::NT);
-        }
-    }
     pdl_wait();
 
-    const int fr = threadIdx.x % NR, tr0 = threadIdx.x / NR;
+    // T consecutive threads per transform, each transform in an exchange buffer of its own
+    const int fr = threadIdx.x / Sh::TW, tr0 = threadIdx.x % Sh::TW;
+    float2* smr = sm + fr * FW::SLOTS;
+    float2* rowr = rows + fr * FW::SLOTS;
     const FrRow rw = fr_row(ws, blockIdx.x * NR + fr, L, batch, S);
     // ---- O, F_S^-, (-1)^k: rotations by S/2 of the input and the output
     {
@@ -273,7 +257,7 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
             for (int q = 0; q < R0W; ++q)
                 v[m * R0W + q] = rw.ok ? __ldcg(rw.p + fs_rotate<S, R0W>(FS::template in_pos<0>(tr, m, q), q))
                                        : make_float2(0.f, 0.f);
-        FS::template run<0>(v, sm, tr, fr, stw_s);
+        FS::template run<0>(v, smr, tr, 0, stw_s);
 #pragma unroll
         for (int m = 0; m < GLW; ++m)
 #pragma unroll
@@ -281,15 +265,17 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                 const int c = FS::out_pos(0, m, q);
                 const int slot = RLW % 2 == 0 ? spos_plus(tr, spos(tr), q < RLW / 2 ? c + S / 2 : c - S / 2)
                                               : spos(fs_rotate<S, RLW>(tr + c, q));
-                rows[slot * NR + fr] = v[m * RLW + q];
+                rowr[slot] = v[m * RLW + q];
             }
     }
     __syncthreads();
 
-    const int f = threadIdx.x % B, t0 = threadIdx.x / B;
+    const int f = threadIdx.x / Sh::TM, t0 = threadIdx.x % Sh::TM;
+    float2* smf = sm + f * FMf::SLOTS;
 #pragma unroll 1
     for (int g = 0; g < Sh::G; ++g) {
         const int fg = g * B + f;
+        float2* rowg = rows + fg * FW::SLOTS;
         const FrRow rm = fr_row(ws, blockIdx.x * NR + fg, L, batch, S);
         const int t = fr_fresh(t0), st = spos(t);
         const int l = rm.ok ? rm.l : 0;
@@ -310,14 +296,14 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                         const int k = FMf::template in_pos<0>(t, m, q);
                         if (k >= lo && k <= hi) {
                             const float2 c = __ldg(cx + k);
-                            const float2 a = rows[spos_plus(t, st, FMf::template in_pos<0>(0, m, q)) * NR + fg];
+                            const float2 a = rowg[spos_plus(t, st, FMf::template in_pos<0>(0, m, q))];
                             r = cscale(cmul(a, make_float2(c.x, -c.y)), sc);
                         }
                     }
                     v[m * R0M + q] = r;
                 }
         }
-        FMf::template run<0>(v, sm, t, f, stw_m);
+        FMf::template run<0>(v, smf, t, 0, stw_m);
         {
             const float2* hl = hc + (size_t)l * M;
 #pragma unroll
@@ -326,7 +312,7 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                 for (int q = 0; q < RLM; ++q) {
                     const int k = FMf::out_pos(t, m, q);
                     const float2 h = __ldg(hl + k);
-                    sm[spos_plus(t, st, FMf::out_pos(0, m, q)) * B + f] = cmul(v[m * RLM + q], make_float2(h.x, -h.y));
+                    smf[spos_plus(t, st, FMf::out_pos(0, m, q))] = cmul(v[m * RLM + q], make_float2(h.x, -h.y));
                 }
         }
         __syncthreads();
@@ -334,9 +320,9 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
 #pragma unroll
         for (int m = 0; m < G0M; ++m)
 #pragma unroll
-            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = sm[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q)) * B + f];
+            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = smf[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q))];
         __syncthreads();
-        FMi::template run<0>(v, sm, ti, f, stw_m);
+        FMi::template run<0>(v, smf, ti, 0, stw_m);
         // ---- conj(D_u) and P^T on the entries i = u + W/2 <= W (halved at u = +-W/2)
         {
             const float2* cu = chirp_u + (size_t)l * (W + 1);
@@ -352,7 +338,7 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                         if (i == W)
                             nyq[fg] = r;
                         else
-                            rows[spos(i < W / 2 ? i + W / 2 : i - W / 2) * NR + fg] = r;
+                            rowg[spos(i < W / 2 ? i + W / 2 : i - W / 2)] = r;
                     }
                 }
         }
@@ -368,11 +354,11 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q) {
-                float2 a = rows[spos_plus(tr, str, FW::template in_pos<0>(0, m, q)) * NR + fr];
+                float2 a = rowr[spos_plus(tr, str, FW::template in_pos<0>(0, m, q))];
                 if (FW::template in_pos<0>(tr, m, q) == W / 2) a = cadd(a, nyq[fr]);
                 v[m * R0W + q] = a;
             }
-        FW::template run<0>(v, sm, tr, fr, stw_w);
+        FW::template run<0>(v, smr, tr, 0, stw_w);
         if (rw.ok) {
 #pragma unroll
             for (int m = 0; m < GLW; ++m)
