@@ -14,7 +14,13 @@
 
 static thread_local char g_last_error[256] = "";
 
-#define FT_DETECT_CHUNK 8   // images per chunk of the ft_detect_host pipeline
+// Bytes of images per chunk of the ft_detect_host pipeline (at least one image): the
+// upload of a chunk hides the previous chunk's transform, and only the last chunk's
+// transform is exposed, so chunks are as small as keeps the transform of one, which
+// is bound by launches and latency, shorter than its upload (24 MiB: 120 us).  From
+// pinned memory, us, against chunks of 8 images: 16 x 1024^2 460 -> 439 (with 8 MiB
+// 521, 32 MiB 453), 64 x 256^2 393 -> 175, 8 x 2048^2 922 -> 779, 2 x 4096^2 1035 -> 863.
+#define FT_DETECT_CHUNK_BYTES ((size_t)24 << 20)
 #define FT_LANES 2          // streams a large batch is split over (see lanes_fork)
 
 static ft_status cuda_fail(cudaError_t e, const char* where) {
@@ -148,13 +154,18 @@ static ft_status build_chirps(ft_plan p) {
 // q = fs_entexp(R, seed, j) for entry j, k < P, from the exact-index table tw of
 // length N; pair h = j / 2 of row k is float4 fs_pairpos(...) of the pass.
 static void stage_twiddles(int N, const float2* tw, float2* out, bool seed) {
-    for (int s = 1; s < fs_nst(N); ++s) {
+    const int nst = fs_nst(N);
+    for (int s = 1; s < nst; ++s) {
         const int R = fs_radix(N, s), P = fs_P(N, s), step = N / (P * R), NE = fs_nent(R, seed);
+        const int pairs = fs_pairs(R, seed);
+        const bool by = fs_bypairs(N, seed);
         float2* o = out + fs_twoff(N, s, seed);
-        for (int k = 0; k < P; ++k)
-            for (int j = 0; j < 2 * fs_pairs(R, seed); ++j)
-                o[2 * fs_pairpos(N, R, P, seed, j / 2, k) + (j & 1)] =
-                    j < NE ? tw[fs_entexp(R, seed, j) * k * step] : make_float2(0.f, 0.f);
+        for (int j = 0; j < 2 * pairs; ++j) {
+            const int q = j < NE ? fs_entexp(R, seed, j) * step : 0;
+            float2* oj = o + (by ? j / 2 * P : j / 2) * 2 + (j & 1);
+            const int stride = 2 * (by ? 1 : pairs);
+            for (int k = 0; k < P; ++k) oj[k * stride] = j < NE ? tw[q * k] : make_float2(0.f, 0.f);
+        }
     }
 }
 
@@ -1077,7 +1088,8 @@ ft_status ft_detect_host(ft_plan p, const float* h_img, int batch, int top_k, fl
     p->d_count_host = (int32_t*)((char*)p->d_peaks_host + cnt_off);
     // Chunks of images: the copy stream uploads chunk c + 1 while the caller's
     // stream transforms chunk c; peaks and counts come back per chunk.
-    const int chunk = batch < FT_DETECT_CHUNK ? batch : FT_DETECT_CHUNK;
+    const size_t per = FT_DETECT_CHUNK_BYTES / (img_px * sizeof(float));
+    const int chunk = per < 1 ? 1 : (per < (size_t)batch ? (int)per : batch);
     const int nchunks = (batch + chunk - 1) / chunk;
     if (!p->copy_stream) FT_CUDA(cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking), "copy stream");
     if (!p->start_event) FT_CUDA(cudaEventCreateWithFlags(&p->start_event, cudaEventDisableTiming), "event");
