@@ -155,9 +155,9 @@ __device__ __forceinline__ bool r2c_block(const float* __restrict__ in, int rows
 
 // The part of step 4 after staging, for column block bx of one image: sm holds
 // the Hermitian half [N/2 + 1][2B] complex (and serves as the FFT's exchange
-// buffer afterwards); arguments as for c2r_block.  TILES: tile maxima can be
-// asked for (the block's threads divide into whole tiles).
-template <int N, int B, bool TILES>
+// buffer afterwards); arguments as for c2r_block.  WARPTILES: a tile's cells are
+// held by whole warps (lengths whose T is a multiple of the tile's rows).
+template <int N, int B, bool WARPTILES>
 __device__ __forceinline__ void c2r_from_stage(float2* sm, int ncols, const float2* __restrict__ stw,
                                                float mid_scale, float* __restrict__ out, int row0, int rows_out,
                                                int out_pitch, float out_scale, unsigned* __restrict__ tmax, int nbx,
@@ -198,38 +198,68 @@ __device__ __forceinline__ void c2r_from_stage(float2* sm, int ncols, const floa
     }
     __syncthreads();
     F::template run<0>(v, sm, t, f, stw);
-    if constexpr (TILES) if (tmax) {
-        // Tile maxima of |map| for the peak pass: thread t holds rows t + T j,
-        // j = m + GL q, of its column pair.  A tile is RS = 128 / B consecutive
-        // rows of one band (rows T j + RS u .. T j + RS u + RS - 1, u < T / RS) of
-        // the block's 2B columns: 256 cells held, one each, by the 128
-        // consecutive threads RS B u .. RS B u + 127, i.e. by whole warps
-        // 4u .. 4u + 3.  Every warp reduces its 32 values of band j with one
-        // redux.sync (max(|re|, |im|) of the stored, scaled values; NaN counts
-        // as 0, like a cell that is never a peak), lane 0 keeps the partial in
-        // the exchange buffer, which the FFT no longer reads, and one thread per
-        // tile combines its four warps' partials.
-        constexpr int NT = fs_T(N) * B;                // threads of the block
-        constexpr int NW = NT / 32;
-        constexpr int RS = 128 / B, TPB = fs_T(N) / RS;   // tile rows, tiles per band
-        static_assert(RS * B == 128 && TPB * RS == fs_T(N), "a tile is 128 threads' values");
-        static_assert(E * NW <= FastFft<N, +1, B>::SLOTS * 2, "partial maxima fit the exchange buffer");
-        unsigned* part = reinterpret_cast<unsigned*>(sm);  // [E][NW]
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if constexpr (WARPTILES) {
+        if (tmax) {
+            // Tile maxima of |map| for the peak pass: thread t holds rows t + T j,
+            // j = m + GL q, of its column pair.  A tile is RS = 128 / B consecutive
+            // rows of one band (rows T j + RS u .. T j + RS u + RS - 1, u < T / RS) of
+            // the block's 2B columns: 256 cells held, one each, by the 128
+            // consecutive threads RS B u .. RS B u + 127, i.e. by whole warps
+            // 4u .. 4u + 3.  Every warp reduces its 32 values of band j with one
+            // redux.sync (max(|re|, |im|) of the stored, scaled values; NaN counts
+            // as 0, like a cell that is never a peak), lane 0 keeps the partial in
+            // the exchange buffer, which the FFT no longer reads, and one thread per
+            // tile combines its four warps' partials.
+            constexpr int NT = fs_T(N) * B;                // threads of the block
+            constexpr int NW = NT / 32;
+            constexpr int RS = 128 / B, TPB = fs_T(N) / RS;   // tile rows, tiles per band
+            static_assert(RS * B == 128 && TPB * RS == fs_T(N), "a tile is 128 threads' values");
+            static_assert(E * NW <= FastFft<N, +1, B>::SLOTS * 2, "partial maxima fit the exchange buffer");
+            unsigned* part = reinterpret_cast<unsigned*>(sm);  // [E][NW]
+            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+            for (int m = 0; m < GL; ++m)
+#pragma unroll
+                for (int q = 0; q < RL; ++q) {
+                    const float a = fabsf(v[m * RL + q].x * out_scale), b = fabsf(v[m * RL + q].y * out_scale);
+                    const unsigned x = __reduce_max_sync(0xffffffffu, colok ? __float_as_uint(fmaxf(fmaxf(a, b), 0.f)) : 0u);
+                    if (lane == 0) part[(m + GL * q) * NW + warp] = x;
+                }
+            __syncthreads();
+            for (int w = threadIdx.x; w < E * TPB; w += NT) {
+                const unsigned* p = part + (w / TPB) * NW + 4 * (w % TPB);
+                const unsigned x = max(max(p[0], p[1]), max(p[2], p[3]));
+                if (FT_IN(bx, nbx, FT_DBG_C2R_STORE)) tmax[(size_t)w * nbx + bx] = x;
+            }
+        }
+    } else if (tmax) {
+        // the same maxima where T is no multiple of a tile's rows: every thread leaves
+        // its cells' |.| in the exchange buffer and warps reduce tiles of it (a separate
+        // read of the map by k_tile_max took 6 us per 8 x 486x648)
+        constexpr int NWF = fs_T(N) * B / 32;          // whole warps
+        constexpr int RS = 128 / B;
+        static_assert(NWF >= 1 && RS * B == 128 && N <= 2 * FastFft<N, +1, B>::SLOTS / B, "tiles of 128 pairs");
+        float* mx = reinterpret_cast<float*>(sm);      // [N][B]
 #pragma unroll
         for (int m = 0; m < GL; ++m)
 #pragma unroll
             for (int q = 0; q < RL; ++q) {
                 const float a = fabsf(v[m * RL + q].x * out_scale), b = fabsf(v[m * RL + q].y * out_scale);
-                const unsigned x = __reduce_max_sync(0xffffffffu, colok ? __float_as_uint(fmaxf(fmaxf(a, b), 0.f)) : 0u);
-                if (lane == 0) part[(m + GL * q) * NW + warp] = x;
+                mx[F::out_pos(t, m, q) * B + f] = colok ? fmaxf(fmaxf(a, b), 0.f) : 0.f;
             }
         __syncthreads();
-        for (int w = threadIdx.x; w < E * TPB; w += NT) {
-            const unsigned* p = part + (w / TPB) * NW + 4 * (w % TPB);
-            const unsigned x = max(max(p[0], p[1]), max(p[2], p[3]));
-            if (FT_IN(bx, nbx, FT_DBG_C2R_STORE)) tmax[(size_t)w * nbx + bx] = x;
-        }
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (warp < NWF)
+            for (int w = warp; w < (N + RS - 1) / RS; w += NWF) {
+                float x = 0.f;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int i = w * 128 + k * 32 + lane;
+                    if (i < N * B) x = fmaxf(x, mx[i]);
+                }
+                const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(x));
+                if (lane == 0 && FT_IN(bx, nbx, FT_DBG_C2R_STORE)) tmax[(size_t)w * nbx + bx] = u;
+            }
     }
     if (!colok) return;
     // row n of the result goes to output row n - row0 when that is in range

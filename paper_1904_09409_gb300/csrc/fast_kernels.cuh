@@ -56,7 +56,7 @@ k_col_c2r_fast(const float2* __restrict__ in, int ncols, int in_pitch, size_t in
     extern __shared__ __align__(128) float2 sm[];
     pdl_trigger_large();
     pdl_wait();
-    constexpr int bands = c2r_tile_rows(N) ? N / c2r_tile_rows(N) : 0;
+    constexpr int bands = c2r_tile_bands(N);
     const float2* src = in + (size_t)blockIdx.y * in_img;
     float* dst = out + (size_t)blockIdx.y * out_img;
     unsigned* tm = tmax ? tmax + (size_t)blockIdx.y * bands * gridDim.x : nullptr;

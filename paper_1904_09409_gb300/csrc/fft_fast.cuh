@@ -441,7 +441,7 @@ cudaError_t launch_col_r2c_loss_fast(const float* map, const float* target, int 
                                      float scale, float gscale, float* partial, int batch, cudaStream_t st,
                                      bool pdl, unsigned* err = nullptr, long long wait = FT_WAIT_CYCLES);
 // tmax (may be NULL; only with row0 = 0 and rows_out = N): the maxima of |out| per
-// tile of c2r_tile_shape rows x columns, [batch][N / rows][ceil(ncols / cols)] as
+// tile of c2r_tile_shape rows x columns, [batch][ceil(N / rows)][ceil(ncols / cols)] as
 // float bits
 // (err, wait: with err given, the staging goes through tensor copies whose
 // bounded waits set bit 2 of *err when they run out; without, cp.async)
@@ -452,10 +452,10 @@ cudaError_t launch_col_c2r_fast(const float2* in, int ncols, int in_pitch, size_
                                 unsigned* err = nullptr, long long wait = FT_WAIT_CYCLES);
 // tiles of the tile maxima of launch_col_c2r_fast for length N: rows x cols
 // cells, bands = N / rows tiles per column block; false without a schedule.
-// A tile is 256 cells: 128 / B rows of one column block of 2B columns, held by
-// whole warps; lengths whose column block does not divide that way (fs_wide)
-// write no maxima (rows 0 here, false from c2r_tile_shape).
-__host__ __device__ constexpr int c2r_tile_rows(int N) { return fs_wide(N) ? 0 : 128 / fs_Bc2r(N); }
+// A tile is 256 cells: 128 / B rows of one column block of 2B columns (the last
+// band of a length that the rows do not divide is ragged).
+__host__ __device__ constexpr int c2r_tile_rows(int N) { return 128 / fs_Bc2r(N); }
+__host__ __device__ constexpr int c2r_tile_bands(int N) { return (N + c2r_tile_rows(N) - 1) / c2r_tile_rows(N); }
 bool c2r_tile_shape(int N, int* rows, int* cols, int* bands);
 // (err: bit 1 set when a bulk-copy wait ran out after `wait` SM cycles)
 cudaError_t launch_nvmt_rows_fast(float2* ws, int W, int Hp, int L, int interp, const FftLen& fx,

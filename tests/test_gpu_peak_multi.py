@@ -39,6 +39,10 @@ CASES = [
     (128, 200, 216, 4096, 100, float("-inf")),    # 32 x 8 tiles
     (64, 16, 16, 8192, 5, float("-inf")),         # 64 x 4 tiles, 4 tile columns
     (64, 4, 4, 8192, 5, float("-inf")),           # one tile column: a tile is its own neighbour
+    (480, 640, 648, 486, 8, float("-inf")),       # tiles reduced through shared memory, a ragged last band
+    (150, 96, 108, 162, 5, float("-inf")),        # 4 x 64 tiles, wider than half the map
+    (1000, 200, 216, 1152, 20, float("-inf")),    # 16 x 16 tiles, S no multiple of 16
+    (300, 60, 64, 3888, 33, float("-inf")),       # 32 x 8 tiles, 36 samples per thread
     (256, 256, 256, 256, 1024, float("-inf")),    # K above the number of tiles
     (256, 256, 256, 256, 64, 30.0),               # a threshold few peaks pass
     (256, 256, 256, 256, 64, 1e9),                # a threshold none passes
