@@ -84,8 +84,7 @@ k_col_c2r_fast(const float2* __restrict__ in, int ncols, int in_pitch, size_t in
 // so that the last one adds them 15 us of 166 per 64 x 1024^2, the fence's wait).  With
 // tma_nb > 0 the map columns arrive by tensor copies into the exchange buffer
 // (pmap, waited for with the bound `wait`; bit 3 of *err when it runs out, and
-// the block returns without writing), their values go to registers, and the
-// target columns (tmapt) follow into the same buffer; the map and target boxes
+// the block returns without writing); the map and target (tmapt) boxes
 // of the block pf blocks later are prefetched into L2.  Everything after the
 // load is r2c_finish.
 template <int N>
@@ -106,7 +105,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
     const bool colok = c < ncols;
     const float* P = map + (size_t)blockIdx.y * img_cells + c;
     const float* Tg = target + (size_t)blockIdx.y * img_cells + c;
-    const float* stg = reinterpret_cast<const float*>(sm);   // [tma_nb tma_h][2B] map, then target values
+    const float* stg = reinterpret_cast<const float*>(sm);   // [tma_nb tma_h][2B] map values
     __shared__ uint64_t mbar;
     const uint32_t mb = smem_u32(&mbar);
     float2 v[E];
@@ -114,11 +113,12 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
     pdl_wait();
     float* part = partial + (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     if (tma_nb > 0) {
-        // the block's map columns by tensor copies into the exchange buffer, their
-        // values to registers, then the target columns into the same buffer
-        // (the mbarrier's second phase; both are read before the FFT's first
-        // exchange); the map and target boxes of the block pf blocks later are
-        // prefetched into L2
+        // the block's map columns by tensor copies into the exchange buffer; their
+        // latency hides that of the target values, which come straight from global
+        // memory to registers (prefetched into L2 like the map by the block pf blocks
+        // before).  A second round of copies for the target, after the map had gone to
+        // registers, took 49.5 us per 16 Mpx of 512^2 and 167 us per 64 x 1024^2, this 44
+        // and 161
         if (threadIdx.x == 0) {
             mbar_init(mb, 1);
             mbar_arrive_expect_tx(mb, (uint32_t)(tma_nb * tma_h * 2 * B * sizeof(float)));
@@ -134,42 +134,32 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
                 }
             }
         }
+    }
+#pragma unroll
+    for (int m = 0; m < G0; ++m)
+#pragma unroll
+        for (int q = 0; q < R0; ++q)
+            v[m * R0 + q] = colok ? __ldg(reinterpret_cast<const float2*>(
+                                        Tg + (size_t)F::template in_pos<0>(t, m, q) * ncols))
+                                  : make_float2(0.f, 0.f);
+    if (tma_nb > 0) {
         __syncthreads();                               // the mbarrier is initialised
-        bool ok = mbar_wait(mb, 0, wait);
+        const bool ok = mbar_wait(mb, 0, wait);
         if (__syncthreads_or(!ok)) {
             if (threadIdx.x == 0 && err) atomicOr(err, 8u);
             mbar_wait(mb, 0);                          // the copies in flight land first
             if (threadIdx.x == 0) *part = __int_as_float(0x7fc00000);   // NaN: the loss is incomplete
             return;
         }
-#pragma unroll
-        for (int m = 0; m < G0; ++m)
-#pragma unroll
-            for (int q = 0; q < R0; ++q)
-                v[m * R0 + q] = *reinterpret_cast<const float2*>(stg + F::template in_pos<0>(t, m, q) * 2 * B + 2 * f);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // these reads before the refill
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            mbar_arrive_expect_tx(mb, (uint32_t)(tma_nb * tma_h * 2 * B * sizeof(float)));
-            for (int k = 0; k < tma_nb; ++k)
-                tma_load_3d(reinterpret_cast<float*>(sm) + k * tma_h * 2 * B, &tmapt, blockIdx.x * 2 * B, k * tma_h,
-                            blockIdx.y, mb);
-        }
-        ok = mbar_wait(mb, 1, wait);
-        if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0 && err) atomicOr(err, 8u);
-            mbar_wait(mb, 1);
-            if (threadIdx.x == 0) *part = __int_as_float(0x7fc00000);
-            return;
-        }
     }
 
-    float acc = 0.f, comp = 0.f;
-    auto add = [&](float y) {                          // compensated sum of r^2
-        const float z = y - comp;
-        const float s2 = acc + z;
-        comp = (s2 - acc) - z;
-        acc = s2;
+    // compensated sums of r^2, one per column of the pair (two chains of dependent adds)
+    float acc2[2] = {0.f, 0.f}, comp2[2] = {0.f, 0.f};
+    auto add = [&](int i, float y) {
+        const float z = y - comp2[i];
+        const float s2 = acc2[i] + z;
+        comp2[i] = (s2 - acc2[i]) - z;
+        acc2[i] = s2;
     };
 #pragma unroll
     for (int m = 0; m < G0; ++m)
@@ -178,18 +168,19 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
             const int row = F::template in_pos<0>(t, m, q);
             float2 g = make_float2(0.f, 0.f);
             if (colok) {
-                const float2 p = tma_nb > 0 ? v[m * R0 + q] : __ldg(reinterpret_cast<const float2*>(P + (size_t)row * ncols));
-                const float2 tt = tma_nb > 0 ? *reinterpret_cast<const float2*>(stg + row * 2 * B + 2 * f)
-                                             : __ldg(reinterpret_cast<const float2*>(Tg + (size_t)row * ncols));
+                const float2 p = tma_nb > 0 ? *reinterpret_cast<const float2*>(stg + row * 2 * B + 2 * f)
+                                            : __ldg(reinterpret_cast<const float2*>(P + (size_t)row * ncols));
+                const float2 tt = v[m * R0 + q];
                 const float r0 = fabsf(p.x) * scale - tt.x, r1 = fabsf(p.y) * scale - tt.y;
-                add(r0 * r0);
-                add(r1 * r1);
+                add(0, r0 * r0);
+                add(1, r1 * r1);
                 const float s0 = p.x > 0.f ? 1.f : (p.x < 0.f ? -1.f : 0.f);
                 const float s1 = p.y > 0.f ? 1.f : (p.y < 0.f ? -1.f : 0.f);
                 g = make_float2(2.f * r0 * scale * s0 * gscale, 2.f * r1 * scale * s1 * gscale);
             }
             v[m * R0 + q] = g;
         }
+    float acc = (acc2[0] + acc2[1]) - (comp2[0] + comp2[1]);
     // the block's partial: a fixed shuffle tree per warp, then over the warps (the
     // last warp may be partial; lane 0's sum takes nothing from lanes it lacks)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

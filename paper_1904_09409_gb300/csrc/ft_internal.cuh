@@ -134,21 +134,16 @@ struct LossSum {
     size_t cells;
     float* loss;
 };
-// The first warp of the block: image img's sum, lane j adding the partials j, j + 32,
-// ... with compensation (Kahan), then a fixed shuffle tree.
+// The first warp of the block: image img's sum in FP64 (a few thousand values), lane
+// j adding the partials j, j + 32, ..., then a fixed shuffle tree.
 __device__ __forceinline__ void loss_sum_block(const LossSum& ls, int img) {
     if (threadIdx.x >= 32) return;
     const float* v = ls.partial + (size_t)img * ls.n;
-    float s = 0.f, comp = 0.f;
-    for (int i = threadIdx.x; i < ls.n; i += 32) {
-        const float y = v[i] - comp;
-        const float t = s + y;
-        comp = (t - s) - y;
-        s = t;
-    }
+    double s = 0.0;
+    for (int i = threadIdx.x; i < ls.n; i += 32) s += (double)v[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) ls.loss[img] = s / (float)ls.cells;
+    if (threadIdx.x == 0) ls.loss[img] = (float)(s / (double)ls.cells);
 }
 
 // ----------------------------------------------------- NVMT index helpers
