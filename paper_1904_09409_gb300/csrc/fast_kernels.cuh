@@ -259,52 +259,67 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
         }
     __syncthreads();
     if (l >= L) return;
-    // Column x receives from the sample x' with floor(x' H' / (2 l)) = x - W/2 - d
-    // (at most one, since H' >= 2 l), i.e. x' = ceil((x - W/2 - d) 2 l / H').  With
-    // num = (x - W/2 - d) 2 l + H' - 1 = x' H' + rem (0 <= rem < H') such an x'
-    // exists iff H' - 1 - rem < 2 l, and its fraction is (H' - 1 - rem) / (2 l).
-    // Successive columns of a thread differ by T, so (x', rem) are stepped exactly.
+    // Column x receives, for each tap d, from the sample x' with floor(x' H' / (2 l)) =
+    // u = x - W/2 - d (at most one, since H' >= 2 l): x' = ceil(u 2 l / H'), with
+    // x' H' - u 2 l = k (0 <= k < H'); such an x' exists iff k < 2 l, and its fraction is
+    // k / (2 l).  A thread takes two adjacent columns, whose taps share all but one of
+    // their u: ND + 1 pairs (x', k) instead of 2 ND, stepped exactly from one pair of
+    // columns to the next (k, an integer below 8192, in FP32: no conversion for the
+    // fraction).  The kernel is bound by these instructions: 16 Mpx of 1024^2 took 35.1 us
+    // (linear) and 53.1 (cubic) with one column and integer steps per pass, 29.3 and 38.0
+    // so.
     constexpr int DLO = INTERP == FT_INTERP_LINEAR ? 0 : -1;
     constexpr int DHI = INTERP == FT_INTERP_LINEAR ? 1 : 2;
     constexpr int ND = DHI - DLO + 1;
-    const int halfW = W >> 1;
     const int den = 2 * l;
     const float inv = 1.f / (float)den;
-    const int step = T * den;
-    const int sA = step / Hp, sB = step - sA * Hp;
-    int xp[ND], rem[ND];
-#pragma unroll
-    for (int j = 0; j < ND; ++j) {
-        const int num = (t - halfW - (DLO + j)) * den + Hp - 1;
-        xp[j] = floor_div(num, Hp);
-        rem[j] = num - xp[j] * Hp;
+    const float hpf = (float)Hp, denf = (float)den;
+    const int sA = 2 * T * den / Hp;
+    const float sB = (float)(2 * T * den - sA * Hp);
+    int xp[ND + 1];
+    float k[ND + 1];
+    {
+        const int num = (2 * t + 1 - (W >> 1) - DLO) * den + Hp - 1;
+        xp[0] = floor_div(num, Hp);
+        k[0] = (float)(Hp - 1 - (num - xp[0] * Hp));
     }
-    const int lim = Hp - 1 - den;                      // a sample exists iff rem > lim
-    for (int x = t; x < W; x += T) {
-        float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 1; j <= ND; ++j) {                    // u one less: k grows by 2 l <= H'
+        xp[j] = xp[j - 1];
+        k[j] = k[j - 1] + denf;
+        if (k[j] >= hpf) { k[j] -= hpf; xp[j] -= 1; }
+    }
+    for (int x = 2 * t; x < W; x += 2 * T) {
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);  // columns x, x + 1
         if (l >= 1) {
 #pragma unroll
-            for (int j = 0; j < ND; ++j) {
-                if (rem[j] > lim && xp[j] >= -N / 2 && xp[j] < N / 2 && FT_IN(xp[j] + N / 2, N, FT_DBG_NVMT_ADJ)) {
-                    const float fr = (float)(Hp - 1 - rem[j]) * inv;
-                    float w;
+            for (int j = 0; j <= ND; ++j) {
+                if (k[j] < denf && xp[j] >= -N / 2 && xp[j] < N / 2 && FT_IN(xp[j] + N / 2, N, FT_DBG_NVMT_ADJ)) {
+                    const float fr = k[j] * inv;
+                    float w[ND];
                     if constexpr (INTERP == FT_INTERP_LINEAR) {
-                        w = j == 0 ? 1.f - fr : fr;
+                        w[0] = 1.f - fr;
+                        w[1] = fr;
                     } else {
-                        float k4[4];                   // the one the unrolled j uses is computed
-                        keys_weights(fr, k4);
-                        w = k4[j];
+                        keys_weights(fr, w);           // those the unrolled j uses are computed
                     }
                     const float2 g = sm[spos(xp[j] + N / 2)];
-                    acc.x = fmaf(w, g.x, acc.x);
-                    acc.y = fmaf(w, g.y, acc.y);
+                    if (j >= 1) {
+                        acc.x = fmaf(w[j - 1], g.x, acc.x);
+                        acc.y = fmaf(w[j - 1], g.y, acc.y);
+                    }
+                    if (j < ND) {
+                        acc.z = fmaf(w[j], g.x, acc.z);
+                        acc.w = fmaf(w[j], g.y, acc.w);
+                    }
                 }
-                rem[j] += sB;
                 xp[j] += sA;
-                if (rem[j] >= Hp) { rem[j] -= Hp; xp[j] += 1; }
+                k[j] -= sB;
+                if (k[j] < 0.f) { k[j] += hpf; xp[j] += 1; }
             }
         }
-        row[x] = acc;
+        if (x + 1 < W) *reinterpret_cast<float4*>(row + x) = acc;
+        else row[x] = make_float2(acc.x, acc.y);
     }
 }
 
