@@ -4,11 +4,12 @@
 // block over a uniform batch; the mixed-size batch kernels of k_batch.cu run
 // them over images of different lengths.  B, the transforms
 // per block, is a template parameter: the block has fs_T(N) * B threads.
-//  * the column R2C reads its first pass directly from global memory; the
-//    other two stage their inputs into shared memory with 16-byte cp.async
-//    copies, all in flight at once (C2R: the Hermitian half, each row read once
-//    for both n and N - n; rows: the B spectrum rows feeding the NVMT gather);
-//    the last pass writes global memory directly where the output order allows;
+//  * the per-plan kernels stage their inputs with tensor and bulk copies, the
+//    grouped ones read the column R2C's first pass directly from global memory
+//    and stage the other two with 16-byte cp.async copies, all in flight at once
+//    (C2R: the Hermitian half, each row read once for both n and N - n; rows: the
+//    B spectrum rows feeding the NVMT gather); the last pass writes global
+//    memory directly where the output order allows;
 //  * the NVMT sample x' H' / (2 l) of successive elements of a thread is stepped
 //    exactly by adding the precomputed quotient and remainder of
 //    (N / R0) H' / (2 l), so the inner loop has no integer division;
@@ -440,21 +441,23 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
         const int den = 2 * l;
         const float inv = 1.f / (float)den;
         const int step = STEPX * Hp;
-        const int sA = step / den, sB = step - sA * den;
+        const int sA = step / den;
+        const float sB = (float)(step - sA * den), denf = (float)den;
         const int halfW = W >> 1;
         const float2 zero = make_float2(0.f, 0.f);
 #pragma unroll
         for (int m = 0; m < G0; ++m) {
             // element q is the sample x' = i for i < N/2, i - N beyond (i = t + m T +
-            // q N / R0: the row rotated by N/2), visited in ascending x'
+            // q N / R0: the row rotated by N/2), visited in ascending x'; the remainder,
+            // an integer below 8192, is stepped in FP32, without a conversion per fraction
             const int i = t + m * T;
             const int num = (i - N / 2) * Hp;
             int qf = floor_div(num, den);
-            int rem = num - qf * den;
+            float rem = (float)(num - qf * den);
 #pragma unroll
             for (int qq = 0; qq < R0; ++qq) {
                 const int q = (qq + R0 / 2) % R0;
-                const float fr = (float)rem * inv;
+                const float fr = rem * inv;
                 const int c0 = qf + halfW;
                 float2 acc;
                 if constexpr (INTERP == FT_INTERP_LINEAR) {
@@ -479,7 +482,7 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
                 v[m * R0 + q] = acc;
                 rem += sB;
                 qf += sA;
-                if (rem >= den) { rem -= den; qf += 1; }
+                if (rem >= denf) { rem -= denf; qf += 1; }
             }
         }
     }
