@@ -105,7 +105,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
     const bool colok = c < ncols;
     const float* P = map + (size_t)blockIdx.y * img_cells + c;
     const float* Tg = target + (size_t)blockIdx.y * img_cells + c;
-    const float* stg = reinterpret_cast<const float*>(sm);   // [tma_nb tma_h][2B] map values
+    const float* stg = reinterpret_cast<const float*>(sm);   // [>= N][2B] map values
     __shared__ uint64_t mbar;
     const uint32_t mb = smem_u32(&mbar);
     float2 v[E];
@@ -134,6 +134,18 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
                 }
             }
         }
+    } else if (colok) {
+        // the same overlap where the tensor copies don't apply (2B columns or an image
+        // row no multiple of 16 bytes): every thread copies its own pairs and waits for
+        // them alone (16 Mpx of 486^2: 83.0 us with the map read in the loop below, 54.8 so)
+        static_assert(N * B <= F::SLOTS, "the map columns fit the exchange buffer");
+#pragma unroll
+        for (int m = 0; m < G0; ++m)
+#pragma unroll
+            for (int q = 0; q < R0; ++q) {
+                const int row = F::template in_pos<0>(t, m, q);
+                cp_async8(reinterpret_cast<float*>(sm) + row * 2 * B + 2 * f, P + (size_t)row * ncols);
+            }
     }
 #pragma unroll
     for (int m = 0; m < G0; ++m)
@@ -151,6 +163,8 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
             if (threadIdx.x == 0) *part = __int_as_float(0x7fc00000);   // NaN: the loss is incomplete
             return;
         }
+    } else {
+        cp_async_wait_all();
     }
 
     // compensated sums of r^2, one per column of the pair (two chains of dependent adds)
@@ -168,8 +182,7 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
             const int row = F::template in_pos<0>(t, m, q);
             float2 g = make_float2(0.f, 0.f);
             if (colok) {
-                const float2 p = tma_nb > 0 ? *reinterpret_cast<const float2*>(stg + row * 2 * B + 2 * f)
-                                            : __ldg(reinterpret_cast<const float2*>(P + (size_t)row * ncols));
+                const float2 p = *reinterpret_cast<const float2*>(stg + row * 2 * B + 2 * f);
                 const float2 tt = v[m * R0 + q];
                 const float r0 = fabsf(p.x) * scale - tt.x, r1 = fabsf(p.y) * scale - tt.y;
                 add(0, r0 * r0);
@@ -180,7 +193,8 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
             }
             v[m * R0 + q] = g;
         }
-    float acc = (acc2[0] + acc2[1]) - (comp2[0] + comp2[1]);
+    const float comp = comp2[0] + comp2[1];
+    float acc = acc2[0] + acc2[1] - (comp == comp ? comp : 0.f);   // NaN once a sum overflows
     // the block's partial: a fixed shuffle tree per warp, then over the warps (the
     // last warp may be partial; lane 0's sum takes nothing from lanes it lacks)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
