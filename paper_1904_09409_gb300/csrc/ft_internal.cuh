@@ -320,12 +320,11 @@ struct ft_plan_s {
     int use_fast_y, use_fast_x;      // fixed-length kernels in use for H' / S
     int variant;            // see ft_plan_set_variant
     int peak_mode;          // peak pass: 0 = the fastest by the cost model, else FT_PASS_*
-    void* d_peak_state;     // per-image words of the pass over the whole GPU (zero between calls)
-    size_t peak_state_bytes;
+    void* d_peak_state;     // per-image words of the peak pass over the whole GPU (zero between calls)
     int num_sms;            // multiprocessors of the plan's device
     int pdl;                // programmatic dependent launch in the forward chain (FT_PDL=0: off)
     int precision;          // ft_precision of step 3 (ft_plan_set_precision)
-    unsigned* d_tc_err;     // error flags of the tensor-core kernels (allocated with the first split precision)
+    unsigned* d_tc_err;     // error flags of the device-side waits; d_peak_state follows in the same allocation
     long long tc_wait;      // bound of every tensor-core wait in SM cycles (ft_plan_set_wait_cycles)
     int alloc_failures;     // device allocations still to fail (ft_plan_inject_alloc_failures)
     // band-limited (chirp-z) interpolator: lengths W and M >= W + S, chirp tables
@@ -416,6 +415,7 @@ cudaError_t launch_peak_sparse(const float* map, const unsigned* tmax, int Hp, i
 // words of peak_multi_state_bytes(batch) that are zero before the first call and
 // that every call leaves so.
 size_t peak_multi_scratch_bytes(int ntiles, int batch);
+#define FT_MULTI_MAX_BATCH 1024   // images per call (more of them fill the GPU with one block each)
 size_t peak_multi_state_bytes(int batch);
 cudaError_t launch_peak_multi(const float* map, const unsigned* tmax, int Hp, int S, int tile_rows, int tile_cols,
                               int batch, int top_k, float threshold, void* scratch, void* state, ft_peak* out,

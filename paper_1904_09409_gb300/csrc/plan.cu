@@ -206,18 +206,12 @@ static ft_status ensure(ft_plan p, void** ptr, size_t* have, size_t need, const 
     return FT_OK;
 }
 
-// ensure() for counters that kernels expect zero and leave zero: a new buffer is
-// cleared on the stream
-static ft_status zeroed(ft_plan p, void** ptr, size_t* have, size_t need, cudaStream_t st, const char* what) {
-    if (need <= *have && *ptr) return FT_OK;
-    const ft_status s = ensure(p, ptr, have, need, what);
-    if (s != FT_OK) return s;
-    const cudaError_t e = cudaMemsetAsync(*ptr, 0, need, st);
-    if (e == cudaSuccess) return FT_OK;
-    cudaFree(*ptr);
-    *ptr = nullptr;
-    *have = 0;
-    return cuda_fail(e, what);
+// a CUDA graph is being captured from this stream: nothing can be allocated
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
 }
 
 static size_t spec_bytes(ft_plan p, int batch) { return (size_t)batch * p->L * p->S * sizeof(float2); }
@@ -393,20 +387,26 @@ ft_status ft_plan_create_space(ft_plan* out, int img_H, int img_W, int n_slope, 
         cuda_fail(e, "cudaMalloc(twiddles)");
         return FT_ERR_OOM;
     }
-    e = cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        cudaFree(p->d_tw);
-        delete p;
-        return cuda_fail(e, "cudaMemcpy(twiddles)");
-    }
-    // the error word of the device-side waits (bulk copies, tensor cores)
-    e = cudaMalloc(&p->d_tc_err, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemset(p->d_tc_err, 0, sizeof(unsigned));
+    // the error word of the device-side waits (bulk copies, tensor cores), and 256
+    // bytes on the per-image words of the peak pass over the whole GPU (allocated on
+    // that pass's first call they made it 50 us longer); the copy of the twiddles
+    // waits for the clearing
+    const size_t zero_bytes = 256 + peak_multi_state_bytes(FT_MULTI_MAX_BATCH);
+    e = cudaMalloc(&p->d_tc_err, zero_bytes);
+    if (e == cudaSuccess) e = cudaMemset(p->d_tc_err, 0, zero_bytes);
     if (e != cudaSuccess) {
         if (p->d_tc_err) cudaFree(p->d_tc_err);
         cudaFree(p->d_tw);
         delete p;
         return cuda_fail(e, "cudaMalloc(error word)");
+    }
+    p->d_peak_state = (char*)p->d_tc_err + 256;
+    e = cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaFree(p->d_tc_err);
+        cudaFree(p->d_tw);
+        delete p;
+        return cuda_fail(e, "cudaMemcpy(twiddles)");
     }
     p->fy.tw = p->d_tw;
     p->fx.tw = p->d_tw + fy.N;
@@ -464,7 +464,6 @@ ft_status ft_plan_destroy(ft_plan p) {
     if (p->d_tw) cudaFree(p->d_tw);
     if (p->d_chirp) cudaFree(p->d_chirp);
     if (p->d_tc_err) cudaFree(p->d_tc_err);
-    if (p->d_peak_state) cudaFree(p->d_peak_state);
     if (p->d_img_host) cudaFree(p->d_img_host);
     if (p->d_map_host) cudaFree(p->d_map_host);
     if (p->d_peaks_host) cudaFree(p->d_peaks_host);
@@ -638,6 +637,7 @@ static bool tc_columns(ft_plan p);
 // (ft_batch) always take it, as does the pipeline of ft_detect_batches, which hides
 // it.  FT_PEAKS=sparse / dense / multi at plan creation fixes the choice.
 static int peak_pass(ft_plan p, int batch, int top_k, bool with_tile_max, bool multi_ok) {
+    if (batch > FT_MULTI_MAX_BATCH) multi_ok = false;
     if (p->peak_mode) return p->peak_mode == FT_PASS_MULTI && !multi_ok ? FT_PASS_SPARSE : p->peak_mode;
     const double cells = (double)p->Hp * p->S, tiles = cells / 256.0;
     const int waves = (batch + p->num_sms - 1) / p->num_sms;
@@ -683,12 +683,20 @@ static size_t peaks_scratch_bytes(ft_plan p, int batch, int top_k) {
 static size_t tmax_bytes(ft_plan p, int batch, int bands, int cols) {
     return al256((size_t)batch * bands * ((p->S + cols - 1) / cols) * sizeof(unsigned));
 }
-static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_ok) {
-    int rows, cols, bands;
-    const int pass = detect_pass(p, batch, top_k, multi_ok, &rows, &cols, &bands);
+static size_t pass_scratch_bytes(ft_plan p, int batch, int pass, int bands, int cols) {
     if (!pass) return 0;
     return tmax_bytes(p, batch, bands, cols) +
            (pass == FT_PASS_MULTI ? peak_multi_scratch_bytes(bands * ((p->S + cols - 1) / cols), batch) : 0);
+}
+static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_ok) {
+    int rows, cols, bands;
+    const int pass = detect_pass(p, batch, top_k, multi_ok, &rows, &cols, &bands);
+    return pass_scratch_bytes(p, batch, pass, bands, cols);
+}
+
+// the buffers of ft_detect's pass are there from earlier calls
+static bool pass_ready(ft_plan p, int batch, int pass, int bands, int cols) {
+    return aux_off(p, batch) + pass_scratch_bytes(p, batch, pass, bands, cols) <= p->ws_bytes;
 }
 
 int ft_detect_launches(ft_plan p, int batch, int top_k) {
@@ -847,14 +855,23 @@ ft_status ft_peaks(ft_plan p, const float* d_map, int batch, int top_k, float th
     // where that pass does not fit.  Scratch after the spectrum workspace.
     int tr, tc;
     tile_max_shape(&tr, &tc);
-    const bool sparse = peaks_use_tile_max(p, batch, top_k);
+    bool sparse = peaks_use_tile_max(p, batch, top_k);
     const size_t tpi = (size_t)((p->Hp + tr - 1) / tr) * ((p->S + tc - 1) / tc);     // tiles per map
     const size_t off = aux_off(p, batch);
-    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + peaks_scratch_bytes(p, batch, top_k), "cudaMalloc(workspace)");
+    cudaStream_t st = (cudaStream_t)stream;
+    size_t scratch = peaks_scratch_bytes(p, batch, top_k);
+    if (off + scratch > p->ws_bytes && capturing(st)) {
+        // the other pass where its scratch is there from earlier calls
+        const size_t other = sparse ? peaks_key_bytes(p->Hp, p->S, batch, top_k) : tile_max_bytes(p, batch);
+        if ((sparse || peak_sparse_fits(tr, tc, top_k)) && off + other <= p->ws_bytes) {
+            sparse = !sparse;
+            scratch = other;
+        }
+    }
+    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + scratch, "cudaMalloc(workspace)");
     if (s != FT_OK) return s;
     unsigned* tmax = (unsigned*)((char*)p->d_ws + off);
     unsigned long long* kbuf = (unsigned long long*)((char*)p->d_ws + off);
-    cudaStream_t st = (cudaStream_t)stream;
     unsigned* bounds = peaks_bounds(kbuf, p->Hp, p->S, batch, top_k);
     const size_t kpi = peaks_tile_keys(p->Hp, p->S, top_k);
     const int lanes = use_lanes(p, batch) ? FT_LANES : 1;
@@ -894,21 +911,21 @@ ft_status ft_detect(ft_plan p, const float* d_img, float* d_map, int batch, int 
     if (!d_img || !d_map || !d_out || !d_count || ((uintptr_t)d_img & 7) || ((uintptr_t)d_map & 7))
         return FT_ERR_INVALID_ARG;
     int rows, cols, bands;
-    const int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
+    cudaStream_t st = (cudaStream_t)stream;
+    int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
+    // the choice depends on the batch and top_k, so a call being captured may ask for
+    // buffers that the calls before it did not: it takes a pass that has them
+    if (pass == FT_PASS_MULTI && !pass_ready(p, batch, pass, bands, cols) && capturing(st)) pass = FT_PASS_SPARSE;
+    if (pass == FT_PASS_SPARSE && !pass_ready(p, batch, pass, bands, cols) && capturing(st)) pass = 0;
     if (!pass) {
         const ft_status s = ft_forward(p, d_img, d_map, batch, stream);
         return s != FT_OK ? s : ft_peaks(p, d_map, batch, top_k, threshold, d_out, d_count, stream);
     }
     // the tile maxima [batch][bands][column blocks] live in the aux region
     const size_t off = aux_off(p, batch);
-    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + detect_scratch_bytes(p, batch, top_k, true),
+    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + pass_scratch_bytes(p, batch, pass, bands, cols),
                          "cudaMalloc(workspace)");
     if (s != FT_OK) return s;
-    if (pass == FT_PASS_MULTI &&
-        (s = zeroed(p, &p->d_peak_state, &p->peak_state_bytes, peak_multi_state_bytes(batch), (cudaStream_t)stream,
-                    "cudaMalloc(peak state)")) != FT_OK)
-        return s;
-    cudaStream_t st = (cudaStream_t)stream;
     float2* ws = (float2*)p->d_ws;
     unsigned* tmax = (unsigned*)((char*)p->d_ws + off);
     const float* src = d_img;
@@ -946,7 +963,8 @@ ft_status ft_detect_batches(ft_plan p, const float* const* d_imgs, int nb, int b
     // the pipeline needs step 1 on the fixed-length kernel right after the peak
     // pass from tile maxima; otherwise one ft_detect per batch
     const bool pipe = p->pdl && p->use_fast_y && !tc_columns(p) && p->space != FT_SPACE_INVERSE &&
-                      detect_pass(p, batch, top_k, false, &rows, &cols, &bands) == FT_PASS_SPARSE;
+                      detect_pass(p, batch, top_k, false, &rows, &cols, &bands) == FT_PASS_SPARSE &&
+                      (pass_ready(p, batch, FT_PASS_SPARSE, bands, cols) || !capturing((cudaStream_t)stream));
     if (!pipe) {
         for (int j = 0; j < nb; ++j) {
             const ft_status s = ft_detect(p, d_imgs[j], d_map, batch, top_k, threshold, d_out + j * recs,
@@ -1108,8 +1126,8 @@ ft_status ft_detect_host(ft_plan p, const float* h_img, int batch, int top_k, fl
         if (peaks_key_bytes(p->Hp, p->S, nb, top_k) > peak_b) peak_b = peaks_key_bytes(p->Hp, p->S, nb, top_k);
         if (aux_off(p, nb) + peak_b > need) need = aux_off(p, nb) + peak_b;
     }
-    if ((s = ensure(p, &p->d_ws, &p->ws_bytes, need, "cudaMalloc(workspace)")) != FT_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
+    if ((s = ensure(p, &p->d_ws, &p->ws_bytes, need, "cudaMalloc(workspace)")) != FT_OK) return s;
     FT_CUDA(cudaEventRecord(p->start_event, st), "event");
     FT_CUDA(cudaStreamWaitEvent(p->copy_stream, p->start_event, 0), "copy stream wait");
     for (int c = 0; c < nchunks; ++c) {

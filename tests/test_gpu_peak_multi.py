@@ -83,3 +83,29 @@ def test_multi_list_overflow(torch, monkeypatch):
     a = _detect(torch, monkeypatch, "multi", H, W, W, H, 1024, float("-inf"), x, calls=2)
     b = _detect(torch, monkeypatch, "sparse", H, W, W, H, 1024, float("-inf"), x)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+
+
+def test_capture_without_the_pass_buffers(torch, monkeypatch):
+    """The pass depends on the batch and K.  A call captured into a graph after
+    calls that took another pass cannot allocate what its own pass would want: it
+    takes one whose buffers are there, with the same records."""
+    monkeypatch.delenv("FT_PEAKS", raising=False)
+    from paper_1904_09409_gb300 import funnel as f
+    n, N, K = 16, 1024, 200
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((n, N, N), generator=g, device="cuda")
+    with f.Plan(N, N, N, N) as plan, f.Plan(N, N, N, N) as fresh:
+        assert f.ft_detect_launches(plan, n, 8) == 4 and f.ft_detect_launches(plan, n, K) == 5
+        m = torch.empty_like(x)
+        out = torch.zeros(n * K * f.PEAK_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+        f.ft_detect(plan, x, m, 8)                       # one block per image: no buffers of the other pass
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            f.ft_detect(plan, x, m, K, out=out, count=cnt)
+        graph.replay()
+        m2 = torch.empty_like(x)
+        out2, cnt2 = f.ft_detect(fresh, x, m2, K)
+        torch.cuda.synchronize()
+    assert torch.equal(m, m2) and torch.equal(cnt, cnt2) and torch.equal(out, out2)
