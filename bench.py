@@ -350,7 +350,7 @@ def varlen_images(pool, shapes):
 
 def time_varlen(f, imgs, shapes, steps, dev):
     """512 mixed-size images (H, W from {128 ... 2048}), forward + top-32 peaks:
-    the grouped kernels (one launch per stage over every image, work queues)
+    the grouped kernels (one launch per stage over every image)
     after autotuning, in one captured graph; returns the JSON record with the
     tuner's table and per-size throughput (each shape alone, as a batch of its
     own with the chosen configuration)."""
@@ -413,7 +413,7 @@ def time_varlen(f, imgs, shapes, steps, dev):
             "per_size_mpx_s": per,
             "workload": "512 images, H and W i.i.d. from {128,192,256,384,512,768,1024,1536,2048}, content as "
                         "the 1024^2 batch, maps H x W, top-32; forward + peaks of every image in the grouped "
-                        "kernels (one persistent launch per stage, device work queues), one CUDA graph launch, "
+                        "kernels (one launch per stage, a block per item), one CUDA graph launch, "
                         "threads per block chosen by the autotuner (tune_ms: r2c/rows/c2r -> ms); per-size "
                         "figures are each shape's images, repeated to >= 16 Mpx, as a batch of their own"}
 

@@ -150,8 +150,10 @@ ft_status ft_peaks(ft_plan plan, const float* d_map, int batch, int top_k, float
  * peak pass reads only the tiles whose maximum can reach the top_k: a peak
  * never exceeds its tile's maximum, so once top_k peaks are known, tiles below
  * the top_k-th value cannot contribute; the list is the same as ft_peaks'
- * (Sec. 4.4; checked equal element by element).  4 launches then (5 in the
- * inverse space), else those of ft_forward and ft_peaks.  threshold must not be
+ * (Sec. 4.4; checked equal element by element).  4 launches then, or 5 where the
+ * model expects the peak pass to be faster spread over the whole GPU (FT_PEAKS=multi
+ * at plan creation fixes that), one more in the inverse space; else those of
+ * ft_forward and ft_peaks.  threshold must not be
  * NaN (FT_ERR_INVALID_ARG, as for ft_peaks). */
 ft_status ft_detect(ft_plan plan, const float* d_img, float* d_map, int batch, int top_k, float threshold,
                     ft_peak* d_out, int32_t* d_count, void* stream);
@@ -204,8 +206,9 @@ ft_status ft_abs_mse_backward(ft_plan plan, const float* d_map, const float* d_t
  * plan-owned device buffer, runs ft_detect (ft_forward and ft_peaks), copies the peaks and
  * counts back to h_out ([batch][top_k]) and h_count ([batch]) and synchronises
  * `stream` before returning.  The batch is processed in chunks of about 24 MiB of
- * images (at least one image): a plan-owned copy stream uploads the next chunk while `stream` transforms the
- * current one (pinned h_img lets the copies run asynchronously). */
+ * images (at least one image): a plan-owned copy stream uploads the next chunk
+ * while `stream` transforms the current one (pinned h_img lets the copies run
+ * asynchronously). */
 ft_status ft_detect_host(ft_plan plan, const float* h_img, int batch, int top_k, float threshold,
                          ft_peak* h_out, int32_t* h_count, void* stream);
 

@@ -6,8 +6,8 @@
 // together (largest first).  Images whose sides both have a fixed-length
 // schedule up to 2048 (128, 192, 256, 384, 512, 768, 1024, 1536, 2048) with the
 // linear or cubic interpolator run in the grouped kernels of k_batch.cu: one
-// persistent launch per stage over all of them (step 1, steps 2-3, step 4 with
-// tile maxima, the peak pass), one block per (image, block) item, with the batch's own
+// launch per stage over all of them (step 1, steps 2-3, step 4 with tile maxima,
+// the peak pass), one block per (image, block) item, with the batch's own
 // workspace.  Every other shape group keeps a plan of its own (tables and
 // workspace) and runs its ft_detect on one of up to FT_BATCH_MAX_STREAMS side
 // streams forked from and joined back into the caller's stream.  With
