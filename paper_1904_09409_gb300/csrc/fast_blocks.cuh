@@ -199,6 +199,7 @@ __device__ __forceinline__ void c2r_from_stage(float2* sm, int ncols, const floa
     }
     __syncthreads();
     F::template run<0>(v, sm, t, f, stw);
+    if constexpr (!c2r_tiles(N)) tmax = nullptr;
     if constexpr (WARPTILES) {
         if (tmax) {
             // Tile maxima of |map| for the peak pass: thread t holds rows t + T j,

@@ -5,8 +5,8 @@
 
 #include "fft_fast.cuh"
 
-#define FT_FAST_POW2(X) X(128) X(256) X(512) X(1024) X(2048) X(4096) X(8192) X(192) X(384) X(768) X(1536)
-#define FT_FAST_SMALL3(X) X(144) X(162) X(216) X(288) X(324) X(432) X(486) X(576)
+#define FT_FAST_POW2(X) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096) X(8192) X(192) X(384) X(768) X(1536)
+#define FT_FAST_SMALL3(X) X(72) X(96) X(108) X(144) X(162) X(216) X(288) X(324) X(432) X(486) X(576)
 #define FT_FAST_MID3(X) X(648) X(864) X(972) X(1152) X(1296) X(1458) X(1728) X(1944)
 #define FT_FAST_LARGE3(X) X(2304) X(2592) X(2916) X(3072) X(3456) X(3888)
 #define FT_FAST_LENGTHS(X) FT_FAST_POW2(X) FT_FAST_SMALL3(X) FT_FAST_MID3(X) FT_FAST_LARGE3(X)

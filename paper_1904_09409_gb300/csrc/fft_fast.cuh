@@ -40,12 +40,19 @@
 // 1296 as 6 6 6 6 with E = 12 against 12 12 9 with E = 36, which spills, the same
 // forward and a faster adjoint (50 against 58).  192, 384, 768 and 1536 start with
 // radix 12 and save a pass against radix 4 passes and a last radix 3 (384^2 40 / 42 /
-// 34 -> 37 / 35 / 32, 1536^2 51 / 41 / 49 -> 47 / 40 / 45).
+// 34 -> 37 / 35 / 32, 1536^2 51 / 41 / 49 -> 47 / 40 / 45).  The shortest, against the
+// generic kernels: 64^2 26 / 31 / 26 (65 / 141 / 54; as 16 4 with E = 16 26 / 37 / 24),
+// 72^2 33 / 35 / 37 (90 / 144 / 78), 96^2 26 / 35 / 29 (67 / 138 / 56; as 12 4 2 32 / 37 /
+// 33), 108^2 28 / 35 / 31 (85 / 142 / 74; as 12 3 3 33 / 43 / 34).
 struct FsSched {
     int N, E, nst, r[6];
 };
 __host__ __device__ constexpr FsSched fs_sched(int N) {
     switch (N) {
+        case 64: return {64, 8, 2, {8, 8}};
+        case 72: return {72, 12, 2, {12, 6}};
+        case 96: return {96, 24, 2, {24, 4}};
+        case 108: return {108, 18, 2, {18, 6}};
         case 128: return {128, 16, 2, {16, 8}};
         case 144: return {144, 12, 2, {12, 12}};
         case 162: return {162, 18, 2, {18, 9}};
@@ -459,6 +466,11 @@ cudaError_t launch_col_c2r_fast(const float2* in, int ncols, int in_pitch, size_
 // cells, bands = N / rows tiles per column block; false without a schedule.
 // A tile is 256 cells: 128 / B rows of one column block of 2B columns (the last
 // band of a length that the rows do not divide is ragged).
+// Maps of fewer than 128 rows have none: ft_detect keeps ft_forward and ft_peaks there,
+// whose tiles are 16 x 16 instead of 4 x 64 (detection, us, with tiles from step 4 /
+// from a pass of their own: 96x486 x 8 30.6 / 27.9, 96^2 x 64 30.2 / 26.9, 64^2 x 64
+// 19.9 / 21.1, 108x4096 x 16 49.4 / 53.6).
+__host__ __device__ constexpr bool c2r_tiles(int N) { return N >= 128; }
 __host__ __device__ constexpr int c2r_tile_rows(int N) { return 128 / fs_Bc2r(N); }
 __host__ __device__ constexpr int c2r_tile_bands(int N) { return (N + c2r_tile_rows(N) - 1) / c2r_tile_rows(N); }
 bool c2r_tile_shape(int N, int* rows, int* cols, int* bands);

@@ -62,6 +62,7 @@ cudaError_t launch_col_c2r_fast(const float2* in, int ncols, int in_pitch, size_
 }
 
 bool c2r_tile_shape(int N, int* rows, int* cols, int* bands) {
+    if (!c2r_tiles(N)) return false;
     switch (N) {
 #define X(n) case n: *rows = c2r_tile_rows(n); *cols = 2 * fs_Bc2r(n); *bands = c2r_tile_bands(n); return true;
         FT_FAST_LENGTHS(X)

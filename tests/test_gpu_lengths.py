@@ -1,7 +1,7 @@
-"""The fixed-length kernels of the lengths 2^a 3^b with wide radices (6 to 36):
-every length as both map sides, with ragged images (odd height, so an uneven
-expansion, and W < S), against the generic kernels of the same plan and, where
-it is quick, the FP64 oracle.
+"""The fixed-length kernels of the lengths 2^a 3^b with wide radices (6 to 36) and of
+the shortest lengths: every length as both map sides, with ragged images (odd
+height, so an uneven expansion, and W < S), against the generic kernels of the
+same plan and, where it is quick, the FP64 oracle.
 
 Tolerances: a forward or adjoint map of these sizes is within 1e-6 of FP64 by
 FP32 rounding alone (three FFTs of at most 6 passes, a few eps each in the
@@ -16,6 +16,7 @@ from tests import _gpu
 
 pytestmark = pytest.mark.gpu
 
+SHORT = [64, 72, 96, 108]
 WIDE = [144, 162, 216, 288, 324, 432, 486, 576, 648, 864, 972, 1152, 1296, 1458, 1728, 1944,
         2304, 2592, 2916, 3072, 3456, 3888]
 
@@ -40,7 +41,7 @@ def _all_results(f, torch, plan, x, g, target):
 
 
 @pytest.mark.parametrize("interp", ["linear", "cubic"])
-@pytest.mark.parametrize("N", WIDE)
+@pytest.mark.parametrize("N", SHORT + WIDE)
 def test_wide_length_matches_generic_kernels_and_oracle(torch, N, interp):
     from paper_1904_09409_gb300 import funnel as f
     H, W, n = N - 5, N - (6 if N % 4 else 2), 2
