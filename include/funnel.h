@@ -144,8 +144,8 @@ ft_status ft_peaks(ft_plan plan, const float* d_map, int batch, int top_k, float
 /* Detection on device buffers: ft_forward (d_img -> d_map) followed by ft_peaks
  * on d_map, with the same arguments, layouts, rules and results (d_map holds
  * the map afterwards).  Where step 4 runs the fixed-length FP32 kernel on the
- * caller's stream (n_intercept with a fixed-length schedule, FP32 precision, no
- * lanes) and ft_peaks' cost model prefers the pass from tile maxima, step 4 also
+ * caller's stream (n_intercept with a fixed-length schedule, 128 or more, FP32
+ * precision, no lanes) and ft_peaks' cost model prefers the pass from tile maxima, step 4 also
  * writes the maximum of |P| of every 256-cell tile of its output and the
  * peak pass reads only the tiles whose maximum can reach the top_k: a peak
  * never exceeds its tile's maximum, so once top_k peaks are known, tiles below
