@@ -36,7 +36,7 @@
 #include "peak_sparse_block.cuh"
 
 #define PM_CAP 65536        // keys per image of the candidate list
-#define PM_BINS 8192        // |P| bits >> 18: exponent (8) and 5 mantissa bits
+#define PM_BINS 8192        // |P| bits >> 18 (no sign bit): exponent (8) and 5 mantissa bits
 #define PM_THREADS 1024
 
 struct PmState {            // per image, zero between calls
@@ -68,7 +68,9 @@ k_peak_bound(const unsigned* __restrict__ tmax, int nty, int ntx, int K, float t
     bool is = false;
     unsigned v = 0u;
     if (i < ntiles) {
-        v = tm[i];
+        // a maximum of |P| has no sign bit; what a step 4 whose wait ran out left
+        // unwritten may have one, and would fall outside the histogram's bins
+        v = tm[i] & 0x7fffffffu;
         if (__uint_as_float(v) >= thr) {
             const int ty = i / ntx, tx = i - ty * ntx;
             const int up = (ty == 0 ? nty - 1 : ty - 1) * ntx, dn = (ty == nty - 1 ? 0 : ty + 1) * ntx, mid = ty * ntx;
