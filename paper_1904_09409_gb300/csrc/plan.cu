@@ -650,14 +650,15 @@ static int peak_pass(ft_plan p, int batch, int top_k, bool with_tile_max, bool m
     return sparse < dense ? FT_PASS_SPARSE : FT_PASS_DENSE;
 }
 
-// The pass ft_detect runs on the tile maxima that step 4 writes (FT_PASS_SPARSE or
-// FT_PASS_MULTI, the tiles' shape in *rows, *cols, *bands), or 0 when it runs
-// ft_forward and ft_peaks instead.  multi_ok: FT_PASS_MULTI may be chosen.
+// The pass ft_detect is expected to be fastest with: FT_PASS_SPARSE or FT_PASS_MULTI
+// on the tile maxima that step 4 writes, FT_PASS_DENSE for ft_forward and ft_peaks
+// (the tiles' shape in *rows, *cols, *bands), or 0 when step 4 can write no tile
+// maxima, so that only ft_forward and ft_peaks remain.  multi_ok: FT_PASS_MULTI may
+// be chosen.
 static int detect_pass(ft_plan p, int batch, int top_k, bool multi_ok, int* rows, int* cols, int* bands) {
     if (!p->use_fast_y || tc_columns(p) || use_lanes(p, batch)) return 0;
     if (!c2r_tile_shape(p->Hp, rows, cols, bands) || !peak_sparse_fits(*rows, *cols, top_k)) return 0;
-    const int pass = peak_pass(p, batch, top_k, false, multi_ok);
-    return pass == FT_PASS_DENSE ? 0 : pass;
+    return peak_pass(p, batch, top_k, false, multi_ok);
 }
 
 // ft_peaks takes the pass from tile maxima (tiles of tile_max_shape)
@@ -684,7 +685,7 @@ static size_t tmax_bytes(ft_plan p, int batch, int bands, int cols) {
     return al256((size_t)batch * bands * ((p->S + cols - 1) / cols) * sizeof(unsigned));
 }
 static size_t pass_scratch_bytes(ft_plan p, int batch, int pass, int bands, int cols) {
-    if (!pass) return 0;
+    if (pass != FT_PASS_SPARSE && pass != FT_PASS_MULTI) return 0;
     return tmax_bytes(p, batch, bands, cols) +
            (pass == FT_PASS_MULTI ? peak_multi_scratch_bytes(bands * ((p->S + cols - 1) / cols), batch) : 0);
 }
@@ -695,15 +696,18 @@ static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_o
 }
 
 // the buffers of ft_detect's pass are there from earlier calls
-static bool pass_ready(ft_plan p, int batch, int pass, int bands, int cols) {
-    return aux_off(p, batch) + pass_scratch_bytes(p, batch, pass, bands, cols) <= p->ws_bytes;
+static bool pass_ready(ft_plan p, int batch, int top_k, int pass, int bands, int cols) {
+    const size_t scratch = pass == FT_PASS_DENSE ? peaks_scratch_bytes(p, batch, top_k)
+                                                 : pass_scratch_bytes(p, batch, pass, bands, cols);
+    return aux_off(p, batch) + scratch <= p->ws_bytes;
 }
 
 int ft_detect_launches(ft_plan p, int batch, int top_k) {
     if (!p || batch <= 0 || top_k < 1 || top_k > FT_MAX_TOPK) return 0;
     int rows, cols, bands;
     const int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
-    if (pass) return (p->space == FT_SPACE_INVERSE ? 1 : 0) + (pass == FT_PASS_MULTI ? 5 : 4);
+    if (pass == FT_PASS_SPARSE || pass == FT_PASS_MULTI)
+        return (p->space == FT_SPACE_INVERSE ? 1 : 0) + (pass == FT_PASS_MULTI ? 5 : 4);
     return ft_forward_launches(p, batch) + ft_peaks_launches(p, batch);
 }
 
@@ -913,11 +917,13 @@ ft_status ft_detect(ft_plan p, const float* d_img, float* d_map, int batch, int 
     int rows, cols, bands;
     cudaStream_t st = (cudaStream_t)stream;
     int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
-    // the choice depends on the batch and top_k, so a call being captured may ask for
-    // buffers that the calls before it did not: it takes a pass that has them
-    if (pass == FT_PASS_MULTI && !pass_ready(p, batch, pass, bands, cols) && capturing(st)) pass = FT_PASS_SPARSE;
-    if (pass == FT_PASS_SPARSE && !pass_ready(p, batch, pass, bands, cols) && capturing(st)) pass = 0;
-    if (!pass) {
+    // the choice depends on the batch and top_k, so a call being captured, which cannot
+    // allocate, may want buffers that the calls before it did not: then the tile maxima
+    // of step 4, which every call on them leaves room for, else ft_peaks, which looks
+    // for the buffers of either of its passes
+    if (pass && !pass_ready(p, batch, top_k, pass, bands, cols) && capturing(st))
+        pass = pass_ready(p, batch, top_k, FT_PASS_SPARSE, bands, cols) ? FT_PASS_SPARSE : FT_PASS_DENSE;
+    if (pass != FT_PASS_SPARSE && pass != FT_PASS_MULTI) {
         const ft_status s = ft_forward(p, d_img, d_map, batch, stream);
         return s != FT_OK ? s : ft_peaks(p, d_map, batch, top_k, threshold, d_out, d_count, stream);
     }
@@ -964,7 +970,7 @@ ft_status ft_detect_batches(ft_plan p, const float* const* d_imgs, int nb, int b
     // pass from tile maxima; otherwise one ft_detect per batch
     const bool pipe = p->pdl && p->use_fast_y && !tc_columns(p) && p->space != FT_SPACE_INVERSE &&
                       detect_pass(p, batch, top_k, false, &rows, &cols, &bands) == FT_PASS_SPARSE &&
-                      (pass_ready(p, batch, FT_PASS_SPARSE, bands, cols) || !capturing((cudaStream_t)stream));
+                      (pass_ready(p, batch, top_k, FT_PASS_SPARSE, bands, cols) || !capturing((cudaStream_t)stream));
     if (!pipe) {
         for (int j = 0; j < nb; ++j) {
             const ft_status s = ft_detect(p, d_imgs[j], d_map, batch, top_k, threshold, d_out + j * recs,

@@ -1,0 +1,60 @@
+"""ft_detect where the buffers of the pass that its cost model prefers are not
+there: a call captured into a graph, which can allocate nothing, takes a pass whose
+buffers earlier calls left, with the same records.
+"""
+import pytest
+
+from tests import _gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    return _gpu.torch_cuda()
+
+
+# (image H, W, n_slope, n_intercept, space, batch and top_k of the call before, batch
+# and top_k of the captured call)
+CAPTURED = [
+    # 32 x 8 tiles from step 4, fewer bytes than the 16 x 16 tiles of ft_peaks: the
+    # captured call prefers the per-tile keys, then a smaller batch that does
+    (768, 648, 648, 768, "regular", 8, 8, 8, 200),
+    (768, 648, 648, 768, "regular", 16, 8, 4, 300),
+    # the same map of the inverse space
+    (648, 768, 648, 768, "inverse", 8, 8, 8, 200),
+    # equal tile counts; the keys' buffers first, then tile maxima
+    (480, 640, 648, 486, "regular", 8, 8, 8, 100),
+    (768, 648, 648, 768, "regular", 8, 200, 8, 8),
+    # whole-GPU pass first, the one-block pass or the keys captured
+    (1024, 1024, 1024, 1024, "regular", 4, 200, 4, 8),
+    (1024, 1024, 1024, 1024, "regular", 4, 100, 4, 1000),
+]
+
+
+@pytest.mark.parametrize("H,W,S,Hp,space,b0,k0,b1,k1", CAPTURED)
+@pytest.mark.parametrize("call", ["ft_detect", "ft_detect_batches"])
+def test_captured_call_takes_buffers_of_earlier_ones(torch, monkeypatch, H, W, S, Hp, space, b0, k0, b1, k1, call):
+    monkeypatch.delenv("FT_PEAKS", raising=False)
+    from paper_1904_09409_gb300 import funnel as f
+    g = torch.Generator(device="cuda").manual_seed(H + k1)
+    x = torch.randn((b0, H, W), generator=g, device="cuda")
+    m = torch.empty((b0, Hp, S), device="cuda")
+    out = torch.zeros(b1 * k1 * f.PEAK_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    cnt = torch.zeros(b1, dtype=torch.int32, device="cuda")
+    xs = x[:b1].contiguous()
+    with f.Plan(H, W, S, Hp, space=space) as plan, f.Plan(H, W, S, Hp, space=space) as fresh:
+        f.ft_detect(plan, x, m, k0)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            if call == "ft_detect":
+                f.ft_detect(plan, xs, m, k1, out=out, count=cnt, batch=b1)
+            else:
+                f.ft_detect_batches(plan, [xs], m, k1, out=out, count=cnt)
+        m.fill_(float("nan"))
+        graph.replay()
+        m2 = torch.empty((b1, Hp, S), device="cuda")
+        out2, cnt2 = f.ft_detect(fresh, xs, m2, k1)
+        torch.cuda.synchronize()
+    assert torch.equal(m[:b1], m2) and torch.equal(cnt, cnt2) and torch.equal(out, out2)
