@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -679,14 +680,16 @@ static size_t peaks_scratch_bytes(ft_plan p, int batch, int top_k) {
     return peaks_use_tile_max(p, batch, top_k) ? tile_max_bytes(p, batch) : peaks_key_bytes(p->Hp, p->S, batch, top_k);
 }
 
-// bytes of ft_detect's tile maxima for this batch, and with the scratch of the pass
-// over the whole GPU (0 when it runs ft_peaks)
+// bytes of ft_detect's tile maxima for this batch, and of its scratch: those or the
+// 16 x 16 tiles of ft_peaks, if they are more (so that a later ft_peaks of the same
+// batch has its buffer, also under capture), and that of the pass over the whole GPU
+// (0 when it runs ft_peaks)
 static size_t tmax_bytes(ft_plan p, int batch, int bands, int cols) {
     return al256((size_t)batch * bands * ((p->S + cols - 1) / cols) * sizeof(unsigned));
 }
 static size_t pass_scratch_bytes(ft_plan p, int batch, int pass, int bands, int cols) {
     if (pass != FT_PASS_SPARSE && pass != FT_PASS_MULTI) return 0;
-    return tmax_bytes(p, batch, bands, cols) +
+    return std::max(tmax_bytes(p, batch, bands, cols), al256(tile_max_bytes(p, batch))) +
            (pass == FT_PASS_MULTI ? peak_multi_scratch_bytes(bands * ((p->S + cols - 1) / cols), batch) : 0);
 }
 static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_ok) {

@@ -58,3 +58,27 @@ def test_captured_call_takes_buffers_of_earlier_ones(torch, monkeypatch, H, W, S
         out2, cnt2 = f.ft_detect(fresh, xs, m2, k1)
         torch.cuda.synchronize()
     assert torch.equal(m[:b1], m2) and torch.equal(cnt, cnt2) and torch.equal(out, out2)
+
+
+@pytest.mark.parametrize("H,W,Hp,n,k0,k1", [(150, 3888, 162, 1, 14, 5),    # 4 x 64 tiles of step 4: 2501, 16 x 16: 2673
+                                            (2500, 2, 2592, 9, 23, 44)])   # 32 x 8 tiles of step 4: 81, 16 x 16: 162
+def test_captured_peaks_after_detect(torch, monkeypatch, H, W, Hp, n, k0, k1):
+    """ft_peaks captured after ft_detect calls alone, at lengths whose tiles in step 4
+    are fewer than those of ft_peaks."""
+    monkeypatch.delenv("FT_PEAKS", raising=False)
+    from paper_1904_09409_gb300 import funnel as f
+    g = torch.Generator(device="cuda").manual_seed(Hp)
+    x = torch.randn((n, H, W), generator=g, device="cuda")
+    m = torch.empty((n, Hp, W), device="cuda")
+    out = torch.zeros(n * k1 * f.PEAK_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+    with f.Plan(H, W, W, Hp) as plan, f.Plan(H, W, W, Hp) as fresh:
+        f.ft_detect(plan, x, m, k0)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            f.ft_peaks(plan, m, k1, out=out, count=cnt)
+        graph.replay()
+        out2, cnt2 = f.ft_peaks(fresh, m, k1)
+        torch.cuda.synchronize()
+    assert torch.equal(cnt, cnt2) and torch.equal(out, out2)
