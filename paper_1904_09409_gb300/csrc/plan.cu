@@ -837,8 +837,14 @@ ft_status ft_abs_mse_backward(ft_plan p, const float* d_map, const float* d_targ
                   "loss");
         return ft_backward(p, gmap, d_grad_img, batch, stream);
     }
+    // the partials, and room for the small scratch of ft_abs_mse_grad and of a peak pass
+    // from tile maxima, so that these find their buffers under capture after this call
     const int nblk = col_r2c_loss_blocks(p->fy, p->S);
-    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + (size_t)batch * nblk * sizeof(float), "cudaMalloc(workspace)");
+    int rows = 0, cols = 0, bands = 0;
+    const bool tiles = c2r_tile_shape(p->Hp, &rows, &cols, &bands);
+    const size_t scratch = std::max({(size_t)batch * nblk * sizeof(float), loss_partial_bytes(batch), tile_max_bytes(p, batch),
+                                     tiles ? pass_scratch_bytes(p, batch, FT_PASS_SPARSE, bands, cols) : (size_t)0});
+    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + scratch, "cudaMalloc(workspace)");
     if (s != FT_OK) return s;
     float2* ws = (float2*)p->d_ws;
     float* partial = (float*)((char*)p->d_ws + off);

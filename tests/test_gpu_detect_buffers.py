@@ -82,3 +82,42 @@ def test_captured_peaks_after_detect(torch, monkeypatch, H, W, Hp, n, k0, k1):
         out2, cnt2 = f.ft_peaks(fresh, m, k1)
         torch.cuda.synchronize()
     assert torch.equal(cnt, cnt2) and torch.equal(out, out2)
+
+
+@pytest.mark.parametrize("H,W,Hp,S", [(150, 160, 162, 162), (480, 640, 486, 648), (70, 72, 72, 72)])
+@pytest.mark.parametrize("call", ["ft_detect", "ft_peaks", "ft_abs_mse_grad"])
+def test_captured_call_after_loss_backward(torch, monkeypatch, H, W, Hp, S, call):
+    """The calls that need little scratch find it under capture after
+    ft_abs_mse_backward alone, whichever way its columns run."""
+    monkeypatch.delenv("FT_PEAKS", raising=False)
+    from paper_1904_09409_gb300 import funnel as f
+    n, K = 3, 5
+    g = torch.Generator(device="cuda").manual_seed(S)
+    x = torch.randn((n, H, W), generator=g, device="cuda")
+    m = torch.randn((n, Hp, S), generator=g, device="cuda")
+    t = torch.rand((n, Hp, S), generator=g, device="cuda")
+    out = torch.zeros(n * K * f.PEAK_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    cnt = torch.zeros(n, dtype=torch.int32, device="cuda")
+    res = []
+    with f.Plan(H, W, S, Hp) as plan, f.Plan(H, W, S, Hp) as fresh:
+        f.ft_abs_mse_backward(plan, m, t, 0.5)
+        torch.cuda.synchronize()
+
+        def go(p):
+            if call == "ft_abs_mse_grad":
+                return f.ft_abs_mse_grad(p, m, t, 0.5)
+            if call == "ft_peaks":
+                f.ft_peaks(p, m, K, out=out, count=cnt)
+            else:
+                f.ft_detect(p, x, m, K, out=out, count=cnt)
+            return out, cnt
+
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            a = go(plan)
+        graph.replay()
+        torch.cuda.synchronize()
+        res = [v.clone() for v in a]
+        b = go(fresh)
+        torch.cuda.synchronize()
+    assert all(torch.equal(u, v) for u, v in zip(res, b))
