@@ -411,10 +411,10 @@ cudaError_t launch_peak_sparse(const float* map, const unsigned* tmax, int Hp, i
                                int batch, int top_k, float threshold, ft_peak* out, int32_t* count, cudaStream_t st,
                                bool pdl = false);
 // The same list again, two launches over the whole GPU (k_peak_multi.cu):
-// scratch of peak_multi_scratch_bytes(tiles per image, batch), and per-image
+// scratch of peak_multi_scratch_bytes(Hp, S, tiles per image, batch), and per-image
 // words of peak_multi_state_bytes(batch) that are zero before the first call and
 // that every call leaves so.
-size_t peak_multi_scratch_bytes(int ntiles, int batch);
+size_t peak_multi_scratch_bytes(int Hp, int S, int ntiles, int batch);
 #define FT_MULTI_MAX_BATCH 1024   // images per call (more of them fill the GPU with one block each)
 size_t peak_multi_state_bytes(int batch);
 cudaError_t launch_peak_multi(const float* map, const unsigned* tmax, int Hp, int S, int tile_rows, int tile_cols,

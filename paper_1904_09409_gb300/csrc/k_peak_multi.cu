@@ -33,9 +33,11 @@
 // works on what the others wrote (fence, then atomic); no block waits for another.
 // The words are zero before the first call and the last block to use one clears
 // it, so calls follow each other without a memset.
+#include <algorithm>
+
 #include "peak_sparse_block.cuh"
 
-#define PM_CAP 65536        // keys per image of the candidate list
+#define PM_CAP 65536        // keys per image of the candidate list, or all that a map can have
 #define PM_BINS 8192        // |P| bits >> 18 (no sign bit): exponent (8) and 5 mantissa bits
 #define PM_THREADS 1024
 
@@ -49,8 +51,10 @@ struct PmState {            // per image, zero between calls
 size_t peak_multi_state_bytes(int batch) { return (size_t)batch * sizeof(PmState); }
 
 static size_t pm_loc_cap(int ntiles) { return (size_t)ntiles / 4 + 1; }
-size_t peak_multi_scratch_bytes(int ntiles, int batch) {
-    return (size_t)batch * (PM_CAP * sizeof(u64) + pm_loc_cap(ntiles) * sizeof(unsigned));
+// a quarter of the cells at most are strict local maxima (a 2 x 2 block holds one)
+static int pm_cap(int Hp, int S) { return (int)std::min((size_t)PM_CAP, (size_t)Hp * S / 4); }
+size_t peak_multi_scratch_bytes(int Hp, int S, int ntiles, int batch) {
+    return (size_t)batch * (pm_cap(Hp, S) * sizeof(u64) + pm_loc_cap(ntiles) * sizeof(unsigned));
 }
 
 __global__ void __launch_bounds__(PM_THREADS)
@@ -143,7 +147,7 @@ k_peak_bound(const unsigned* __restrict__ tmax, int nty, int ntx, int K, float t
 
 __global__ void __launch_bounds__(PM_THREADS)
 k_peak_scan(const float* __restrict__ map, const unsigned* __restrict__ tmax, int Hp, int S, int TH, int logTW,
-            int nty, int ntx, int K, float thr, u64* __restrict__ cands, PmState* __restrict__ state,
+            int nty, int ntx, int K, float thr, u64* __restrict__ cands, int cap, PmState* __restrict__ state,
             ft_peak* __restrict__ out, int32_t* __restrict__ count) {
     extern __shared__ __align__(16) unsigned char spsm[];
     __shared__ SparseShared sh;
@@ -154,7 +158,7 @@ k_peak_scan(const float* __restrict__ map, const unsigned* __restrict__ tmax, in
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const float* m = map + (size_t)img * Hp * S;
     const unsigned* tm = tmax + (size_t)img * ntiles;
-    u64* cand = cands + (size_t)img * PM_CAP;
+    u64* cand = cands + (size_t)img * cap;
     PmState* st = state + img;
     const float bound = fmaxf(thr, __uint_as_float(st->bound));
     float* stg = reinterpret_cast<float*>(spsm) + (size_t)warp * (TH + 2) * ((1 << logTW) + 8);
@@ -184,7 +188,7 @@ k_peak_scan(const float* __restrict__ map, const unsigned* __restrict__ tmax, in
         for (int j = warp; j < nl; j += nw) {
             unsigned long long mask;
             const unsigned best = tester.test(list[j], bound, mask);
-            if (best) tester.append(list[j], bound, mask, cand, &st->ncand, PM_CAP);
+            if (best) tester.append(list[j], bound, mask, cand, &st->ncand, cap);
             __syncwarp();
         }
         __syncthreads();
@@ -202,7 +206,7 @@ k_peak_scan(const float* __restrict__ map, const unsigned* __restrict__ tmax, in
     __syncthreads();
     if (!last) return;
     const int n = sh.ncand;
-    if (n > PM_CAP) {
+    if (n > cap) {
         __syncthreads();
         peak_sparse_block(m, tm, Hp, S, TH, logTW, nty, ntx, K, thr, out + (size_t)img * K, count + img, spsm, sh);
         return;
@@ -245,7 +249,8 @@ cudaError_t launch_peak_multi(const float* map, const unsigned* tmax, int Hp, in
     const int nw = sparse_warps(tile_rows, tile_cols, top_k);
     if (nw == 0) return cudaErrorInvalidValue;
     u64* cands = static_cast<u64*>(scratch);
-    unsigned* loc = reinterpret_cast<unsigned*>(cands + (size_t)batch * PM_CAP);
+    const int cap = pm_cap(Hp, S);
+    unsigned* loc = reinterpret_cast<unsigned*>(cands + (size_t)batch * cap);
     PmState* ps = static_cast<PmState*>(state);
     cudaError_t e = launch_maybe_pdl(k_peak_bound, dim3((ntiles + PM_THREADS - 1) / PM_THREADS, batch),
                                      dim3(PM_THREADS), 0, st, pdl, tmax, nty, ntx, top_k, threshold, loc,
@@ -256,5 +261,5 @@ cudaError_t launch_peak_multi(const float* map, const unsigned* tmax, int Hp, in
     if (e != cudaSuccess) return e;
     // 256 tiles per block: one round of listing
     return launch_maybe_pdl(k_peak_scan, dim3((ntiles + 255) / 256, batch), dim3(nw * 32), sm, st, pdl, map, tmax, Hp,
-                            S, tile_rows, logTW, nty, ntx, top_k, threshold, cands, ps, out, count);
+                            S, tile_rows, logTW, nty, ntx, top_k, threshold, cands, cap, ps, out, count);
 }

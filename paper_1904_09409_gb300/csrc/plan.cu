@@ -200,6 +200,7 @@ static ft_status ensure(ft_plan p, void** ptr, size_t* have, size_t need, const 
         e = cudaMalloc(ptr, need);
     if (e != cudaSuccess) {
         *ptr = nullptr;
+        cudaGetLastError();                            // not the next launch's error
         cuda_fail(e, what);
         return FT_ERR_OOM;
     }
@@ -690,7 +691,7 @@ static size_t tmax_bytes(ft_plan p, int batch, int bands, int cols) {
 static size_t pass_scratch_bytes(ft_plan p, int batch, int pass, int bands, int cols) {
     if (pass != FT_PASS_SPARSE && pass != FT_PASS_MULTI) return 0;
     return std::max(tmax_bytes(p, batch, bands, cols), al256(tile_max_bytes(p, batch))) +
-           (pass == FT_PASS_MULTI ? peak_multi_scratch_bytes(bands * ((p->S + cols - 1) / cols), batch) : 0);
+           (pass == FT_PASS_MULTI ? peak_multi_scratch_bytes(p->Hp, p->S, bands * ((p->S + cols - 1) / cols), batch) : 0);
 }
 static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_ok) {
     int rows, cols, bands;
@@ -698,11 +699,13 @@ static size_t detect_scratch_bytes(ft_plan p, int batch, int top_k, bool multi_o
     return pass_scratch_bytes(p, batch, pass, bands, cols);
 }
 
-// the buffers of ft_detect's pass are there from earlier calls
+// the workspace of ft_detect's pass, and whether it is there from earlier calls
+static size_t pass_need(ft_plan p, int batch, int top_k, int pass, int bands, int cols) {
+    return aux_off(p, batch) + (pass == FT_PASS_DENSE ? peaks_scratch_bytes(p, batch, top_k)
+                                                      : pass_scratch_bytes(p, batch, pass, bands, cols));
+}
 static bool pass_ready(ft_plan p, int batch, int top_k, int pass, int bands, int cols) {
-    const size_t scratch = pass == FT_PASS_DENSE ? peaks_scratch_bytes(p, batch, top_k)
-                                                 : pass_scratch_bytes(p, batch, pass, bands, cols);
-    return aux_off(p, batch) + scratch <= p->ws_bytes;
+    return pass_need(p, batch, top_k, pass, bands, cols) <= p->ws_bytes;
 }
 
 int ft_detect_launches(ft_plan p, int batch, int top_k) {
@@ -882,6 +885,10 @@ ft_status ft_peaks(ft_plan p, const float* d_map, int batch, int top_k, float th
         }
     }
     ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + scratch, "cudaMalloc(workspace)");
+    if (s == FT_ERR_OOM && !sparse && peak_sparse_fits(tr, tc, top_k)) {
+        sparse = true;                                 // no memory for the keys: the maxima need less
+        s = ensure(p, &p->d_ws, &p->ws_bytes, off + tile_max_bytes(p, batch), "cudaMalloc(workspace)");
+    }
     if (s != FT_OK) return s;
     unsigned* tmax = (unsigned*)((char*)p->d_ws + off);
     unsigned long long* kbuf = (unsigned long long*)((char*)p->d_ws + off);
@@ -926,20 +933,28 @@ ft_status ft_detect(ft_plan p, const float* d_img, float* d_map, int batch, int 
     int rows, cols, bands;
     cudaStream_t st = (cudaStream_t)stream;
     int pass = detect_pass(p, batch, top_k, true, &rows, &cols, &bands);
-    // the choice depends on the batch and top_k, so a call being captured, which cannot
+    // The choice depends on the batch and top_k, so a call being captured, which cannot
     // allocate, may want buffers that the calls before it did not: then the tile maxima
     // of step 4, which every call on them leaves room for, else ft_peaks, which looks
-    // for the buffers of either of its passes
-    if (pass && !pass_ready(p, batch, top_k, pass, bands, cols) && capturing(st))
-        pass = pass_ready(p, batch, top_k, FT_PASS_SPARSE, bands, cols) ? FT_PASS_SPARSE : FT_PASS_DENSE;
+    // for the buffers of either of its passes.  A call without the memory for what it
+    // prefers also takes the tile maxima, the pass that needs the least.
+    ft_status s = FT_OK;
+    if (pass && !pass_ready(p, batch, top_k, pass, bands, cols)) {
+        if (capturing(st)) {
+            pass = pass_ready(p, batch, top_k, FT_PASS_SPARSE, bands, cols) ? FT_PASS_SPARSE : FT_PASS_DENSE;
+        } else {
+            s = ensure(p, &p->d_ws, &p->ws_bytes, pass_need(p, batch, top_k, pass, bands, cols), "cudaMalloc(workspace)");
+            if (s != FT_OK && pass == FT_PASS_SPARSE) return s;
+            if (s != FT_OK) pass = FT_PASS_SPARSE;
+        }
+    }
     if (pass != FT_PASS_SPARSE && pass != FT_PASS_MULTI) {
-        const ft_status s = ft_forward(p, d_img, d_map, batch, stream);
+        s = ft_forward(p, d_img, d_map, batch, stream);
         return s != FT_OK ? s : ft_peaks(p, d_map, batch, top_k, threshold, d_out, d_count, stream);
     }
     // the tile maxima [batch][bands][column blocks] live in the aux region
     const size_t off = aux_off(p, batch);
-    ft_status s = ensure(p, &p->d_ws, &p->ws_bytes, off + pass_scratch_bytes(p, batch, pass, bands, cols),
-                         "cudaMalloc(workspace)");
+    s = ensure(p, &p->d_ws, &p->ws_bytes, pass_need(p, batch, top_k, pass, bands, cols), "cudaMalloc(workspace)");
     if (s != FT_OK) return s;
     float2* ws = (float2*)p->d_ws;
     unsigned* tmax = (unsigned*)((char*)p->d_ws + off);

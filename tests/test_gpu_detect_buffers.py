@@ -1,6 +1,7 @@
 """ft_detect where the buffers of the pass that its cost model prefers are not
 there: a call captured into a graph, which can allocate nothing, takes a pass whose
-buffers earlier calls left, with the same records.
+buffers earlier calls left, and a call whose allocation fails the pass that needs the
+least, with the same records.
 """
 import pytest
 
@@ -121,3 +122,52 @@ def test_captured_call_after_loss_backward(torch, monkeypatch, H, W, Hp, S, call
         b = go(fresh)
         torch.cuda.synchronize()
     assert all(torch.equal(u, v) for u, v in zip(res, b))
+
+
+# the preferred passes: over the whole GPU, per-tile keys, tile maxima; ft_peaks with keys
+@pytest.mark.parametrize("call,H,W,n,K,more", [("ft_detect", 1024, 1024, 16, 200, True), ("ft_detect", 768, 648, 8, 200, True),
+                                               ("ft_detect", 1024, 1024, 16, 8, False), ("ft_peaks", 768, 648, 8, 200, True)])
+def test_failed_allocation_takes_the_pass_of_least_memory(torch, monkeypatch, call, H, W, n, K, more):
+    """One failed allocation of the preferred pass leaves the one from tile maxima; a
+    second one is the call's error, and the plan stays usable."""
+    monkeypatch.delenv("FT_PEAKS", raising=False)
+    from paper_1904_09409_gb300 import funnel as f
+    g = torch.Generator(device="cuda").manual_seed(K)
+    x = torch.randn((n, H, W), generator=g, device="cuda")
+    m = torch.empty_like(x)
+
+    def go(p):
+        return f.ft_detect(p, x, m, K) if call == "ft_detect" else f.ft_peaks(p, m, K)
+
+    with f.Plan(H, W, W, H) as plan, f.Plan(H, W, W, H) as fresh:
+        f.ft_forward(fresh, x, m)
+        want = go(fresh)
+        f.ft_plan_inject_alloc_failures(plan, 2 if more else 1)
+        with pytest.raises(f.FunnelError) as e:
+            go(plan)
+        assert e.value.status == f.FT_ERR_OOM
+        f.ft_plan_inject_alloc_failures(plan, 1 if more else 0)
+        a = go(plan)
+        b = go(plan)                                     # allocates what it prefers
+        torch.cuda.synchronize()
+    for u, v, w in zip(a, b, want):
+        assert torch.equal(u, w) and torch.equal(v, w)
+
+
+def test_scratch_of_the_pass_over_the_whole_gpu_follows_the_map(torch, monkeypatch):
+    """The candidate list of a small map holds the strict local maxima it can have (a
+    quarter of its cells): 256 maps of 64 x 128 take 4 MiB, not 65536 keys each (128 MiB)."""
+    monkeypatch.setenv("FT_PEAKS", "multi")
+    from paper_1904_09409_gb300 import funnel as f
+    n, H, W, K = 256, 128, 64, 4
+    x = torch.randn((n, H, W), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    m = torch.empty_like(x)
+    with f.Plan(H, W, W, H) as plan:
+        f.ft_detect(plan, x, m, K)                       # modules loaded, outputs in torch's pool
+    torch.cuda.synchronize()
+    with f.Plan(H, W, W, H) as plan:
+        assert f.ft_detect_launches(plan, n, K) == 5
+        free0 = torch.cuda.mem_get_info()[0]
+        f.ft_detect(plan, x, m, K)
+        used = free0 - torch.cuda.mem_get_info()[0]
+    assert used <= (32 << 20), used                      # 8 MiB of spectra, 4 of keys, allocation granules
