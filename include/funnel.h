@@ -206,9 +206,9 @@ ft_status ft_abs_mse_backward(ft_plan plan, const float* d_map, const float* d_t
  * plan-owned device buffer, runs ft_detect (ft_forward and ft_peaks), copies the peaks and
  * counts back to h_out ([batch][top_k]) and h_count ([batch]) and synchronises
  * `stream` before returning.  The batch is processed in chunks of about 24 MiB of
- * images (at least one image): a plan-owned copy stream uploads the next chunk
- * while `stream` transforms the current one (pinned h_img lets the copies run
- * asynchronously). */
+ * images (at least one image; no more than have 256 MiB of maps, or 8): a
+ * plan-owned copy stream uploads the next chunk while `stream` transforms the
+ * current one (pinned h_img lets the copies run asynchronously). */
 ft_status ft_detect_host(ft_plan plan, const float* h_img, int batch, int top_k, float threshold,
                          ft_peak* h_out, int32_t* h_count, void* stream);
 

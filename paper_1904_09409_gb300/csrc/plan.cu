@@ -19,9 +19,15 @@ static thread_local char g_last_error[256] = "";
 // upload of a chunk hides the previous chunk's transform, and only the last chunk's
 // transform is exposed, so chunks are as small as keeps the transform of one, which
 // is bound by launches and latency, shorter than its upload (24 MiB: 120 us).  From
-// pinned memory, us, against chunks of 8 images: 16 x 1024^2 460 -> 439 (with 8 MiB
-// 521, 32 MiB 453), 64 x 256^2 393 -> 175, 8 x 2048^2 922 -> 779, 2 x 4096^2 1035 -> 863.
+// pinned memory, us, with 8 / 16 / 24 / 32 MiB: 16 x 1024^2 529 / 428 / 426 / 441, 45 x
+// 480x640 529 / 391 / 393 / 371; against chunks of 8 images 64 x 256^2 393 -> 164, 8 x
+// 2048^2 922 -> 762, 2 x 4096^2 1035 -> 842.
+// The workspace grows with the chunk's maps: where these are larger than the images, a
+// chunk holds no more images than have 256 MiB of maps, or 8 if that is fewer (64
+// images of 64^2 in maps of 1024^2: one chunk 251 us, chunks of 8 589).
 #define FT_DETECT_CHUNK_BYTES ((size_t)24 << 20)
+#define FT_DETECT_CHUNK_MAP_BYTES ((size_t)256 << 20)
+#define FT_DETECT_CHUNK_IMAGES 8
 #define FT_LANES 2          // streams a large batch is split over (see lanes_fork)
 
 static ft_status cuda_fail(cudaError_t e, const char* where) {
@@ -1136,9 +1142,26 @@ ft_status ft_detect_host(ft_plan p, const float* h_img, int batch, int top_k, fl
     p->d_count_host = (int32_t*)((char*)p->d_peaks_host + cnt_off);
     // Chunks of images: the copy stream uploads chunk c + 1 while the caller's
     // stream transforms chunk c; peaks and counts come back per chunk.
-    const size_t per = FT_DETECT_CHUNK_BYTES / (img_px * sizeof(float));
-    const int chunk = per < 1 ? 1 : (per < (size_t)batch ? (int)per : batch);
-    const int nchunks = (batch + chunk - 1) / chunk;
+    const size_t per_img = std::max(FT_DETECT_CHUNK_BYTES / (img_px * sizeof(float)), (size_t)1);
+    const size_t per_map = std::max(FT_DETECT_CHUNK_MAP_BYTES / (map_px * sizeof(float)), (size_t)FT_DETECT_CHUNK_IMAGES);
+    int chunk = (int)std::min({per_img, per_map, (size_t)batch}), nchunks = 0;
+    // size the workspace for one chunk before any copy is in flight (the largest of
+    // the peak passes' scratch; a smaller last chunk may take another pass: room for
+    // every kind); without the memory for it, chunks of 8 images
+    for (;;) {
+        nchunks = (batch + chunk - 1) / chunk;
+        size_t need = 0;
+        for (int nb : {chunk, batch - (nchunks - 1) * chunk}) {
+            size_t peak_b = detect_scratch_bytes(p, nb, top_k, true);
+            if (tile_max_bytes(p, nb) > peak_b) peak_b = tile_max_bytes(p, nb);
+            if (peaks_key_bytes(p->Hp, p->S, nb, top_k) > peak_b) peak_b = peaks_key_bytes(p->Hp, p->S, nb, top_k);
+            if (aux_off(p, nb) + peak_b > need) need = aux_off(p, nb) + peak_b;
+        }
+        s = ensure(p, &p->d_ws, &p->ws_bytes, need, "cudaMalloc(workspace)");
+        if (s == FT_OK) break;
+        if (chunk <= FT_DETECT_CHUNK_IMAGES) return s;
+        chunk = FT_DETECT_CHUNK_IMAGES;
+    }
     if (!p->copy_stream) FT_CUDA(cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking), "copy stream");
     if (!p->start_event) FT_CUDA(cudaEventCreateWithFlags(&p->start_event, cudaEventDisableTiming), "event");
     while ((int)p->chunk_events.size() < nchunks) {
@@ -1146,18 +1169,7 @@ ft_status ft_detect_host(ft_plan p, const float* h_img, int batch, int top_k, fl
         FT_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event");
         p->chunk_events.push_back(e);
     }
-    // size the workspace for one chunk before any copy is in flight (the larger
-    // of the two peak passes' scratch: tile maxima or per-tile keys)
-    // (a smaller last chunk may take the other peak pass: room for every kind)
-    size_t need = 0;
-    for (int nb : {chunk, batch - (nchunks - 1) * chunk}) {
-        size_t peak_b = detect_scratch_bytes(p, nb, top_k, true);
-        if (tile_max_bytes(p, nb) > peak_b) peak_b = tile_max_bytes(p, nb);
-        if (peaks_key_bytes(p->Hp, p->S, nb, top_k) > peak_b) peak_b = peaks_key_bytes(p->Hp, p->S, nb, top_k);
-        if (aux_off(p, nb) + peak_b > need) need = aux_off(p, nb) + peak_b;
-    }
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = ensure(p, &p->d_ws, &p->ws_bytes, need, "cudaMalloc(workspace)")) != FT_OK) return s;
     FT_CUDA(cudaEventRecord(p->start_event, st), "event");
     FT_CUDA(cudaStreamWaitEvent(p->copy_stream, p->start_event, 0), "copy stream wait");
     for (int c = 0; c < nchunks; ++c) {
