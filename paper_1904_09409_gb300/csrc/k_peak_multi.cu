@@ -17,8 +17,9 @@
 //                 cell by cell exactly as k_peak_sparse does (TileTester) and
 //                 their strict local maxima at or above the bound appended to a
 //                 list per image; the last block of an image selects and sorts its
-//                 best top_k.  A list that overflows its PM_CAP keys (maps of
-//                 plateaus) is dropped and that block runs the one-block pass on
+//                 best top_k.  A list that overflows its PM_CAP keys (noise with fewer
+//                 strict tile maxima than a large top_k: the bound is then the
+//                 threshold) is dropped and that block runs the one-block pass on
 //                 the image instead.
 // Every key of the dense list lies in a tile that is tested and is at or above the
 // bound, so the list is the same.
