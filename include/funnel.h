@@ -468,7 +468,8 @@ ft_status ft_fma_probe(float* d_out, int blocks, int iters, void* stream);
  * kernels and the peak pass; an index out of range is skipped (a load reads 0)
  * and sets a bit in a flag word: 1 step-1 loads, 2 step-1 stores, 4 step-4
  * staging, 8 step-4 stores, 16 NVMT taps, 32 FFT exchange slots, 64 NVMT
- * transpose, 128 peak staging.  ft_debug_flags waits for the device, returns
+ * transpose, 128 peak staging, 256 tile maxima, 512 peak lists, 1024 row stores,
+ * 2048 chirp-z rows.  ft_debug_flags waits for the device, returns
  * the bits recorded since the last call in *flags and clears them (0 in the
  * normal build, where the checks do not exist).  ft_debug_build returns 1 for
  * the debug build, 0 otherwise. */

@@ -247,7 +247,8 @@ __device__ __forceinline__ void c2r_from_stage(float2* sm, int ncols, const floa
 #pragma unroll
             for (int q = 0; q < RL; ++q) {
                 const float a = fabsf(v[m * RL + q].x * out_scale), b = fabsf(v[m * RL + q].y * out_scale);
-                mx[F::out_pos(t, m, q) * B + f] = colok ? fmaxf(fmaxf(a, b), 0.f) : 0.f;
+                const int o = F::out_pos(t, m, q) * B + f;
+                if (FT_IN(o, N * B, FT_DBG_TILE_MAX)) mx[o] = colok ? fmaxf(fmaxf(a, b), 0.f) : 0.f;
             }
         __syncthreads();
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -496,6 +497,9 @@ __device__ __forceinline__ bool rows_block(float2* __restrict__ base, int W, int
 #pragma unroll
     for (int m = 0; m < GL; ++m)
 #pragma unroll
-        for (int q = 0; q < RL; ++q) row[fs_rotate<N, RL>(F::out_pos(t, m, q), q)] = v[m * RL + q];
+        for (int q = 0; q < RL; ++q) {
+            const int o = fs_rotate<N, RL>(F::out_pos(t, m, q), q);
+            if (FT_IN(o, N, FT_DBG_ROW_STORE)) row[o] = v[m * RL + q];
+        }
     return true;
 }

@@ -144,16 +144,19 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
 #pragma unroll
             for (int q = 0; q < R0; ++q) {
                 const int row = F::template in_pos<0>(t, m, q);
-                cp_async8(reinterpret_cast<float*>(sm) + row * 2 * B + 2 * f, P + (size_t)row * ncols);
+                if (FT_IN(row, N, FT_DBG_R2C_LOAD) && FT_IN(c + 1, ncols, FT_DBG_R2C_LOAD) &&
+                    FT_IN(row * B + f, F::SLOTS, FT_DBG_FFT_SLOT))
+                    cp_async8(reinterpret_cast<float*>(sm) + row * 2 * B + 2 * f, P + (size_t)row * ncols);
             }
     }
 #pragma unroll
     for (int m = 0; m < G0; ++m)
 #pragma unroll
         for (int q = 0; q < R0; ++q)
-            v[m * R0 + q] = colok ? __ldg(reinterpret_cast<const float2*>(
-                                        Tg + (size_t)F::template in_pos<0>(t, m, q) * ncols))
-                                  : make_float2(0.f, 0.f);
+            v[m * R0 + q] = colok && FT_IN(c + 1, ncols, FT_DBG_R2C_LOAD)
+                                ? __ldg(reinterpret_cast<const float2*>(
+                                      Tg + (size_t)F::template in_pos<0>(t, m, q) * ncols))
+                                : make_float2(0.f, 0.f);
     if (tma_nb > 0) {
         __syncthreads();                               // the mbarrier is initialised
         const bool ok = mbar_wait(mb, 0, wait);
@@ -257,7 +260,9 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
     for (int m = 0; m < G0; ++m)
 #pragma unroll
         for (int q = 0; q < R0; ++q)
-            v[m * R0 + q] = (l < L) ? row[fs_rotate<N, R0>(F::template in_pos<0>(t, m, q), q)] : make_float2(0.f, 0.f);
+            v[m * R0 + q] = l < L && FT_IN((fs_rotate<N, R0>(F::template in_pos<0>(t, m, q), q)), N, FT_DBG_NVMT_ADJ)
+                                ? row[fs_rotate<N, R0>(F::template in_pos<0>(t, m, q), q)]
+                                : make_float2(0.f, 0.f);
     F::template run<0>(v, sm, t, 0, stw);
     // gV[x'] = (-1)^{i + N/2} z[i], i = x' + N/2, z the transform of (-1)^s g[s]: the
     // signs are the rotations of the transform's input and output by N/2
@@ -269,7 +274,7 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
             const int c = F::out_pos(0, m, q);
             const int o = RL % 2 == 0 ? spos_plus(t, st, q < RL / 2 ? c + N / 2 : c - N / 2)
                                       : spos(fs_rotate<N, RL>(t + c, q));
-            sm[o] = v[m * RL + q];
+            if (FT_IN(o, F::SLOTS, FT_DBG_FFT_SLOT)) sm[o] = v[m * RL + q];
         }
     __syncthreads();
     if (l >= L) return;
@@ -332,6 +337,7 @@ k_nvmt_rows_adjoint_fast(float2* __restrict__ ws, int W, int Hp, int L, const fl
                 if (k[j] < 0.f) { k[j] += hpf; xp[j] += 1; }
             }
         }
+        if (!FT_IN(x, N, FT_DBG_ROW_STORE)) continue;
         if (x + 1 < W) *reinterpret_cast<float4*>(row + x) = acc;
         else row[x] = make_float2(acc.x, acc.y);
     }

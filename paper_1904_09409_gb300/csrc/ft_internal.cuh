@@ -31,6 +31,10 @@
 #define FT_DBG_FFT_SLOT 32u       // exchange slots of the register FFT
 #define FT_DBG_NVMT_ADJ 64u       // transpose of step 2: samples gathered back
 #define FT_DBG_PEAK_STAGE 128u    // peak pass: staged tile cells
+#define FT_DBG_TILE_MAX 256u      // step 4: map values exchanged for the tile maxima
+#define FT_DBG_PEAK_LIST 512u     // peak pass over the whole GPU: histogram, tile and candidate lists
+#define FT_DBG_ROW_STORE 1024u    // steps 2-3 and their adjoint: row samples and columns written
+#define FT_DBG_CHIRP 2048u        // chirp-z rows: shared rows, Nyquist slots, row samples
 #ifdef FT_DEBUG
 static __device__ unsigned g_ft_debug;
 __device__ __forceinline__ bool ft_in_range(long long i, long long n, unsigned code) {
@@ -55,6 +59,8 @@ __device__ __forceinline__ bool ft_in_range(long long i, long long n, unsigned c
 unsigned ft_debug_read_fast();
 unsigned ft_debug_read_peak_sparse();
 unsigned ft_debug_read_peak_multi();
+unsigned ft_debug_read_fourier_fast();
+unsigned ft_debug_read_batch();
 
 // One FFT length N = 2^a 3^b: its radix sequence and twiddle table
 // tw[t] = exp(-2 pi i t / N), t in [0, N), rounded to FP32 from FP64 values.

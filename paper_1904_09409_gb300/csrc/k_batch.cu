@@ -106,6 +106,8 @@ k_batch_peaks(const BatchImg* __restrict__ imgs, const float* __restrict__ maps,
                       out + (size_t)d.pos * K, count + d.pos, spsm, sh);
 }
 
+FT_DEBUG_READER(ft_debug_read_batch)
+
 // ---------------------------------------------------------------- host side
 bool batch_threads_ok(int stage, int threads) {
     if (stage == 1) return threads == 128 || threads == 256;

@@ -102,13 +102,17 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q)
-                v[m * R0W + q] = rw.ok ? __ldcg(rw.p + fs_rotate<W, R0W>(FW::template in_pos<0>(tr, m, q), q))
-                                       : make_float2(0.f, 0.f);
+                v[m * R0W + q] = rw.ok && FT_IN((fs_rotate<W, R0W>(FW::template in_pos<0>(tr, m, q), q)), W, FT_DBG_CHIRP)
+                                     ? __ldcg(rw.p + fs_rotate<W, R0W>(FW::template in_pos<0>(tr, m, q), q))
+                                     : make_float2(0.f, 0.f);
         FW::template run<0>(v, smr, tr, 0, stw_w);
 #pragma unroll
         for (int m = 0; m < GLW; ++m)
 #pragma unroll
-            for (int q = 0; q < RLW; ++q) rowr[spos_plus(tr, spos(tr), FW::out_pos(0, m, q))] = v[m * RLW + q];
+            for (int q = 0; q < RLW; ++q) {
+                const int o = spos_plus(tr, spos(tr), FW::out_pos(0, m, q));
+                if (FT_IN(o, FW::SLOTS, FT_DBG_CHIRP)) rowr[o] = v[m * RLW + q];
+            }
     }
     __syncthreads();
 
@@ -140,7 +144,7 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
                             slot = spos_plus(t, st, q < R0M / 4 ? c + W / 2 : c - W / 2);
                         else
                             slot = spos(i < W / 2 ? i + W / 2 : i - W / 2);
-                        float2 a = rowg[slot];
+                        float2 a = FT_IN(slot, FW::SLOTS, FT_DBG_CHIRP) ? rowg[slot] : make_float2(0.f, 0.f);
                         if (m == 0 && (q == 0 || q == R0M / 2) && t == 0) a = cscale(a, 0.5f);
                         y = cmul(a, __ldg(cu + i));
                     }
@@ -156,7 +160,9 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
 #pragma unroll
                 for (int q = 0; q < RLM; ++q) {
                     const int k = FMf::out_pos(t, m, q);
-                    smf[spos_plus(t, st, FMf::out_pos(0, m, q))] = cmul(v[m * RLM + q], __ldg(hl + k));
+                    const int o = spos_plus(t, st, FMf::out_pos(0, m, q));
+                    if (FT_IN(k, M, FT_DBG_CHIRP) && FT_IN(o, FMf::SLOTS, FT_DBG_FFT_SLOT))
+                        smf[o] = cmul(v[m * RLM + q], __ldg(hl + k));
                 }
         }
         __syncthreads();
@@ -164,7 +170,10 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
 #pragma unroll
         for (int m = 0; m < G0M; ++m)
 #pragma unroll
-            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = smf[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q))];
+            for (int q = 0; q < R0M; ++q) {
+                const int o = spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q));
+                v[m * R0M + q] = FT_IN(o, FMi::SLOTS, FT_DBG_FFT_SLOT) ? smf[o] : make_float2(0.f, 0.f);
+            }
         __syncthreads();
         FMi::template run<0>(v, smf, ti, 0, stw_m);
         // ---- V[k] = z[k] / (W M) x post-chirp inside the support, for k < S = M / 2 (the
@@ -188,7 +197,7 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
                             slot = spos_plus(ti, sti, FMi::out_pos(0, m, q) + (q < RLM / 4 ? S / 2 : -S / 2));
                         else
                             slot = spos(k < S / 2 ? k + S / 2 : k - S / 2);
-                        rowg[slot] = r;
+                        if (FT_IN(slot, FW::SLOTS, FT_DBG_CHIRP)) rowg[slot] = r;
                     }
                 }
         }
@@ -203,14 +212,19 @@ k_nvmt_rows_fourier_fast(float2* __restrict__ ws, int Hp, int L, int batch, cons
 #pragma unroll
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
-            for (int q = 0; q < R0W; ++q)
-                v[m * R0W + q] = rowr[spos_plus(tr, str, FS::template in_pos<0>(0, m, q))];
+            for (int q = 0; q < R0W; ++q) {
+                const int o = spos_plus(tr, str, FS::template in_pos<0>(0, m, q));
+                v[m * R0W + q] = FT_IN(o, FW::SLOTS, FT_DBG_CHIRP) ? rowr[o] : make_float2(0.f, 0.f);
+            }
         FS::template run<0>(v, smr, tr, 0, stw_s);
         if (rw.ok) {
 #pragma unroll
             for (int m = 0; m < GLW; ++m)
 #pragma unroll
-                for (int q = 0; q < RLW; ++q) rw.p[fs_rotate<S, RLW>(FS::out_pos(tr, m, q), q)] = v[m * RLW + q];
+                for (int q = 0; q < RLW; ++q) {
+                    const int o = fs_rotate<S, RLW>(FS::out_pos(tr, m, q), q);
+                    if (FT_IN(o, S, FT_DBG_CHIRP)) rw.p[o] = v[m * RLW + q];
+                }
         }
     }
 }
@@ -255,8 +269,9 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q)
-                v[m * R0W + q] = rw.ok ? __ldcg(rw.p + fs_rotate<S, R0W>(FS::template in_pos<0>(tr, m, q), q))
-                                       : make_float2(0.f, 0.f);
+                v[m * R0W + q] = rw.ok && FT_IN((fs_rotate<S, R0W>(FS::template in_pos<0>(tr, m, q), q)), S, FT_DBG_CHIRP)
+                                     ? __ldcg(rw.p + fs_rotate<S, R0W>(FS::template in_pos<0>(tr, m, q), q))
+                                     : make_float2(0.f, 0.f);
         FS::template run<0>(v, smr, tr, 0, stw_s);
 #pragma unroll
         for (int m = 0; m < GLW; ++m)
@@ -265,7 +280,7 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                 const int c = FS::out_pos(0, m, q);
                 const int slot = RLW % 2 == 0 ? spos_plus(tr, spos(tr), q < RLW / 2 ? c + S / 2 : c - S / 2)
                                               : spos(fs_rotate<S, RLW>(tr + c, q));
-                rowr[slot] = v[m * RLW + q];
+                if (FT_IN(slot, FS::SLOTS, FT_DBG_CHIRP)) rowr[slot] = v[m * RLW + q];
             }
     }
     __syncthreads();
@@ -296,7 +311,8 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                         const int k = FMf::template in_pos<0>(t, m, q);
                         if (k >= lo && k <= hi) {
                             const float2 c = __ldg(cx + k);
-                            const float2 a = rowg[spos_plus(t, st, FMf::template in_pos<0>(0, m, q))];
+                            const int o = spos_plus(t, st, FMf::template in_pos<0>(0, m, q));
+                            const float2 a = FT_IN(o, FS::SLOTS, FT_DBG_CHIRP) ? rowg[o] : make_float2(0.f, 0.f);
                             r = cscale(cmul(a, make_float2(c.x, -c.y)), sc);
                         }
                     }
@@ -312,7 +328,9 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                 for (int q = 0; q < RLM; ++q) {
                     const int k = FMf::out_pos(t, m, q);
                     const float2 h = __ldg(hl + k);
-                    smf[spos_plus(t, st, FMf::out_pos(0, m, q))] = cmul(v[m * RLM + q], make_float2(h.x, -h.y));
+                    const int o = spos_plus(t, st, FMf::out_pos(0, m, q));
+                    if (FT_IN(k, M, FT_DBG_CHIRP) && FT_IN(o, FMf::SLOTS, FT_DBG_FFT_SLOT))
+                        smf[o] = cmul(v[m * RLM + q], make_float2(h.x, -h.y));
                 }
         }
         __syncthreads();
@@ -320,7 +338,10 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
 #pragma unroll
         for (int m = 0; m < G0M; ++m)
 #pragma unroll
-            for (int q = 0; q < R0M; ++q) v[m * R0M + q] = smf[spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q))];
+            for (int q = 0; q < R0M; ++q) {
+                const int o = spos_plus(ti, sti, FMi::template in_pos<0>(0, m, q));
+                v[m * R0M + q] = FT_IN(o, FMi::SLOTS, FT_DBG_FFT_SLOT) ? smf[o] : make_float2(0.f, 0.f);
+            }
         __syncthreads();
         FMi::template run<0>(v, smf, ti, 0, stw_m);
         // ---- conj(D_u) and P^T on the entries i = u + W/2 <= W (halved at u = +-W/2)
@@ -337,7 +358,7 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
                         if (i == 0 || i == W) r = cscale(r, 0.5f);
                         if (i == W)
                             nyq[fg] = r;
-                        else
+                        else if (FT_IN(spos(i < W / 2 ? i + W / 2 : i - W / 2), FW::SLOTS, FT_DBG_CHIRP))
                             rowg[spos(i < W / 2 ? i + W / 2 : i - W / 2)] = r;
                     }
                 }
@@ -354,7 +375,8 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
         for (int m = 0; m < G0W; ++m)
 #pragma unroll
             for (int q = 0; q < R0W; ++q) {
-                float2 a = rowr[spos_plus(tr, str, FW::template in_pos<0>(0, m, q))];
+                const int o = spos_plus(tr, str, FW::template in_pos<0>(0, m, q));
+                float2 a = FT_IN(o, FW::SLOTS, FT_DBG_CHIRP) ? rowr[o] : make_float2(0.f, 0.f);
                 if (FW::template in_pos<0>(tr, m, q) == W / 2) a = cadd(a, nyq[fr]);
                 v[m * R0W + q] = a;
             }
@@ -363,10 +385,15 @@ k_nvmt_rows_fourier_adj_fast(float2* __restrict__ ws, int Hp, int L, int batch, 
 #pragma unroll
             for (int m = 0; m < GLW; ++m)
 #pragma unroll
-                for (int q = 0; q < RLW; ++q) rw.p[fs_rotate<W, RLW>(FW::out_pos(tr, m, q), q)] = v[m * RLW + q];
+                for (int q = 0; q < RLW; ++q) {
+                    const int o = fs_rotate<W, RLW>(FW::out_pos(tr, m, q), q);
+                    if (FT_IN(o, W, FT_DBG_CHIRP)) rw.p[o] = v[m * RLW + q];
+                }
         }
     }
 }
+
+FT_DEBUG_READER(ft_debug_read_fourier_fast)
 
 // ------------------------------------------------------------------ dispatch
 #define FR_FAST_LENGTHS(X) \

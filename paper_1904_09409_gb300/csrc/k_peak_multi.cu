@@ -111,7 +111,10 @@ k_peak_bound(const unsigned* __restrict__ tmax, int nty, int ntx, int K, float t
     if (n >= K) {
         for (int b = threadIdx.x; b < PM_BINS; b += PM_THREADS) hist[b] = 0u;
         __syncthreads();
-        for (int j = threadIdx.x; j < n; j += PM_THREADS) atomicAdd(&hist[__ldcg(list + j) >> 18], 1u);
+        for (int j = threadIdx.x; j < n; j += PM_THREADS) {
+            const unsigned b = __ldcg(list + j) >> 18;
+            if (FT_IN(b, PM_BINS, FT_DBG_PEAK_LIST)) atomicAdd(&hist[b], 1u);
+        }
         __syncthreads();
         // thread t owns bins PM_BINS - 1 - 8 t - (0 .. 7), descending; an inclusive scan of
         // the owned counts finds the thread whose bins pass K
@@ -182,7 +185,8 @@ k_peak_scan(const float* __restrict__ map, const unsigned* __restrict__ tmax, in
             int pos = 0;
             if (lane == 0 && bal) pos = atomicAdd(&sh.nlist, __popc(bal));
             pos = __shfl_sync(0xffffffffu, pos, 0);
-            if (w) list[pos + __popc(bal & ((1u << lane) - 1u))] = (int)t;
+            pos += __popc(bal & ((1u << lane) - 1u));
+            if (w && FT_IN(pos, 256, FT_DBG_PEAK_LIST)) list[pos] = (int)t;
         }
         __syncthreads();
         const int nl = sh.nlist;
@@ -228,7 +232,10 @@ k_peak_scan(const float* __restrict__ map, const unsigned* __restrict__ tmax, in
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const u64 key = keys[i];
-        if (selected(key, sh.st)) keep[atomicAdd(&sh.st.count, 1)] = key;
+        if (selected(key, sh.st)) {
+            const int o = atomicAdd(&sh.st.count, 1);
+            if (FT_IN(o, K, FT_DBG_PEAK_LIST)) keep[o] = key;
+        }
     }
     __syncthreads();
     const int cnt = sh.st.count, Kp = next_pow2(max(cnt, 1));

@@ -323,7 +323,8 @@ ft_status ft_debug_flags(uint32_t* flags) {
     if (!flags) return FT_ERR_INVALID_ARG;
     *flags = 0;
     FT_CUDA(cudaDeviceSynchronize(), "ft_debug_flags");
-    *flags = ft_debug_read_fast() | ft_debug_read_peak_sparse() | ft_debug_read_peak_multi();
+    *flags = ft_debug_read_fast() | ft_debug_read_peak_sparse() | ft_debug_read_peak_multi() |
+             ft_debug_read_fourier_fast() | ft_debug_read_batch();
     return FT_OK;
 }
 
