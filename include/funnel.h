@@ -265,9 +265,9 @@ int ft_plan_get_variant(ft_plan plan);
  * [n][top_k] rows and counts as [n] in the same packed order.  Equal shapes are
  * contiguous, largest first.
  *
- * Images whose sides both have a fixed-length schedule up to 2048 (128, 192,
- * 256, 384, 512, 768, 1024, 1536, 2048), with the linear or cubic interpolator,
- * run in the grouped kernels: one launch per stage over all of them (step 1;
+ * Images whose sides both are among the grouped lengths (128, 192, 256, 384,
+ * 512, 768, 1024, 1536, 2048), with the linear or cubic interpolator, run in the
+ * grouped kernels: one launch per stage over all of them (step 1;
  * steps 2-3; step 4 with the maxima of |P| per 256-cell tile; the peak pass from
  * those maxima), each block running the fixed-length code of one (image, block)
  * item's length; 4 launches (3 with top_k = 0) whatever the number of shapes.

@@ -3,9 +3,9 @@
 //
 // The batch fixes a packed layout: images (and maps, and peak rows) are stored
 // back to back in the order of ft_batch_layout, which groups equal shapes
-// together (largest first).  Images whose sides both have a fixed-length
-// schedule up to 2048 (128, 192, 256, 384, 512, 768, 1024, 1536, 2048) with the
-// linear or cubic interpolator run in the grouped kernels of k_batch.cu: one
+// together (largest first).  Images whose sides both are among the grouped lengths
+// (128, 192, 256, 384, 512, 768, 1024, 1536, 2048) with the linear or cubic
+// interpolator run in the grouped kernels of k_batch.cu: one
 // launch per stage over all of them (step 1, steps 2-3, step 4 with tile maxima,
 // the peak pass), one block per (image, block) item, with the batch's own
 // workspace.  Every other shape group keeps a plan of its own (tables and
@@ -50,7 +50,10 @@ struct Group {
 // threads below length 1024 and 512 from there on, where 256 threads hold 4 column
 // pairs or fewer: setup_grouped takes 512 when the images of at least 1024 rows hold
 // more than half of the pixels (96 images of all sizes 483 us with 256, 459 with 512;
-// 64 images up to 768 80 and 86)
+// 64 images up to 768 80 and 86; two 2048^2 with a hundred 256^2 142 and 135).  Where
+// the other half are images of 128 rows it loses (six 1024^2 with forty 128x1024 104
+// and 111 us): their tiles are then 2 x 128 cells, which the peak pass stages cell by
+// cell.
 const int kThreadOpts[3][2] = {{256, 512}, {128, 256}, {256, 512}};
 const int kDefaultThreads[3] = {512, 128, 256};
 
@@ -395,8 +398,8 @@ static ft_status setup_grouped(ft_batch_s* b) {
     if (2 * tall > all) b->threads[2] = 512;
     // steps 2-3 walk the images backwards: their first blocks read the half
     // spectra step 1 wrote last, still in L2, and step 4 starts on the rows
-    // written last (every item holds the same number of samples, so the order
-    // does not change the tail of a launch)
+    // written last (an item holds 12 or 16 samples per thread whatever its image,
+    // so the order changes the tail of a launch by little)
     for (int o = 0; o < 2; ++o) std::reverse(items[2 + o].begin(), items[2 + o].end());
     cudaError_t e = cudaMalloc(&b->d_imgs, b->himgs.size() * sizeof(BatchImg));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_imgs, b->himgs.data(), b->himgs.size() * sizeof(BatchImg), cudaMemcpyHostToDevice);

@@ -220,7 +220,8 @@ k_col_r2c_loss_fast(const float* __restrict__ map, const float* __restrict__ tar
                               mid_scale);
 }
 
-// at most 64 registers, so that 4 blocks of 256 threads share a multiprocessor
+// 64 threads per block at most lengths and at most 64 registers (fs_minblocks: 72 to 112
+// where a thread holds 18 to 36 samples), so that 16 blocks share a multiprocessor
 template <int N, int INTERP>
 __global__ void __launch_bounds__(fs_T(N) * fs_Brow(N), fs_minblocks(N, fs_T(N) * fs_Brow(N)))
 k_nvmt_rows_fast(float2* __restrict__ ws, int W, int Hp, int L, const float2* __restrict__ stw,

@@ -1,7 +1,7 @@
 // Register-resident Stockham FFT with compile-time schedules.
 //
-// For the lengths below every thread of a transform holds E elements (16, or 12
-// when N has a factor 3) in registers; a transform of length N uses T = N / E
+// For the lengths below every thread of a transform holds E elements (16 for the
+// powers of two, 8 at 64; 12, 18, 24 or 36 when N has a factor 3) in registers; a transform of length N uses T = N / E
 // threads, and a block runs B transforms side by side (transform f's sample n
 // lives at smem[spos(n) * B + f]).  A pass with radix R and P = product of the
 // earlier radices does, for butterfly i in [0, N/R) with k = i mod P:
@@ -38,7 +38,10 @@
 // 12 12 4 4 40 / 30 / 41 (55 / 35 / 53), 576 as 24 24 against 12 12 4 30 / 35 / 28
 // (35 / 35 / 37); but 288 as 12 12 2 against 24 12 29 / 38 / 28 (29 / 47 / 27), and
 // 1296 as 6 6 6 6 with E = 12 against 12 12 9 with E = 36, which spills, the same
-// forward and a faster adjoint (50 against 58).  192, 384, 768 and 1536 start with
+// forward and a faster adjoint (50 against 58).  2592 and 3888 hold 36 all the same
+// (step 1 of 2592 spills 252 bytes, step 4 and the loss kernel about 140): forward and
+// backward of two 2592^2 images 99 and 105 us (generic 374 and 363), of one 3888^2 125
+// and 131 (476 and 454); schedules with fewer samples there were not compared.  192, 384, 768 and 1536 start with
 // radix 12 and save a pass against radix 4 passes and a last radix 3 (384^2 40 / 42 /
 // 34 -> 37 / 35 / 32, 1536^2 51 / 41 / 49 -> 47 / 40 / 45).  The shortest, against the
 // generic kernels: 64^2 26 / 31 / 26 (65 / 141 / 54; as 16 4 with E = 16 26 / 37 / 24),

@@ -109,7 +109,10 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // With few blocks there is no such wave, and the waiting blocks of the successor
 // only get in the way (forward, us, trigger always / never: 4 x 512^2 17.4 / 10.5,
 // 1024^2 20.3 / 14.4, 1536x576 25.3 / 16.6; 32 x 512^2 38.9 / 39.3, 64 x 1024^2 268.2 /
-// 269.9; the line at 1024 blocks has the better of the two in every case).
+// 269.9).  The line is a rough one: what counts is the waves, and 1024 blocks are 3.4
+// waves of step 1 at 1024 but 0.4 of the row kernels.  Just above it, always / this
+// line / never: 2 x 1024^2 25.4 / 17.4 / 17.2, 4 x 1024^2 27.4 / 26.6 / 26.0, 3 x 2048^2
+// 75.0 / 74.3 / 73.7, one 4096^2 122.2 / 121.7 / 120.9, 12 x 1024^2 65.4 / 65.5 / 65.6.
 __device__ __forceinline__ void pdl_trigger_large() {
     if (gridDim.x * gridDim.y >= 1024u) pdl_trigger();
 }
@@ -479,7 +482,8 @@ struct BatchImg {
     const float2* stw_y;    // per-pass twiddles of length H (steps 1 and 4)
     const float2* stw_x;    // per-pass twiddles of length W (step 3)
 };
-// lengths the grouped kernels take (every fixed-length schedule up to 2048)
+// lengths the grouped kernels take (the powers of two from 128 and 3 x 2^a from 192 to
+// 2048; the other fixed lengths go through plans of their own)
 __host__ __device__ constexpr bool batch_len_ok(int n) {
     return n == 128 || n == 192 || n == 256 || n == 384 || n == 512 || n == 768 || n == 1024 || n == 1536 ||
            n == 2048;

@@ -8,8 +8,8 @@
 // fast_blocks.cuh for that image's length, chosen by a switch on the length.
 // The threads per block are fixed per launch (the autotuner's knob for each
 // stage), so the transforms per block follow from the length: B = threads /
-// fs_T(length), and every item holds the same number of samples (E x threads),
-// whatever its image.  The hardware hands the blocks out in order, which
+// fs_T(length), and an item holds E x threads samples whatever its image (E = 16, or 12
+// for 192, 384, 768 and 1536).  The hardware hands the blocks out in order, which
 // balances the stage; a persistent kernel taking the items from an atomic
 // counter in a loop did the same but kept the index arithmetic of all nine
 // lengths live across the loop (500 bytes spilled at 64 registers with the
